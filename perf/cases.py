@@ -232,3 +232,45 @@ def tolerance(case):
     # fp32 sums and one rounding to fp16 differ from the same product in 64 bits by 2.1e-4 (largest
     # element: 4.9e-4) whatever the size; three roundings in a row by 4.2e-4 (2.0e-3).  Four times that.
     return {"rel": 1.7e-3, "max": 8e-3} if case["op"] == "block" else {"rel": 8e-4, "max": 2e-3}
+
+
+# ---- the same results in 64 bits -------------------------------------------------------------------
+def _linear(W, Xt, bias, act):
+    """act(Xt W^T + b) in 64 bits."""
+    y = Xt @ W.double().T
+    if bias is not None:
+        y += bias.double()
+    if act == "relu":
+        return y.relu_()
+    if act == "silu":
+        return y / (1.0 + torch.exp(-y))
+    if act == "gelu_tanh":
+        return 0.5 * y * (1.0 + torch.tanh(math.sqrt(2.0 / math.pi) * (y + 0.044715 * y ** 3)))
+    return y
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, from the dense weights (the draws are those of prepare())."""
+    op, M, K, N = case["op"], case["M"], case["K"], case["N"]
+    if op in ("convert", "save", "load"):
+        return None                                                 # bytes
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    if op == "block":
+        layers = []
+        for r, c in [(M, M)] * 4 + [(K, M), (M, K)]:
+            W, b = _weights(g, r, c, case["sparsity"], case["mask"]), _bias(g, case, r)
+            _activations(g, N, r)                                   # the output buffer's first contents
+            layers.append((W, b))
+        x = _activations(g, N, M).double()
+        (q, bq), (k, bk), (v, bv), (o, bo), (f1, b1), (f2, b2) = layers
+        yq, yk, yv = _linear(q, x, bq, "none"), _linear(k, x, bk, "none"), _linear(v, x, bv, "none")
+        yo = _linear(o, yv, bo, "none")
+        y1 = _linear(f1, yo, b1, case["act"])
+        return [yq, yk, yv, yo, y1, _linear(f2, y1, b2, "none")]
+    W = _weights(g, M, K, case["sparsity"], case["mask"])
+    if op == "nt":
+        X = _activations(g, N, K).double()
+        return _linear(W, X, _bias(g, case, M), case["act"])
+    X = _activations(g, K, N) if op == "spmm" else torch.randn((K, N), generator=g, device="cuda").half()
+    y = W.double() @ X.double()
+    return y if op == "spmm" else y.cpu().numpy()
