@@ -2,25 +2,30 @@
 // of Sec. 3.2, byte for byte what tl3_encode() builds on the host.  (The paper converts on the CPU,
 // 41-93 s per model, Sec. 5.3 "Storage Format Conversion".)
 //
-// Tiles are independent, so one CTA of 128 threads takes one 128 x 128 tile; thread r owns row r of
-// the tile -- its 32 windows, and later the PDD chain of the surplus weights of that row.
-//   pass A   every thread classifies its 32 windows (which two weights stay, which slots are
-//            empty, which weights are surplus) and counts its surplus weights and empty slots;
-//   scan     a block-wide exclusive scan of both counts gives every row the index of its first
-//            surplus weight and of its first empty slot in the tile's row-major order;
-//   pass B   the same classification again, this time writing the kept values and the metadata to
-//            the container and the surplus list (position, value) and the empty-slot list into
-//            shared memory at their scanned positions -- both lists come out sorted;
-//   chains   the i-th surplus weight is parked in the i-th empty slot; thread r walks the pairs
-//            whose surplus weight lies in row r, writes the parked values into the value array,
-//            and forms the chain: 16-bit starts, 4-bit delta pairs, dummy points for spans above
-//            the 4-bit range, cut after 255 bytes;
+// Tiles are independent, so one CTA of eight warps takes one 128 x 128 tile.
+//   classify a lane loads one window of four weights, a warp one row at a time (a coalesced 256-byte
+//            load); four votes turn the row's non-zeros into four 32-bit masks, one per in-window
+//            index, and from there on a row is classified with a few bit operations on its masks
+//            (which two weights stay, which slots are empty, which weights are surplus);
+//   lists    one thread per row and kind writes the positions of the row's empty slots and of its
+//            surplus weights into shared memory at their scanned places, sorted by construction;
+//   pairs    the i-th surplus weight is parked in the i-th empty slot.  A thread takes a run of
+//            consecutive pairs and a scan over the threads gives every pair the place of its delta
+//            bytes: the chains of a tile (one per row: 16-bit starts, 4-bit delta pairs, dummy points
+//            for spans above the 4-bit range) follow each other in the order of the pairs.  Only a
+//            tile with a chain of more than 255 bytes, which is cut there, walks rows one by one;
 //   residual what found no empty slot (and what a cut chain left over) goes to the Residual list.
 // The kernel runs twice: first it only counts the PDD bytes and Residual entries of every tile,
 // a one-block scan turns the counts into the offsets of the tile directory, then it runs again
 // and writes the bytes where they belong.
+// What bounds it is the number of instructions it issues (its memory traffic, W once per pass and the
+// container once, is a few microseconds).  Two passes on 5120 x 5120 at 50 % sparsity: 31 + 52 us.
+// A thread per row, two-byte accesses a row pitch apart and 512 atomics per tile on four
+// addresses took 351 + 898 us; coalesced rows that every lane classified for itself, with chains
+// walked by a thread per row, 57 + 89 us.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <new>
 #include <vector>
@@ -43,8 +48,9 @@ void set_cuda_error(int e);
 
 namespace {
 
-constexpr int kEncThreads = 128;
-constexpr int kMaxd = 15;
+constexpr int kEncThreads = 256;
+constexpr int kEncRows = kTileM / (kEncThreads / 32);   // rows per warp
+constexpr uint32_t kMaxd = 15;
 constexpr int kChainCap = 255;
 
 struct EncodeArgs {
@@ -52,6 +58,7 @@ struct EncodeArgs {
   long long M, K, ldw;
   long long K_pad;
   int tiles_k;
+  int vec;                      // windows may be loaded as 8 bytes (base and row pitch are multiples of 8 bytes)
   uint16_t* tc_vals;            // [M_pad][K_pad / 2]
   uint8_t* tc_meta;             // [M_pad][K_pad / 8]
   uint16_t* chain_tau0;         // [tiles][128]
@@ -65,244 +72,341 @@ struct EncodeArgs {
   int emit;                     // 0: count pass (fills pdd_len and res_cnt of the directory), 1: write everything
 };
 
-__device__ __forceinline__ bool nonzero(uint16_t h) { return (h & 0x7FFFu) != 0; }
-
-// One window of four consecutive weights (Sec. 3.2, Sparse-TC layer): the first two non-zeros stay;
-// a window short of two completes its index pair with the lowest unused positions (those slots are
-// empty); the third and fourth non-zero are surplus and always sit at in-window index 2 or 3.
-struct Window {
-  int idx0, idx1;               // in-window index carried by slot 0 / slot 1
-  bool kept0, kept1;
-  int n_surplus;
-  int sur[2];                   // in-window indices of the surplus weights
-};
-
-__device__ __forceinline__ Window classify(const uint16_t w[4]) {
-  Window c;
-  int nz[4], n = 0;
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    if (nonzero(w[i])) nz[n++] = i;
-  if (n >= 2) { c.idx0 = nz[0]; c.idx1 = nz[1]; c.kept0 = true; c.kept1 = true; }
-  else if (n == 1) {
-    if (nz[0] == 0) { c.idx0 = 0; c.idx1 = 1; c.kept0 = true; c.kept1 = false; }
-    else { c.idx0 = 0; c.idx1 = nz[0]; c.kept0 = false; c.kept1 = true; }
-  } else { c.idx0 = 0; c.idx1 = 1; c.kept0 = false; c.kept1 = false; }
-  c.n_surplus = n > 2 ? n - 2 : 0;
-  c.sur[0] = n > 2 ? nz[2] : 0;
-  c.sur[1] = n > 3 ? nz[3] : 0;
-  return c;
-}
-
-// exclusive scan of one int per thread over the 128 threads of the CTA; *total gets the sum
-__device__ __forceinline__ int block_exclusive_scan(int v, int* s_warp, int* total) {
+// exclusive scan over the threads of the CTA; *total gets the sum in every thread
+__device__ __forceinline__ uint32_t scan_cta(uint32_t v, uint32_t* s_warp, uint32_t* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
+  uint32_t x = v;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
     if (lane >= d) x += y;
   }
   if (lane == 31) s_warp[warp] = x;
   __syncthreads();
-  int base = 0;
-  for (int w = 0; w < warp; ++w) base += s_warp[w];
-  *total = s_warp[0] + s_warp[1] + s_warp[2] + s_warp[3];
+  uint32_t base = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < kEncThreads / 32; ++w) {
+    base += w < warp ? s_warp[w] : 0u;
+    all += s_warp[w];
+  }
+  *total = all;
   __syncthreads();
   return base + x - v;
 }
 
-__global__ void __launch_bounds__(kEncThreads)
+// dummy points in front of a pair that lies gt slots and gr positions behind the one before it
+__device__ __forceinline__ uint32_t dummies(uint32_t gt, uint32_t gr) {
+  return (gt > kMaxd ? (gt - 1) / kMaxd : 0u) + (gr > kMaxd ? (gr - 1) / kMaxd : 0u);
+}
+
+// One window of four consecutive weights (Sec. 3.2, Sparse-TC layer): the first two non-zeros stay;
+// a window short of two completes its index pair with the lowest unused positions (those slots are
+// empty); the third and fourth non-zero are surplus and always sit at in-window index 2 or 3.
+// Entry p of the table, for non-zeros at the positions set in p: x = byte selector that puts the two
+// weights of the index pair into one word | metadata nibble << 16, y = mask of the occupied slots.
+__device__ __forceinline__ uint2 window_entry(uint32_t p) {
+  const uint32_t first = __ffs(p) - 1u, second = __ffs(p & (p - 1u)) - 1u;
+  uint32_t i0 = 0, i1 = 1, mask = 0;
+  if (__popc(p) >= 2) { i0 = first; i1 = second; mask = 0xFFFFFFFFu; }
+  else if (p == 1u) mask = 0x0000FFFFu;
+  else if (p != 0u) { i1 = first; mask = 0xFFFF0000u; }
+  return make_uint2((0x10u + 0x22u * i0) | (0x10u + 0x22u * i1) << 8 | (i0 | i1 << 2) << 16, mask);
+}
+
+struct EncodeSmem {
+  uint16_t vals[kTileM * kH];   // image of W_t (kept values, then the parked ones too)
+  uint32_t high[kTileM * 32];   // weights 2 and 3 of every window: the surplus value at position rho is half-word rho
+  uint16_t list[kTileM * kH];   // empty slots ascending, then surplus positions ascending: a window has empty slots
+                                // or surplus weights, not both, and never more than two of them
+  uint8_t nib[kTileM * 32];     // metadata of every window; later the code bytes of the tile, while they fit
+  uint32_t nz[4][kTileM];       // non-zeros of a row by in-window index, one bit per window
+  uint2 window[16];
+  uint16_t first[kTileM];       // delta bytes before the first pair of the row
+  uint16_t last[kTileM];        // ... and after its last pair
+  uint16_t parked_end[kTileM];  // first pair of the row that is not parked any more
+  uint16_t moved[kTileM];       // delta bytes that cut chains before this row have lost
+  uint32_t warp_tmp[kEncThreads / 32];
+  int nnz, n_chains;
+};
+constexpr int kCodeStage = kTileM * 32;       // a tile has 1.5-2 KB of code bytes as a rule
+
+__global__ void __launch_bounds__(kEncThreads, 4)
 tl3_encode_kernel(const EncodeArgs a) {
-  __shared__ uint16_t s_rho[kTileM * kH];      // surplus weights of the tile, ascending position in W_r
-  __shared__ uint16_t s_tau[kTileM * kH];      // empty slots of the tile, ascending position in W_t
-  __shared__ int s_warp[4];
-  const int r = threadIdx.x;
+  extern __shared__ __align__(16) uint8_t encode_smem_raw[];
+  EncodeSmem& sm = *reinterpret_cast<EncodeSmem*>(encode_smem_raw);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long tile = blockIdx.x;
   const long long tm = tile / a.tiles_k, tk = tile % a.tiles_k;
-  const long long row = tm * kTileM + r;
   const long long half_ld = a.K_pad / 2, meta_ld = a.K_pad / 8;
-  const bool row_in = row < a.M;
-  const uint16_t* wrow = a.W + row * a.ldw + tk * kTileK;
-  auto load_window = [&](int q, uint16_t w[4]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const long long col = tk * kTileK + 4 * q + i;
-      w[i] = (row_in && col < a.K) ? wrow[4 * q + i] : uint16_t{0};
-    }
-  };
+  if (tid < 16) sm.window[tid] = window_entry(static_cast<uint32_t>(tid));
+  if (tid == 16) { sm.nnz = 0; sm.n_chains = 0; }
 
-  // ---- pass A: count the surplus weights and the empty slots of this row
-  int nS = 0, nE = 0, nnz = 0;
-  for (int q = 0; q < kTileK / 4; ++q) {
-    uint16_t w[4];
-    load_window(q, w);
-    const Window c = classify(w);
-    nS += c.n_surplus;
-    nE += (c.kept0 ? 0 : 1) + (c.kept1 ? 0 : 1);
-    nnz += (c.kept0 ? 1 : 0) + (c.kept1 ? 1 : 0) + c.n_surplus;
-  }
-  int totS = 0, totE = 0;
-  const int offS = block_exclusive_scan(nS, s_warp, &totS);
-  const int offE = block_exclusive_scan(nE, s_warp, &totE);
-  const int P = totS < totE ? totS : totE;     // pairs: the i-th surplus weight goes to the i-th empty slot
-
-  // ---- pass B: kept values and metadata to the container, both lists to shared memory
+  // ---- classify: lane q holds window q of the warp's rows
+  uint2 w[kEncRows];
   {
-    int iS = offS, iE = offE;
-    uint32_t* mrow = reinterpret_cast<uint32_t*>(a.tc_meta + row * meta_ld + tk * (kTileK / 8));   // 16 bytes of this row, 4-byte aligned
-    uint32_t word = 0;                         // eight nibbles: windows 8k .. 8k + 7, even window in the low nibble of its byte
-    for (int q = 0; q < kTileK / 4; ++q) {
-      uint16_t w[4];
-      load_window(q, w);
-      const Window c = classify(w);
-      word |= static_cast<uint32_t>(c.idx0 | (c.idx1 << 2)) << (4 * (q & 7));
-      if (a.emit) {
-        uint16_t* v = a.tc_vals + row * half_ld + tk * kH + 2 * q;
-        v[0] = c.kept0 ? w[c.idx0] : uint16_t{0};
-        v[1] = c.kept1 ? w[c.idx1] : uint16_t{0};
-        if ((q & 7) == 7) mrow[q >> 3] = word;
+    const int row0 = warp * kEncRows;
+    const long long left_m = a.M - tm * kTileM - row0, left_k = a.K - tk * kTileK - 4 * lane;
+    const int rows = left_m < kEncRows ? static_cast<int>(left_m) : kEncRows;          // (may be negative)
+    const int cols = left_k < 4 ? static_cast<int>(left_k) : 4;
+    const uint16_t* src = a.W + (tm * kTileM + row0) * a.ldw + tk * kTileK + 4 * lane;
+    if (a.vec && rows == kEncRows && cols == 4) {
+#pragma unroll
+      for (int k = 0; k < kEncRows; ++k, src += a.ldw) w[k] = __ldg(reinterpret_cast<const uint2*>(src));
+    } else {
+#pragma unroll
+      for (int k = 0; k < kEncRows; ++k, src += a.ldw) {
+        uint32_t h[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) h[i] = k < rows && i < cols ? src[i] : 0u;
+        w[k] = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
       }
-      if ((q & 7) == 7) word = 0;
-      if (!c.kept0) s_tau[iE++] = static_cast<uint16_t>(r * kH + 2 * q);
-      if (!c.kept1) s_tau[iE++] = static_cast<uint16_t>(r * kH + 2 * q + 1);
-      for (int j = 0; j < c.n_surplus; ++j) s_rho[iS++] = static_cast<uint16_t>(r * kH + 2 * q + (c.sur[j] - 2));
+    }
+  }
+  __syncthreads();                             // (the window table)
+  uint32_t mine[4] = {0u, 0u, 0u, 0u};         // lane k: masks of the warp's row k
+#pragma unroll
+  for (int k = 0; k < kEncRows; ++k) {
+    // a half-word without its sign is non-zero if adding 0x7FFF carries into its top bit
+    const uint32_t x = (w[k].x & 0x7FFF7FFFu) + 0x7FFF7FFFu, y = (w[k].y & 0x7FFF7FFFu) + 0x7FFF7FFFu;
+    const uint32_t m0 = __ballot_sync(0xFFFFFFFFu, (x & 0x8000u) != 0), m1 = __ballot_sync(0xFFFFFFFFu, static_cast<int>(x) < 0);
+    const uint32_t m2 = __ballot_sync(0xFFFFFFFFu, (y & 0x8000u) != 0), m3 = __ballot_sync(0xFFFFFFFFu, static_cast<int>(y) < 0);
+    if (lane == k) { mine[0] = m0; mine[1] = m1; mine[2] = m2; mine[3] = m3; }
+    if (a.emit) {
+      const int at = (warp * kEncRows + k) * 32 + lane;
+      const uint32_t bits = ((x >> 15) & 0x00010001u) | ((y >> 13) & 0x00040004u);
+      const uint2 e = sm.window[(bits | bits >> 15) & 15u];
+      reinterpret_cast<uint32_t*>(sm.vals)[at] = __byte_perm(w[k].x, w[k].y, e.x) & e.y;
+      sm.high[at] = w[k].y;
+      sm.nib[at] = static_cast<uint8_t>(e.x >> 16);
+    }
+  }
+  if (lane < kEncRows) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) sm.nz[i][warp * kEncRows + lane] = mine[i];
+  }
+  __syncthreads();
+
+  // ---- lists: threads 0..127 the empty slots of row tid, threads 128..255 the surplus weights of row tid - 128
+  const int row = tid & (kTileM - 1);
+  const bool surplus = tid >= kTileM;
+  uint32_t lo, hi;                             // windows whose even / odd position is listed
+  {
+    const uint32_t n0 = sm.nz[0][row], n1 = sm.nz[1][row], n2 = sm.nz[2][row], n3 = sm.nz[3][row];
+    const uint32_t two = (n0 & n1) | ((n0 | n1) & (n2 | n3)) | (n2 & n3);          // at least two non-zeros
+    if (surplus) {
+      lo = n0 & n1 & n2;                                                            // the weight at index 2 is a third one
+      hi = n3 & ((n0 & n1) | ((n0 | n1) & n2));                                     // the weight at index 3 is a third or fourth
+    } else {
+      lo = ~two & ~n0;                                                              // slot 0 (index 0) is empty
+      hi = ~two & ~(n1 | n2 | n3);                                                  // slot 1 is empty
+      const int n = __popc(n0) + __popc(n1) + __popc(n2) + __popc(n3);
+      const int sum = __reduce_add_sync(0xFFFFFFFFu, n);
+      if (lane == 0) atomicAdd(&sm.nnz, sum);
+    }
+  }
+  const uint32_t count = static_cast<uint32_t>(__popc(lo) + __popc(hi));
+  uint32_t tot = 0;
+  uint32_t at = scan_cta(count | (surplus ? count << 16 : 0u), sm.warp_tmp, &tot);   // low half: both kinds, high half: surplus
+  const int totS = static_cast<int>(tot >> 16), totE = static_cast<int>(tot & 0xFFFFu) - totS;
+  const int P = totS < totE ? totS : totE;     // pairs: the i-th surplus weight goes to the i-th empty slot
+  const int my_first = static_cast<int>(at >> 16);                                   // (surplus threads: index of the row's first surplus weight)
+  at &= 0xFFFFu;
+  for (uint32_t any = lo | hi; any; any &= any - 1u) {
+    const uint32_t bit = any & (0u - any), pos = static_cast<uint32_t>(row * kH) + 2u * (31u - __clz(bit));
+    if (lo & bit) sm.list[at++] = static_cast<uint16_t>(pos);
+    if (hi & bit) sm.list[at++] = static_cast<uint16_t>(pos + 1);
+  }
+  if (surplus) {
+    const int end = my_first + static_cast<int>(count);
+    sm.parked_end[row] = static_cast<uint16_t>(end < P ? end : P);
+    sm.moved[row] = 0;
+  }
+  if (a.emit) {
+    // metadata: eight windows per word, the even one in the low nibble of its byte
+#pragma unroll
+    for (int i = tid; i < kTileM * 4; i += kEncThreads) {
+      const uint2 v = reinterpret_cast<const uint2*>(sm.nib)[i];
+      const uint32_t x = v.x | v.x >> 4, y = v.y | v.y >> 4;
+      *reinterpret_cast<uint32_t*>(a.tc_meta + (tm * kTileM + (i >> 2)) * meta_ld + tk * (kTileK / 8) + (i & 3) * 4) = __byte_perm(x, y, 0x6420u);
     }
   }
   __syncthreads();
 
-  // value of the surplus weight at position rho of W_r (it lies in this thread's row)
-  auto surplus_value = [&](int rho) -> uint16_t {
-    const int s = rho - r * kH;                // slot of W_r in this row: window s / 2, in-window index 2 + (s & 1)
-    return wrow[4 * (s >> 1) + 2 + (s & 1)];
-  };
-  auto park = [&](int tau, uint16_t v) {       // the value goes into empty slot tau of the tile's value array
-    a.tc_vals[(tm * kTileM + tau / kH) * half_ld + tk * kH + tau % kH] = v;
-  };
-
-  // ---- chains, first walk: length of this row's chain, what a cut leaves over
-  const int i0 = offS, i1 = (offS + nS) < P ? (offS + nS) : (P > offS ? P : offS);   // pairs [i0, i1) of this row
-  int len = 0, n_cut = 0, n_sf = 0, n_dummy = 0;
-  if (i1 > i0) {
-    int tau = s_tau[i0], rho = s_rho[i0];
-    n_sf = 1;
-    bool cut = false;
-    for (int i = i0 + 1; i < i1; ++i) {
-      if (!cut) {
-        const int gt = s_tau[i] - tau, gr = s_rho[i] - rho;
-        const int need = 1 + (gt - 1) / kMaxd + (gr - 1) / kMaxd;
-        if (len + need > kChainCap) cut = true;
-        else { len += need; n_dummy += need - 1; tau = s_tau[i]; rho = s_rho[i]; ++n_sf; }
-      }
-      if (cut) ++n_cut;
+  // ---- pairs: thread t takes pairs [t * run, (t + 1) * run).  A pair that is the first of its row
+  //      (rho in another row than the one before) starts a chain and has no delta byte.
+  const uint16_t* const tau_list = sm.list;
+  const uint16_t* const rho_list = sm.list + totE;
+  const int run = (P + kEncThreads - 1) / kEncThreads;
+  const int p0 = tid * run < P ? tid * run : P, p1 = p0 + run < P ? p0 + run : P;
+  uint32_t bytes = 0;
+  int chains = 0;
+  uint32_t tau_before = 0, rho_before = 0xFFFFFFFFu;                                 // of the pair in front of this run
+  if (p0 > 0 && p0 < p1) { tau_before = tau_list[p0 - 1]; rho_before = rho_list[p0 - 1]; }
+  {
+    uint32_t tau = tau_before, rho = rho_before;
+    for (int i = p0; i < p1; ++i) {
+      const uint32_t nt = tau_list[i], nr = rho_list[i];
+      if (nr / kH == rho / kH) bytes += 1u + dummies(nt - tau, nr - rho);
+      else ++chains;
+      tau = nt;
+      rho = nr;
     }
   }
-  int tot_len = 0, tot_cut = 0;
-  const int off_len = block_exclusive_scan(len, s_warp, &tot_len);
-  const int off_cut = block_exclusive_scan(n_cut, s_warp, &tot_cut);
+  uint32_t tot_len = 0;
+  uint32_t pre = scan_cta(bytes, sm.warp_tmp, &tot_len);                             // delta bytes before this run (at most 4096 pairs + 2 * 546 dummies)
+  int tot_cut = 0;
+  {
+    // where every row's chain begins and ends: the run has to be walked again for it, by the few
+    // threads that hold the first or last pair of a row
+    uint32_t tau = tau_before, rho = rho_before, at_byte = pre;
+    for (int i = p0; i < p1; ++i) {
+      const uint32_t nt = tau_list[i], nr = rho_list[i];
+      if (nr / kH == rho / kH) at_byte += 1u + dummies(nt - tau, nr - rho);
+      else sm.first[nr / kH] = static_cast<uint16_t>(at_byte);
+      if (i + 1 == P || rho_list[i + 1] / kH != nr / kH) sm.last[nr / kH] = static_cast<uint16_t>(at_byte);
+      tau = nt;
+      rho = nr;
+    }
+  }
+  __syncthreads();
+  const bool has_chain = surplus && my_first < P && count > 0;
+  int len = has_chain ? sm.last[row] - sm.first[row] : 0;
+  if (__syncthreads_or(len > kChainCap)) {
+    // ---- a chain is cut: its row is walked for the last pair that fits, what follows is Residual
+    int n_cut = 0, lost = 0;
+    if (len > kChainCap) {
+      const int end = sm.parked_end[row];
+      int i = my_first + 1, fit = 0;
+      for (; i < end; ++i) {
+        const int need = 1 + static_cast<int>(dummies(tau_list[i] - tau_list[i - 1], rho_list[i] - rho_list[i - 1]));
+        if (fit + need > kChainCap) break;
+        fit += need;
+      }
+      n_cut = end - i;
+      lost = len - fit;
+      len = fit;
+      sm.parked_end[row] = static_cast<uint16_t>(i);
+    }
+    uint32_t t2 = 0;
+    const uint32_t before = scan_cta(static_cast<uint32_t>(lost) | static_cast<uint32_t>(n_cut) << 16, sm.warp_tmp, &t2);
+    if (surplus) sm.moved[row] = static_cast<uint16_t>(before & 0xFFFFu);
+    tot_cut = static_cast<int>(t2 >> 16);
+    tot_len -= t2 & 0xFFFFu;
+    if (a.emit && n_cut) {
+      uint32_t to = a.tile_dir[tile * 4 + 2] + (before >> 16);
+      const int end = my_first + static_cast<int>(count) < P ? my_first + static_cast<int>(count) : P;
+      for (int i = end - n_cut; i < end; ++i, ++to) {
+        a.res_rho[to] = rho_list[i];
+        a.res_val[to] = reinterpret_cast<const uint16_t*>(sm.high)[rho_list[i]];
+      }
+    }
+    __syncthreads();
+  }
   const int n_beyond = totS - P;               // surplus weights that found no empty slot
   if (!a.emit) {
-    if (r == 0) {
-      a.tile_dir[tile * 4 + 1] = static_cast<uint32_t>(tot_len);
+    if (tid == 0) {
+      a.tile_dir[tile * 4 + 1] = tot_len;
       a.tile_dir[tile * 4 + 3] = static_cast<uint32_t>(tot_cut + n_beyond);
     }
     return;
   }
 
-  // ---- second walk: write the chain, park the values, list the Residual entries
+  // ---- the code bytes (dummy points: a zero nibble moves nothing), the parked values, the chain starts
   const uint32_t pdd_off = a.tile_dir[tile * 4 + 0], res_off = a.tile_dir[tile * 4 + 2];
-  const long long ch = tile * kTileM + r;
-  if (i1 > i0) {
-    int tau = s_tau[i0], rho = s_rho[i0];
-    a.chain_tau0[ch] = static_cast<uint16_t>(tau);
-    a.chain_rho0[ch] = static_cast<uint16_t>(rho);
-    park(tau, surplus_value(rho));
-    uint8_t* code = a.pdd_bytes + pdd_off + off_len;
-    uint32_t res_at = res_off + off_cut;
-    int at = 0;
-    bool cut = false;
-    for (int i = i0 + 1; i < i1; ++i) {
-      if (!cut) {
-        int gt = s_tau[i] - tau, gr = s_rho[i] - rho;
-        const int need = 1 + (gt - 1) / kMaxd + (gr - 1) / kMaxd;
-        if (at + need > kChainCap) cut = true;
-        else {
-          while (gt > kMaxd) { code[at++] = static_cast<uint8_t>(kMaxd); gt -= kMaxd; }        // dummy points: a zero nibble moves nothing
-          while (gr > kMaxd) { code[at++] = static_cast<uint8_t>(kMaxd << 4); gr -= kMaxd; }
-          code[at++] = static_cast<uint8_t>(gt | gr << 4);
-          tau = s_tau[i];
-          rho = s_rho[i];
-          park(tau, surplus_value(rho));
+  const bool staged = tot_len <= static_cast<uint32_t>(kCodeStage);                  // (the metadata in that place has left)
+  uint8_t* const code = staged ? sm.nib : a.pdd_bytes + pdd_off;
+  const uint16_t* const high = reinterpret_cast<const uint16_t*>(sm.high);
+  {
+    uint32_t tau = tau_before, rho = rho_before;
+    for (int i = p0; i < p1; ++i) {
+      const uint32_t nt = tau_list[i], nr = rho_list[i], r = nr / kH;
+      const bool parked = i < sm.parked_end[r];
+      if (r == rho / kH) {
+        uint32_t gt = nt - tau, gr = nr - rho;
+        if (parked) {
+          uint8_t* c = code + (pre - sm.moved[r]);
+          pre += 1u + dummies(gt, gr);
+          while (gt > kMaxd) { *c++ = static_cast<uint8_t>(kMaxd); gt -= kMaxd; }
+          while (gr > kMaxd) { *c++ = static_cast<uint8_t>(kMaxd << 4); gr -= kMaxd; }
+          *c = static_cast<uint8_t>(gt | gr << 4);
+        } else {
+          pre += 1u + dummies(gt, gr);
         }
       }
-      if (cut) {                               // the chain is full: the rest of the row goes to the Residual layer
-        a.res_rho[res_at] = s_rho[i];
-        a.res_val[res_at] = surplus_value(s_rho[i]);
-        ++res_at;
-      }
+      if (parked) sm.vals[nt] = high[nr];
+      tau = nt;
+      rho = nr;
     }
-    a.chain_len[ch] = static_cast<uint8_t>(at);
-  } else {
-    a.chain_tau0[ch] = 0xFFFFu;
-    a.chain_rho0[ch] = 0xFFFFu;
-    a.chain_len[ch] = 0;
+  }
+  if (surplus) {
+    const long long ch = tile * kTileM + row;
+    a.chain_tau0[ch] = has_chain ? tau_list[my_first] : uint16_t{0xFFFFu};
+    a.chain_rho0[ch] = has_chain ? rho_list[my_first] : uint16_t{0xFFFFu};
+    a.chain_len[ch] = static_cast<uint8_t>(len);
   }
   // surplus weights beyond the number of empty slots: Residual entries after the cut leftovers
-  {
-    const int b0 = offS > P ? offS : P, b1 = offS + nS;
-    for (int i = b0; i < b1; ++i) {
-      const uint32_t at = res_off + tot_cut + (i - P);
-      a.res_rho[at] = s_rho[i];
-      a.res_val[at] = surplus_value(s_rho[i]);
-    }
+  for (int i = P + tid; i < totS; i += kEncThreads) {
+    const uint32_t to = res_off + static_cast<uint32_t>(tot_cut + (i - P)), rho = rho_list[i];
+    a.res_rho[to] = static_cast<uint16_t>(rho);
+    a.res_val[to] = high[rho];
   }
-  // layer statistics (Sec. 3.2 quotes their shares)
-  const int n_tc = nnz - nS;
-  atomicAdd(a.stats + 0, static_cast<unsigned long long>(nnz));
-  atomicAdd(a.stats + 1, static_cast<unsigned long long>(n_tc));
-  atomicAdd(a.stats + 2, static_cast<unsigned long long>(n_sf));
-  atomicAdd(a.stats + 4, static_cast<unsigned long long>(n_dummy));
-  if (r == 0) {
-    atomicAdd(a.stats + 3, static_cast<unsigned long long>(tot_cut + n_beyond));
-    atomicAdd(a.stats + 5, static_cast<unsigned long long>(totE - P + tot_cut));
+  chains = __reduce_add_sync(0xFFFFFFFFu, chains);
+  if (lane == 0 && chains) atomicAdd(&sm.n_chains, chains);
+  __syncthreads();
+  // ---- the tile leaves: 128 bytes of values per row, and the code bytes
+#pragma unroll
+  for (int i = tid; i < kTileM * kH / 8; i += kEncThreads)
+    *reinterpret_cast<uint4*>(a.tc_vals + (tm * kTileM + (i >> 3)) * half_ld + tk * kH + (i & 7) * 8) = reinterpret_cast<const uint4*>(sm.vals)[i];
+  if (staged)
+    for (uint32_t i = tid; i < tot_len; i += kEncThreads) a.pdd_bytes[pdd_off + i] = sm.nib[i];
+  // layer statistics (Sec. 3.2 quotes their shares): one addition per tile and counter.  Every parked
+  // weight that does not start a chain has one byte, the other bytes are dummy points.
+  if (tid < 6) {
+    const int n_sf = P - tot_cut;
+    const int v = tid == 0 ? sm.nnz : tid == 1 ? sm.nnz - totS : tid == 2 ? n_sf : tid == 3 ? tot_cut + n_beyond
+                : tid == 4 ? static_cast<int>(tot_len) - (n_sf - sm.n_chains) : totE - n_sf;
+    if (v) atomicAdd(a.stats + tid, static_cast<unsigned long long>(v));
   }
 }
 
-// Exclusive scan of the per-tile byte and entry counts into the offsets of the tile directory
-// (one CTA; the directory has a few thousand to a hundred thousand tiles).
+// Exclusive scan of the per-tile byte and entry counts into the offsets of the tile directory: one
+// CTA, each thread sums a run of consecutive tiles, so that there is one scan however many tiles
+// there are.
 __global__ void __launch_bounds__(1024)
 tl3_encode_scan_kernel(uint32_t* tile_dir, long long n_tiles, unsigned long long* totals) {
   __shared__ unsigned long long s_part[2][32];
-  __shared__ unsigned long long s_carry[2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) { s_carry[0] = 0; s_carry[1] = 0; }
-  __syncthreads();
-  for (long long base = 0; base < n_tiles; base += 1024) {
-    const long long t = base + tid;
-    unsigned long long v[2] = {0, 0};
-    if (t < n_tiles) { v[0] = tile_dir[t * 4 + 1]; v[1] = tile_dir[t * 4 + 3]; }
-    unsigned long long x[2] = {v[0], v[1]};
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-#pragma unroll
-      for (int d = 1; d < 32; d <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x[k], d);
-        if (lane >= d) x[k] += y;
-      }
-      if (lane == 31) s_part[k][warp] = x[k];
-    }
-    __syncthreads();
-    unsigned long long pre[2] = {s_carry[0], s_carry[1]};
-    for (int w = 0; w < warp; ++w) { pre[0] += s_part[0][w]; pre[1] += s_part[1][w]; }
-    if (t < n_tiles) {
-      tile_dir[t * 4 + 0] = static_cast<uint32_t>(pre[0] + x[0] - v[0]);
-      tile_dir[t * 4 + 2] = static_cast<uint32_t>(pre[1] + x[1] - v[1]);
-    }
-    __syncthreads();
-    if (tid == 1023) { s_carry[0] = pre[0] + x[0]; s_carry[1] = pre[1] + x[1]; }
-    __syncthreads();
+  const long long per = (n_tiles + 1023) / 1024;
+  const long long t0 = per * tid < n_tiles ? per * tid : n_tiles, t1 = t0 + per < n_tiles ? t0 + per : n_tiles;
+  uint4* dir = reinterpret_cast<uint4*>(tile_dir);
+  unsigned long long v[2] = {0, 0};
+  for (long long t = t0; t < t1; ++t) {
+    const uint4 d = dir[t];
+    v[0] += d.y;
+    v[1] += d.w;
   }
-  if (tid == 0) { totals[0] = s_carry[0]; totals[1] = s_carry[1]; }
+  unsigned long long x[2] = {v[0], v[1]};
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xFFFFFFFFu, x[k], d);
+      if (lane >= d) x[k] += y;
+    }
+    if (lane == 31) s_part[k][warp] = x[k];
+  }
+  __syncthreads();
+  unsigned long long at[2] = {x[0] - v[0], x[1] - v[1]};
+  for (int w = 0; w < warp; ++w) { at[0] += s_part[0][w]; at[1] += s_part[1][w]; }
+  if (tid == 1023) { totals[0] = at[0] + v[0]; totals[1] = at[1] + v[1]; }
+  for (long long t = t0; t < t1; ++t) {
+    uint4 d = dir[t];
+    d.x = static_cast<uint32_t>(at[0]);
+    d.z = static_cast<uint32_t>(at[1]);
+    dir[t] = d;
+    at[0] += d.y;
+    at[1] += d.w;
+  }
 }
 
 }  // namespace
@@ -310,6 +414,17 @@ tl3_encode_scan_kernel(uint32_t* tile_dir, long long n_tiles, unsigned long long
 
 namespace tl3 {
 namespace {
+// More than 48 KB of dynamic shared memory is opted into once per device (a repeated call sets the same value).
+cudaError_t configure_encode_kernel() {
+  static std::atomic<bool> done[64] = {};
+  int dev = 0;
+  if (cudaError_t e = cudaGetDevice(&dev)) return e;
+  if (dev < 64 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+  if (cudaError_t e = cudaFuncSetAttribute(tl3_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(EncodeSmem)))) return e;
+  if (dev < 64) done[dev].store(true, std::memory_order_release);
+  return cudaSuccess;
+}
+
 void release_encoded(void* p) {
   DeviceCanon* c = static_cast<DeviceCanon*>(p);
   if (!c) return;
@@ -360,8 +475,10 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
     a.chain_len = scratch + o_len;
     a.tile_dir = reinterpret_cast<uint32_t*>(scratch + o_dir);
     a.stats = reinterpret_cast<unsigned long long*>(scratch + o_stats);
+    a.vec = (reinterpret_cast<uintptr_t>(dW) & 7) == 0 && (ldw & 3) == 0;
     a.emit = 0;
-    tl3_encode_kernel<<<static_cast<unsigned>(m->n_tiles), kEncThreads, 0, st>>>(a);
+    TL3_ENC_CUDA(configure_encode_kernel());
+    tl3_encode_kernel<<<static_cast<unsigned>(m->n_tiles), kEncThreads, sizeof(EncodeSmem), st>>>(a);
     tl3_encode_scan_kernel<<<1, 1024, 0, st>>>(a.tile_dir, m->n_tiles, a.stats + 8);
     TL3_ENC_CUDA(cudaGetLastError());
     TL3_ENC_CUDA(cudaMemcpyAsync(totals, a.stats + 8, sizeof(totals), cudaMemcpyDeviceToHost, st));
@@ -373,7 +490,7 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
     a.res_rho = reinterpret_cast<uint16_t*>(var + o_res_rho);
     a.res_val = reinterpret_cast<uint16_t*>(var + o_res_val);
     a.emit = 1;
-    tl3_encode_kernel<<<static_cast<unsigned>(m->n_tiles), kEncThreads, 0, st>>>(a);
+    tl3_encode_kernel<<<static_cast<unsigned>(m->n_tiles), kEncThreads, sizeof(EncodeSmem), st>>>(a);
     TL3_ENC_CUDA(cudaGetLastError());
     if (keep_on_device) {
       TL3_ENC_CUDA(cudaMemcpyAsync(stats, a.stats, sizeof(stats), cudaMemcpyDeviceToHost, st));

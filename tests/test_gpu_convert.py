@@ -1,0 +1,57 @@
+"""Edges of the conversion kernels on the GPU: byte equality with the host library (needs a B200)."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def tl3():
+    import torch
+    assert torch.cuda.is_available()
+    from paper_2607_08786_b200 import build, tl3 as mod
+    build.build_library()
+    mod.lib()
+    return mod
+
+
+def _runs(M, K, run):
+    """Full and empty windows in runs of `run`: every boundary costs a dummy byte, so that a tile has
+    close to the largest possible number of pairs and more than 4096 code bytes."""
+    rng = np.random.default_rng([M, K, run])
+    W = (rng.standard_normal((M, K)) * 0.05 + 0.3).astype(np.float16)
+    window = np.arange(M)[:, None] * (K // 4) + np.arange(K)[None, :] // 4
+    W[(window // run) % 2 == 1] = 0
+    return W
+
+
+def _random(M, K, p):
+    rng = np.random.default_rng([M, K])
+    W = (rng.standard_normal((M, K)) * 0.02).astype(np.float16)
+    return np.where(rng.random((M, K)) < p, W, np.float16(0))
+
+
+@pytest.mark.parametrize("W,pitch,shift", [(_runs(128, 128, 9), 128, 0),         # code bytes beyond the staging area
+                                           (_random(129, 131, 0.5), 131, 0),     # one row and three columns over, odd pitch
+                                           (_random(7, 3, 1.0), 3, 0),           # less than a window
+                                           (_random(200, 250, 0.6), 252, 1),     # base not on 8 bytes
+                                           (_random(200, 250, 0.6), 252, 4),     # 8-byte windows, ragged last one
+                                           (_random(130, 900, 0.3), 904, 0)])
+def test_conversion_of_awkward_sources(tl3, W, pitch, shift):
+    """Container and packed blob, each byte for byte the host library's: tiles at the edges of the
+    matrix, sources that 8-byte loads cannot read, a tile with more code bytes than are staged."""
+    import torch
+    M, K = W.shape
+    ref = tl3.encode(W)
+    buf = torch.zeros(M * pitch + shift, dtype=torch.float16, device="cuda")
+    src = buf[shift:].view(M, pitch)[:, :K]
+    src.copy_(torch.from_numpy(W))
+    m = tl3.Matrix.encode_on_device(src)
+    for name in tl3.CANONICAL:
+        assert np.array_equal(m.canonical(name), ref.canonical(name)), name
+    assert m.serialize() == ref.serialize()
+    want = ref.pack()
+    assert np.array_equal(m.upload_packed_on_device().cpu().numpy(), want)
+    only = tl3.Matrix.encode_on_device(src, device_only=True)
+    assert np.array_equal(only.upload_packed_on_device().cpu().numpy(), want)
+    assert only.stats()["canonical_bytes"] == ref.stats()["canonical_bytes"]
