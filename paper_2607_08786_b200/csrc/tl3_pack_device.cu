@@ -4,12 +4,17 @@
 // chains per bank, the same number of transposed code words for every chain of a tile, the tails
 // as Residual entries).
 //
-// One CTA of 128 threads per 128 x 128 tile.  In turn a thread is the owner of canonical chain r
-// (to lift the parked values out of the value array), of 64 consecutive bank-major slot
-// coordinates (to list the empty slots and the surplus weights in that order), and of device
-// chain c (bank c / 4, run c % 4).  The kernel runs twice: a count pass that yields every tile's
+// One CTA of 256 threads per 128 x 128 tile.  In turn a thread is the owner of canonical chain r (to
+// lift the parked values out of the value array), of row r of a quarter of the value array (to mark
+// the empty slots), of 32 consecutive bank-major slot coordinates (to list the empty slots and the
+// surplus weights in that order), and of device chain c (bank c / 4, run c % 4).  The sets are
+// bitmaps over the bank-major coordinate -- a warp's ballot over 32 rows is one word of it -- so the
+// listing costs one step per set bit.  The kernel runs twice: a count pass that yields every tile's
 // number of code words and Residual entries, from which the host lays the blocks out exactly as
 // plan_device_layout() does, and an emit pass that writes the blocks.
+// What bounds it is the latency of a tile's serial steps (the chains), hidden by three tiles per SM.
+// With two-byte copies, a thread per 64 coordinates tested one by one and one thread sharing out the
+// banks, the two passes took 181 + 247 us on 5120 x 5120 at 50 % sparsity; now 57 + 77 us.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -27,6 +32,9 @@ namespace {
 
 constexpr int kSlots = kTileM * kH;        // 8192
 constexpr int kChains = 128;
+constexpr int kPackThreads = 256;
+constexpr int kFlagWords = kSlots / 32;    // 256: one per thread
+constexpr int kStagedPdd = 4096;           // canonical PDD bytes staged in shared memory (a tile has 1.5-2 KB as a rule)
 
 struct PackArgs {
   // canonical container (device copies)
@@ -63,67 +71,72 @@ __device__ __forceinline__ uint32_t pos_of_u(uint32_t u) {
 __device__ __forceinline__ uint32_t delta_bytes(uint32_t gt, uint32_t gr) { return (gt - 1) / 15 + (gr - 1) / 15 + 1; }
 __device__ __forceinline__ uint32_t align_up_d(uint32_t x, uint32_t a) { return (x + a - 1) / a * a; }
 
-// exclusive scan over the 128 threads of the CTA
-__device__ __forceinline__ int scan128(int v, int* s_warp, int* total) {
+// exclusive scan over the threads of the CTA (two 16-bit sums per word where a caller packs them)
+__device__ __forceinline__ uint32_t scan_cta(uint32_t v, uint32_t* s_warp, uint32_t* total) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int x = v;
+  uint32_t x = v;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    const int y = __shfl_up_sync(0xFFFFFFFFu, x, d);
+    const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
     if (lane >= d) x += y;
   }
   if (lane == 31) s_warp[warp] = x;
   __syncthreads();
-  int base = 0;
-  for (int w = 0; w < warp; ++w) base += s_warp[w];
-  *total = s_warp[0] + s_warp[1] + s_warp[2] + s_warp[3];
+  uint32_t base = 0, all = 0;
+#pragma unroll
+  for (int w = 0; w < kPackThreads / 32; ++w) {
+    base += w < warp ? s_warp[w] : 0u;
+    all += s_warp[w];
+  }
+  *total = all;
   __syncthreads();
   return base + x - v;
 }
 
 // dynamic shared memory of the pack kernel
 struct PackSmem {
-  uint16_t vals[kSlots];       // value slots of the tile by row-major position; parked values lifted out, later re-parked
-  uint16_t sval[kSlots];       // value of the surplus weight at bank-major coordinate u
-  uint16_t cand[kSlots];       // empty slots, ascending u
-  uint16_t sur[kSlots];        // surplus weights, ascending u
-  uint16_t sel[kSlots];        // selected empty slots, ascending u
-  uint32_t flag[kSlots / 32];  // bit u set: a surplus weight sits at u
-  int off_cand[kChains + 1];   // first candidate of the thread that owns u in [64 t, 64 t + 64)
-  int take[kChains], src[kChains], off_sel[kChains + 1];
-  int len[kChains];            // delta bytes of device chain c
+  uint16_t vals[kSlots];         // value slots of the tile by row-major position; parked values lifted out, later re-parked
+  uint16_t sval[kSlots];         // value of the surplus weight at bank-major coordinate u
+  uint16_t cand[kSlots];         // empty slots, ascending u
+  uint16_t sur[kSlots];          // surplus weights, ascending u
+  uint32_t flag[kFlagWords];     // bit u set: a surplus weight sits at u
+  uint32_t empty[kFlagWords];    // bit u set: slot u is empty
+  uint8_t pdd[kStagedPdd];       // canonical code bytes; later the chain starts and code words of the block
+  uint32_t bank_cand[33];        // empty slots before bank b
+  int carry[kChains];            // parked elements that run i hands on to the next
+  int len[kChains];              // delta bytes of device chain c
   int beyond[4];
-  int real_bytes;
-  int warp_tmp[4];
+  int real_bytes[4];
+  uint32_t warp_tmp[kPackThreads / 32];
 };
+static_assert(kStagedPdd >= 16 + 4 * kChains + 3 * 4 * kChains, "the block's info words, chain starts and code words fit the staging area");
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(kPackThreads, 3)
 tl3_pack_kernel(const PackArgs a) {
   extern __shared__ __align__(16) uint8_t pack_smem_raw[];
   PackSmem& sm = *reinterpret_cast<PackSmem*>(pack_smem_raw);
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long t = blockIdx.x;
   const long long tm = t / a.tiles_k, tk = t % a.tiles_k;
   const long long half_ld = a.K_pad / 2, meta_ld = a.K_pad / 8;
+  const uint4 dir = *reinterpret_cast<const uint4*>(a.tile_dir + t * 4);       // pdd_off, pdd_len, res_off, res_cnt
 
-  // (1) the tile's value slots; thread r copies row r
-  {
-    const uint16_t* src = a.tc_vals + (tm * kTileM + tid) * half_ld + tk * kH;
-    for (int s = 0; s < kH; ++s) sm.vals[tid * kH + s] = src[s];
-    sm.flag[tid] = 0u;
-    sm.flag[tid + 128] = 0u;
-    if (tid < 4) sm.beyond[tid] = 0;
-    if (tid == 0) sm.real_bytes = 0;
-  }
-  __syncthreads();
+  // (1) the tile's value slots and code bytes
+#pragma unroll
+  for (int i = tid; i < kSlots / 8; i += kPackThreads)
+    reinterpret_cast<uint4*>(sm.vals)[i] = *reinterpret_cast<const uint4*>(a.tc_vals + (tm * kTileM + (i >> 3)) * half_ld + tk * kH + (i & 7) * 8);
+  const bool staged = dir.y <= static_cast<uint32_t>(kStagedPdd);
+  if (staged)
+    for (uint32_t i = tid; i < dir.y; i += kPackThreads) sm.pdd[i] = a.pdd_bytes[dir.x + i];
+  sm.flag[tid] = 0u;
+  if (tid < 4) { sm.beyond[tid] = 0; sm.real_bytes[tid] = 0; }
+  const int canon_len = tid < kChains ? a.chain_len[t * kTileM + tid] : 0;
+  uint32_t tot = 0;
+  const uint32_t at0 = scan_cta(static_cast<uint32_t>(canon_len), sm.warp_tmp, &tot);
 
   // (2) Algorithm 1 over the canonical chains (one per tile row): lift every parked value out of
   //     its slot and note it at the bank-major coordinate of the position it belongs to
-  {
-    const int len = a.chain_len[t * kTileM + tid];
-    int tot = 0;
-    const int at0 = scan128(len, sm.warp_tmp, &tot);
-    const uint8_t* code = a.pdd_bytes + a.tile_dir[t * 4] + at0;
+  if (tid < kChains) {
     uint32_t tau = a.chain_tau0[t * kTileM + tid], rho = a.chain_rho0[t * kTileM + tid];
     auto lift = [&](uint32_t ta, uint32_t rh) {
       const uint32_t ur = u_of_pos(rh);
@@ -133,7 +146,8 @@ tl3_pack_kernel(const PackArgs a) {
     };
     if (tau != 0xFFFFu) {
       lift(tau, rho);
-      for (int k = 0; k < len; ++k) {
+      const uint8_t* code = staged ? sm.pdd + at0 : a.pdd_bytes + dir.x + at0;
+      for (int k = 0; k < canon_len; ++k) {
         const uint32_t b = code[k], dt = b & 15u, dr = b >> 4;
         tau += dt;
         rho += dr;
@@ -143,184 +157,199 @@ tl3_pack_kernel(const PackArgs a) {
   }
   __syncthreads();
 
-  // (3) empty slots and surplus weights in bank-major order; thread t owns u in [64 t, 64 t + 64)
+  // (3) empty slots and surplus weights in bank-major order.  A lane looks at one row: four of its
+  //     eight 16-byte chunks (warps 0-3 the first four bank groups, warps 4-7 the others), in the
+  //     order in which chunk j of row r holds the banks 4 (j ^ (r & 7)) ...: the lanes' accesses
+  //     then spread over all shared-memory banks.
+  {
+    const int row = (warp & 3) * 32 + lane;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int b4 = (warp >> 2) * 4 + g;
+      const uint4 v = reinterpret_cast<const uint4*>(sm.vals)[row * 8 + (b4 ^ (row & 7))];
+      const uint32_t word[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const uint32_t e0 = __ballot_sync(0xFFFFFFFFu, (word[i] & 0x7FFFu) == 0), e1 = __ballot_sync(0xFFFFFFFFu, (word[i] & 0x7FFF0000u) == 0);
+        if (lane == 2 * i) sm.empty[(4 * b4 + i) * 8 + (warp & 3)] = e0;
+        if (lane == 2 * i + 1) sm.empty[(4 * b4 + i) * 8 + 4 + (warp & 3)] = e1;
+      }
+    }
+  }
+  __syncthreads();
   int n_cand = 0, n_pairs = 0;
   {
-    int nc = 0, ns = 0;
-    for (uint32_t u = 64u * tid; u < 64u * tid + 64u; ++u) {
-      nc += (sm.vals[pos_of_u(u)] & 0x7FFFu) == 0 ? 1 : 0;
-      ns += (sm.flag[u >> 5] >> (u & 31u)) & 1u;
-    }
-    int oc = scan128(nc, sm.warp_tmp, &n_cand);
-    int os = scan128(ns, sm.warp_tmp, &n_pairs);
-    sm.off_cand[tid] = oc;
-    if (tid == 0) sm.off_cand[kChains] = n_cand;
-    for (uint32_t u = 64u * tid; u < 64u * tid + 64u; ++u) {
-      if ((sm.vals[pos_of_u(u)] & 0x7FFFu) == 0) sm.cand[oc++] = static_cast<uint16_t>(u);
-      if ((sm.flag[u >> 5] >> (u & 31u)) & 1u) sm.sur[os++] = static_cast<uint16_t>(u);
-    }
+    uint32_t e = sm.empty[tid], f = sm.flag[tid];
+    const uint32_t off = scan_cta(static_cast<uint32_t>(__popc(e)) | static_cast<uint32_t>(__popc(f)) << 16, sm.warp_tmp, &tot);
+    n_cand = static_cast<int>(tot & 0xFFFFu);
+    n_pairs = static_cast<int>(tot >> 16);
+    uint32_t oc = off & 0xFFFFu, os = off >> 16;
+    if ((tid & 7) == 0) sm.bank_cand[tid >> 3] = oc;
+    if (tid == 0) sm.bank_cand[32] = static_cast<uint32_t>(n_cand);
+    for (; e; e &= e - 1u) sm.cand[oc++] = static_cast<uint16_t>(tid * 32 + __ffs(e) - 1);
+    for (; f; f &= f - 1u) sm.sur[os++] = static_cast<uint16_t>(tid * 32 + __ffs(f) - 1);
   }
   __syncthreads();
 
   // (4) every bank gets a share of the parked elements proportional to its empty slots; its empty
-  //     slots are cut into four runs of equal count and run q uses its first slots (one thread:
-  //     what a run cannot take is carried to the next)
-  if (tid == 0) {
-    uint32_t cum = 0, carry = 0;
-    int base = 0;
-    for (int b = 0; b < 32; ++b) {
-      const uint32_t N_b = static_cast<uint32_t>(sm.off_cand[4 * b + 4] - sm.off_cand[4 * b]);
-      const uint32_t lo = n_cand ? static_cast<uint32_t>(static_cast<unsigned long long>(cum) * n_pairs / n_cand) : 0u;
-      cum += N_b;
-      const uint32_t hi = n_cand ? static_cast<uint32_t>(static_cast<unsigned long long>(cum) * n_pairs / n_cand) : 0u;
-      const uint32_t n_b = hi - lo;
-      for (uint32_t q = 0; q < 4; ++q) {
-        const uint32_t first = N_b * q / 4, size = N_b * (q + 1) / 4 - first;
-        const uint32_t want = n_b * (q + 1) / 4 - n_b * q / 4 + carry;
-        const uint32_t tk_ = want < size ? want : size;
-        carry = want - tk_;
-        sm.take[4 * b + q] = static_cast<int>(tk_);
-        sm.src[4 * b + q] = base + static_cast<int>(first);
-      }
-      base += static_cast<int>(N_b);
-    }
-  }
-  __syncthreads();
-  int n_sel = 0;
-  const int my_take = sm.take[tid];
-  const int my_off = scan128(my_take, sm.warp_tmp, &n_sel);
-  sm.off_sel[tid] = my_off;
-  for (int i = 0; i < my_take; ++i) sm.sel[my_off + i] = sm.cand[sm.src[tid] + i];
-  __syncthreads();
-
-  // (5) device chain c = the pairs [off, off + take) of run c; how many entries end beyond 0, 4, 8, 12 delta bytes
-  const int n_use = n_sel < n_pairs ? n_sel : n_pairs;
-  const int i0 = my_off, i1 = (my_off + my_take) < n_use ? (my_off + my_take) : (n_use > my_off ? n_use : my_off);
+  //     slots are cut into four runs of equal count and run q uses its first slots.  What a run
+  //     cannot take is carried to the next: with d = wanted - size of a run, S its inclusive prefix
+  //     sum, the carry out of run i is S_i - min(0, S_0 .. S_i), two scans over the 128 runs.
+  int my_take = 0, my_src = 0;
   {
-    uint32_t end = 0;
-    int by[4] = {0, 0, 0, 0};
-    for (int i = i0 + 1; i < i1; ++i) {
-      end += delta_bytes(static_cast<uint32_t>(sm.sel[i] - sm.sel[i - 1]), static_cast<uint32_t>(sm.sur[i] - sm.sur[i - 1]));
+    int want = 0, size = 0;
+    if (tid < kChains) {
+      const uint32_t b = static_cast<uint32_t>(tid) >> 2, q = tid & 3u;
+      const uint32_t c0 = sm.bank_cand[b], c1 = sm.bank_cand[b + 1], N_b = c1 - c0;
+      const uint32_t lo = n_cand ? c0 * n_pairs / n_cand : 0u, hi = n_cand ? c1 * n_pairs / n_cand : 0u;   // (<= 8192^2)
+      const uint32_t n_b = hi - lo, first = N_b * q / 4;
+      size = static_cast<int>(N_b * (q + 1) / 4 - first);
+      want = static_cast<int>(n_b * (q + 1) / 4 - n_b * q / 4);
+      my_src = static_cast<int>(c0 + first);
+    }
+    const int d = want - size;
+    int S = d;
 #pragma unroll
-      for (int w = 0; w < 4; ++w) by[w] += end > 4u * w ? 1 : 0;
+    for (int k = 1; k < 32; k <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, S, k);
+      if (lane >= k) S += y;
+    }
+    if (lane == 31) sm.warp_tmp[warp] = static_cast<uint32_t>(S);
+    __syncthreads();
+    for (int w = 0; w < warp && w < 4; ++w) S += static_cast<int>(sm.warp_tmp[w]);
+    __syncthreads();
+    int low = S < 0 ? S : 0;
+#pragma unroll
+    for (int k = 1; k < 32; k <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, low, k);
+      if (lane >= k && y < low) low = y;
+    }
+    if (lane == 31) sm.warp_tmp[warp] = static_cast<uint32_t>(low);
+    __syncthreads();
+    for (int w = 0; w < warp && w < 4; ++w) { const int y = static_cast<int>(sm.warp_tmp[w]); low = y < low ? y : low; }
+    if (tid < kChains) sm.carry[tid] = S - low;
+    __syncthreads();
+    if (tid < kChains) my_take = want + (tid ? sm.carry[tid - 1] : 0) - sm.carry[tid];
+  }
+  uint32_t n_sel = 0;
+  const int i0 = static_cast<int>(scan_cta(static_cast<uint32_t>(my_take), sm.warp_tmp, &n_sel));   // (n_sel <= n_pairs)
+  const uint16_t* const sel = sm.cand + my_src;                // this thread's run of empty slots
+
+  // (5) device chain c = the pairs [i0, i1) of run c.  One walk: for a chain of at most 0, 4, 8 and
+  //     12 delta bytes, how many bytes it has, how many entries move a value, how many are cut off.
+  int by[4] = {0, 0, 0, 0}, end_at[4] = {0, 0, 0, 0};
+  {
+    int end = 0;
+    for (int i = 1; i < my_take; ++i) {
+      end += static_cast<int>(delta_bytes(static_cast<uint32_t>(sel[i] - sel[i - 1]), static_cast<uint32_t>(sm.sur[i0 + i] - sm.sur[i0 + i - 1])));
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        if (end > 4 * w) ++by[w];
+        else end_at[w] = end;
+      }
     }
 #pragma unroll
-    for (int w = 0; w < 4; ++w)
-      if (by[w]) atomicAdd(&sm.beyond[w], by[w]);
+    for (int w = 0; w < 4; ++w) {
+      const int sum = __reduce_add_sync(0xFFFFFFFFu, by[w]);
+      const int real = __reduce_add_sync(0xFFFFFFFFu, my_take > 1 ? my_take - 1 - by[w] : 0);
+      if (lane == 0 && sum) atomicAdd(&sm.beyond[w], sum);
+      if (lane == 0 && real) atomicAdd(&sm.real_bytes[w], real);
+    }
   }
   __syncthreads();
   uint32_t n_words = 0;
   for (uint32_t w = 1; w < 4; ++w)
     if (512u * w + 4u * sm.beyond[w] < 512u * n_words + 4u * sm.beyond[n_words]) n_words = w;
-  const uint32_t cap = 4u * n_words;
-
-  // (6) first walk of the device chain: its delta bytes within the cap, what the cut leaves over
-  int n_bytes = 0, n_tail = 0, n_real = 0;
-  {
-    bool cut = false;
-    for (int i = i0 + 1; i < i1; ++i) {
-      const uint32_t need = delta_bytes(static_cast<uint32_t>(sm.sel[i] - sm.sel[i - 1]), static_cast<uint32_t>(sm.sur[i] - sm.sur[i - 1]));
-      if (cut || n_bytes + need > cap) { cut = true; ++n_tail; }
-      else { n_bytes += need; ++n_real; }
-    }
-  }
-  sm.len[tid] = n_bytes;
-  if (n_real) atomicAdd(&sm.real_bytes, n_real);
-  int tot_tail = 0;
-  const int off_tail = scan128(n_tail, sm.warp_tmp, &tot_tail);
-  const uint32_t canon_res_off = a.tile_dir[t * 4 + 2], canon_res_cnt = a.tile_dir[t * 4 + 3];
+  const int n_tail = n_words == 0 ? by[0] : n_words == 1 ? by[1] : n_words == 2 ? by[2] : by[3];
+  const int n_bytes = n_words == 0 ? end_at[0] : n_words == 1 ? end_at[1] : n_words == 2 ? end_at[2] : end_at[3];
+  const uint32_t tot_tail = static_cast<uint32_t>(sm.beyond[n_words]);
   const uint32_t pdd_len = n_words * 4u * kChains;
-  const uint32_t res_cnt = static_cast<uint32_t>(tot_tail + (n_pairs - n_use)) + canon_res_cnt;
-  __syncthreads();
+  const uint32_t n_left = static_cast<uint32_t>(n_pairs) - n_sel;
+  const uint32_t res_cnt = tot_tail + n_left + dir.w;
   if (!a.emit) {
     if (tid == 0) {
       a.sizes[t * 3 + 0] = pdd_len;
       a.sizes[t * 3 + 1] = res_cnt;
-      a.sizes[t * 3 + 2] = static_cast<uint32_t>(sm.real_bytes);
+      a.sizes[t * 3 + 2] = static_cast<uint32_t>(sm.real_bytes[n_words]);
     }
     return;
   }
+  if (tid < kChains) sm.len[tid] = n_bytes;
+  const uint32_t off_tail = scan_cta(static_cast<uint32_t>(n_tail), sm.warp_tmp, &tot);
 
-  // (7) the block
+  // (7) the block.  Info words, chain starts and code words are put together in shared memory.
   uint8_t* blk = a.blob + a.block_off[t];
-  const uint32_t block_bytes = align_up_d(kPddOff + align_up_d(pdd_len, 4) + 4u * res_cnt, 16);
-  {
-    // everything behind the metadata starts from zero (padding of short chains, alignment)
-    uint32_t* z = reinterpret_cast<uint32_t*>(blk + kInfoOff);
-    const uint32_t n = (align_up_d(block_bytes, kBlockAlign) - kInfoOff) / 4;
-    for (uint32_t i = tid; i < n; i += 128) z[i] = 0u;
-  }
+  const uint32_t block_bytes = align_up_d(kPddOff + pdd_len + 4u * res_cnt, 16);
+  constexpr uint32_t kHead = kPddOff - kInfoOff;               // info words and chain starts
+  const uint32_t head_words = (kHead + pdd_len) / 4;
+  uint32_t* head = reinterpret_cast<uint32_t*>(sm.pdd);
+  for (uint32_t i = tid; i < head_words; i += kPackThreads) head[i] = 0u;      // (padding of short chains)
   __syncthreads();
-  // chain slot w * 32 + l holds the w-th longest of the four chains of bank l (ties: lower chain first)
-  int slot;
-  {
+  uint32_t* res = reinterpret_cast<uint32_t*>(blk + kPddOff + pdd_len);
+  if (tid < kChains) {
+    // chain slot w * 32 + l holds the w-th longest of the four chains of bank l (ties: lower chain first)
     const int b = tid >> 2;
     int w = 0;
     for (int c = 4 * b; c < 4 * b + 4; ++c)
       if (sm.len[c] > n_bytes || (sm.len[c] == n_bytes && c < tid)) ++w;
-    slot = w * 32 + b;
-  }
-  uint32_t* res = reinterpret_cast<uint32_t*>(blk + kPddOff + align_up_d(pdd_len, 4));
-  {
+    const uint32_t slot = static_cast<uint32_t>(w * 32 + b);
     uint32_t hdr = 0xFFFFFFFFu;
-    uint8_t* code = blk + kPddOff;
-    uint32_t at = 0, res_at = static_cast<uint32_t>(off_tail);
-    bool cut = false;
-    for (int i = i0; i < i1; ++i) {
-      const uint32_t u = sm.sel[i], r_u = sm.sur[i];
-      const uint16_t v = sm.sval[r_u];
-      if (i == i0) {
+    uint8_t* code = sm.pdd + kHead + slot * 4u;
+    uint32_t at = 0;
+    const int kept = my_take - n_tail;
+    uint32_t u0 = 0, r0 = 0;
+    for (int i = 0; i < kept; ++i) {
+      const uint32_t u = sel[i], r_u = sm.sur[i0 + i];
+      if (i == 0) {
         hdr = u | r_u << 16;
       } else {
-        uint32_t gt = u - sm.sel[i - 1], gr = r_u - sm.sur[i - 1];
-        const uint32_t need = delta_bytes(gt, gr);
-        if (cut || at + need > cap) {          // the chain is full: the rest of its run goes to the Residual list
-          cut = true;
-          res[res_at++] = r_u | static_cast<uint32_t>(v) << 16;
-          continue;
-        }
-        auto put = [&](uint8_t b) { code[((at >> 2) * kChains + static_cast<uint32_t>(slot)) * 4u + (at & 3u)] = b; ++at; };
+        uint32_t gt = u - u0, gr = r_u - r0;
+        auto put = [&](uint8_t v) { code[(at >> 2) * (4u * kChains) + (at & 3u)] = v; ++at; };
         while (gt > 15) { put(0x0F); gt -= 15; }           // dummy points (a zero nibble moves nothing)
         while (gr > 15) { put(0xF0); gr -= 15; }
         put(static_cast<uint8_t>(gt | gr << 4));
       }
-      sm.vals[pos_of_u(u)] = v;                // the value is parked in its new slot
+      u0 = u;
+      r0 = r_u;
+      sm.vals[pos_of_u(u)] = sm.sval[r_u];     // the value is parked in its new slot
     }
-    reinterpret_cast<uint32_t*>(blk + kHdrOff)[slot] = hdr;
-  }
-  // surplus weights beyond the selected empty slots, then the canonical Residual entries
-  for (int i = n_use + tid; i < n_pairs; i += 128)
-    res[tot_tail + (i - n_use)] = sm.sur[i] | static_cast<uint32_t>(sm.sval[sm.sur[i]]) << 16;
-  for (uint32_t j = tid; j < canon_res_cnt; j += 128)
-    res[tot_tail + (n_pairs - n_use) + j] = u_of_pos(a.res_rho[canon_res_off + j]) | static_cast<uint32_t>(a.res_val[canon_res_off + j]) << 16;
-  __syncthreads();
-  // values: row r of the K-major 128-byte-swizzled image; word `bank` of the row holds both slots of one window
-  {
-    uint32_t* row = reinterpret_cast<uint32_t*>(blk + tid * 128);
-    for (uint32_t bank = 0; bank < 32; ++bank) {
-      const uint32_t p0 = pos_of_u(bank << 8 | static_cast<uint32_t>(tid));
-      row[bank] = static_cast<uint32_t>(sm.vals[p0]) | static_cast<uint32_t>(sm.vals[p0 + 1]) << 16;
+    head[4 + slot] = hdr;
+    for (int i = kept; i < my_take; ++i) {     // the chain is full: the rest of its run goes to the Residual list
+      const uint32_t r_u = sm.sur[i0 + i];
+      res[off_tail + static_cast<uint32_t>(i - kept)] = r_u | static_cast<uint32_t>(sm.sval[r_u]) << 16;
     }
-  }
-  // metadata in tensor-memory lane order
-  {
-    const int L = tid, mrow = (L & 7) + 16 * (L >> 4), half = (L >> 3) & 1;
-    uint32_t* meta = reinterpret_cast<uint32_t*>(blk + kMetaOff);
-    for (int kb = 0; kb < 4; ++kb) {
-      const uint8_t* lo = a.tc_meta + (tm * kTileM + mrow) * meta_ld + tk * (kTileK / 8) + 4 * kb + 2 * half;
-      const uint8_t* hi = a.tc_meta + (tm * kTileM + mrow + 8) * meta_ld + tk * (kTileK / 8) + 4 * kb + 2 * half;
-      meta[L * 4 + kb] = static_cast<uint32_t>(lo[0]) | static_cast<uint32_t>(lo[1]) << 8 |
-                         static_cast<uint32_t>(hi[0]) << 16 | static_cast<uint32_t>(hi[1]) << 24;
+  } else {
+    // meanwhile the other warps: metadata in tensor-memory lane order ...
+    {
+      const int L = tid - kChains, mrow = (L & 7) + 16 * (L >> 4), half = (L >> 3) & 1;
+      const uint8_t* m0 = a.tc_meta + (tm * kTileM + mrow) * meta_ld + tk * (kTileK / 8);
+      const uint4 lo = *reinterpret_cast<const uint4*>(m0), hi = *reinterpret_cast<const uint4*>(m0 + 8 * meta_ld);
+      const uint32_t sel2 = half ? 0x7632u : 0x5410u;           // this half's two bytes of either word
+      reinterpret_cast<uint4*>(blk + kMetaOff)[L] = make_uint4(__byte_perm(lo.x, hi.x, sel2), __byte_perm(lo.y, hi.y, sel2),
+                                                               __byte_perm(lo.z, hi.z, sel2), __byte_perm(lo.w, hi.w, sel2));
     }
+    // ... and surplus weights beyond the selected empty slots, the canonical Residual entries, the padding
+    const uint32_t j0 = static_cast<uint32_t>(tid - kChains);
+    for (uint32_t i = n_sel + j0; i < static_cast<uint32_t>(n_pairs); i += kPackThreads - kChains)
+      res[tot_tail + (i - n_sel)] = sm.sur[i] | static_cast<uint32_t>(sm.sval[sm.sur[i]]) << 16;
+    for (uint32_t j = j0; j < dir.w; j += kPackThreads - kChains)
+      res[tot_tail + n_left + j] = u_of_pos(a.res_rho[dir.z + j]) | static_cast<uint32_t>(a.res_val[dir.z + j]) << 16;
+    const uint32_t n_pad = (align_up_d(block_bytes, kBlockAlign) - (kPddOff + pdd_len + 4u * res_cnt)) / 4;
+    if (j0 < n_pad) res[res_cnt + j0] = 0u;
   }
   if (tid == 0) {
-    uint32_t* info = reinterpret_cast<uint32_t*>(blk + kInfoOff);
-    info[0] = pdd_len;
-    info[1] = res_cnt;
-    info[2] = n_words;
-    DirEntry* dir = reinterpret_cast<DirEntry*>(a.blob + a.dir_offset);
-    dir[t] = DirEntry{static_cast<uint32_t>(a.block_off[t] / 16), block_bytes, pdd_len, res_cnt};
+    head[0] = pdd_len;
+    head[1] = res_cnt;
+    head[2] = n_words;
+    DirEntry* out = reinterpret_cast<DirEntry*>(a.blob + a.dir_offset);
+    out[t] = DirEntry{static_cast<uint32_t>(a.block_off[t] / 16), block_bytes, pdd_len, res_cnt};
   }
+  __syncthreads();
+  // values: row r of the K-major 128-byte-swizzled image; word `bank` of the row holds both slots of one window
+#pragma unroll
+  for (int i = tid; i < kSlots / 8; i += kPackThreads)
+    reinterpret_cast<uint4*>(blk)[i] = reinterpret_cast<const uint4*>(sm.vals)[i ^ ((i >> 3) & 7)];
+  for (uint32_t i = tid; i < head_words / 4; i += kPackThreads) reinterpret_cast<uint4*>(blk + kInfoOff)[i] = reinterpret_cast<const uint4*>(head)[i];
 }
 
 }  // namespace
@@ -419,7 +448,7 @@ extern "C" int tl3_plan_device(tl3_matrix* m, void* stream) {
   TL3_PK_CUDA(cudaMalloc(reinterpret_cast<void**>(&d_sizes), static_cast<size_t>(m->n_tiles) * 12));
   a.sizes = d_sizes;
   a.emit = 0;
-  tl3_pack_kernel<<<static_cast<unsigned>(m->n_tiles), 128, sizeof(PackSmem), st>>>(a);
+  tl3_pack_kernel<<<static_cast<unsigned>(m->n_tiles), kPackThreads, sizeof(PackSmem), st>>>(a);
   std::vector<uint32_t> sizes;
   int rc = TL3_OK;
   try { sizes.resize(static_cast<size_t>(m->n_tiles) * 3); } catch (const std::bad_alloc&) { rc = TL3_ERR_NO_MEMORY; }
@@ -455,7 +484,7 @@ extern "C" int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream) {
     a.block_off = d_off;
     a.dir_offset = m->dir_offset;
     a.emit = 1;
-    tl3_pack_kernel<<<static_cast<unsigned>(m->n_tiles), 128, sizeof(PackSmem), st>>>(a);
+    tl3_pack_kernel<<<static_cast<unsigned>(m->n_tiles), kPackThreads, sizeof(PackSmem), st>>>(a);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);          // header, offsets and the canonical copies are released below
