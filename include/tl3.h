@@ -204,13 +204,13 @@ int tl3_workspace_init(void* workspace, size_t bytes, void* stream);
  * folded into the same accumulators, one final reduction).
  *   X: device, fp16, K x N row-major, leading dimension ldx >= N, ldx % 8 == 0, 16-byte aligned.
  *   Y: device, fp16, M x N row-major, leading dimension ldy >= N; fully overwritten.
- *   1 <= N <= TL3_MAX_N.  Up to 64 columns are one kernel launch (the decode-phase case the
- *   kernels are built for); wider blocks are processed 64 columns at a time, each streaming W
- *   again.  fp32 accumulation, fp16 round-to-nearest-even output.  W and X are assumed finite (an
- *   empty slot multiplies an exact zero with an element of X).
+ *   1 <= N <= TL3_MAX_N.  One kernel launch; W is streamed and decoded once for up to 64 columns (the
+ *   decode phase), beyond that once for every 64 to 256 columns.  fp32 accumulation, fp16
+ *   round-to-nearest-even output.  W and X are assumed finite (an empty slot multiplies an exact zero
+ *   with an element of X).
  * Asynchronous on `stream`; allocates nothing; does not synchronise.  Calls that share a
  * workspace must not overlap on the GPU; the workspace must hold tl3_workspace_bytes(m, N) bytes
- * for THIS N (it grows with N: 16, 32 or 64 columns of partial sums per slot), the call cannot
+ * for THIS N (it grows with N up to 256: that many columns of partial sums per CTA), the call cannot
  * check that.  Calls on different streams, each with its own workspace, may be in flight together.
  * A row-tile shared by several CTAs is finished by the CTA that owns its first tile, which waits
  * (bounded, status code 11) for CTAs with a higher index; that those get to run while other

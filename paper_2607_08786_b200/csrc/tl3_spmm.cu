@@ -31,21 +31,13 @@
 #include <mutex>
 #include <vector>
 
+#include "tl3_device.cuh"
 #include "tl3_internal.h"
 
 namespace tl3 {
 
 static thread_local int g_last_cuda_error = 0;
 void set_cuda_error(int e) { g_last_cuda_error = e; }
-
-#define TL3_CUDA(expr)                                        \
-  do {                                                        \
-    cudaError_t e_ = (expr);                                  \
-    if (e_ != cudaSuccess) {                                  \
-      tl3::set_cuda_error(static_cast<int>(e_));              \
-      return TL3_ERR_CUDA;                                    \
-    }                                                         \
-  } while (0)
 
 // ---------------------------------------------------------------------------------------------
 // Kernel configuration
@@ -62,26 +54,11 @@ constexpr int kEpilogueWarp0 = kDecodeWarp0 + 4 * kGroups;
 constexpr int kThreads = (kEpilogueWarp0 + 4) * 32;
 constexpr int kSetupBarrier = 2 + kGroups;   // named barriers: 0 = whole CTA, 1 + kGroups = epilogue warps, 2 + kGroups = set-up
 constexpr int kMaxStages = 8;
-constexpr uint32_t kWrBytes = 16384;
 constexpr int kMaxWrBuffers = 5;          // W_r ring: tile i uses buffer i % num_wr (4 or 5, see the launcher)
 constexpr uint32_t kTmemCols = 256;
 constexpr uint32_t kColMetaT = 128;       // + 4 * (W_r buffer): metadata of W_t, four columns per tile in flight
 constexpr uint32_t kColMetaR = 152;       // two columns of 0xEEEEEEEE
-constexpr uint32_t kSmemLimit = 232448;   // 227 KB
 constexpr uint32_t kBarrierBytes = 1024;
-constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s without progress, per wait
-#ifndef TL3_TRYWAIT_HINT_NS
-#define TL3_TRYWAIT_HINT_NS 20000u
-#endif
-constexpr uint32_t kTryWaitHintNs = TL3_TRYWAIT_HINT_NS;     // how long one barrier probe may park the thread
-
-// status codes written to the workspace status word (0 = ok)
-enum : uint32_t {
-  kStProducer = 1, kStDecodeFull = 2, kStDecodeWrFree = 3, kStMmaDecoded = 4, kStMmaAccEmpty = 5,
-  kStEpilogueAccFull = 6, kStDrain = 7, kStClearWrFree = 8, kStDecodeWrReady = 9, kStEpilogueTail = 10, kStEpilogueFlags = 11, kStMmaX = 12,
-  kStBadBlock = 16           // a block's lengths or a decoded position were out of range (+ detail in bits 8..)
-};
-
 struct KernelArgs {
   const uint8_t* blob;       // base of the packed blob (device)
   const DirEntry* dir;       // tile directory (device)
@@ -125,258 +102,8 @@ __device__ __forceinline__ long long clock_now() { long long c; asm volatile("mo
 #endif
 
 // ---------------------------------------------------------------------------------------------
-// PTX helpers
-// ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-__device__ __forceinline__ unsigned long long global_timer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {   // more bytes to come, no arrival
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-// One probe of the barrier phase.  The hint lets the hardware park the thread (up to that many
-// nanoseconds, or until the phase completes) instead of spinning, so waiting warps do not take
-// issue slots from the warps that have work.
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n\t.reg .pred q;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2, %3;\n\t"
-      "selp.u32 %0, 1, 0, q;\n\t}"
-      : "=r"(done) : "r"(bar), "r"(parity), "r"(kTryWaitHintNs) : "memory");
-  return done != 0;
-}
-
-// Shared state every wait looks at: the abort flag (set by whoever gives up first) and the
-// status word in global memory.
-struct WaitCtx {
-  volatile int* abort_flag;
-  unsigned int* status;
-};
-
-// Bounded wait.  Returns false if the CTA is aborting (this or another waiter ran out of time).
-// The limit runs from the moment THIS wait began to look slow (its sixteenth unsuccessful probe), not
-// from the start of the kernel: a wait that completes is progress, so a long launch, or one whose
-// context was switched out for a while earlier on, does not use up the allowance of later waits.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& w, uint32_t code) {
-  unsigned long long t_slow = 0;
-  for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
-    if ((it & 15u) == 15u) {
-      if (*w.abort_flag) return false;
-      const unsigned long long now = global_timer();
-      if (t_slow == 0) t_slow = now;
-      if (now - t_slow > kWaitLimitNs) {
-        atomicCAS(w.status, 0u, code);
-        *w.abort_flag = 1;
-        return false;
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
-__device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void named_bar_sync(int id, int threads) {
-  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
-// barrier + AND-reduction of a predicate over the `threads` threads that use barrier `id`
-__device__ __forceinline__ bool named_bar_all(int id, int threads, bool pred) {
-  uint32_t out;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\t"
-      "setp.ne.b32 q, %3, 0;\n\t"
-      "bar.red.and.pred p, %1, %2, q;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(out) : "r"(id), "r"(threads), "r"(static_cast<uint32_t>(pred)) : "memory");
-  return out != 0;
-}
-
-// The weight blocks are read once: they are marked evict-first in L2 so that what is read again
-// (X, the kernel's own code, partial sums) is not pushed out by the stream.
-__device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
-  uint64_t policy;
-  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar), "l"(policy) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
-  asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-               ::"r"(dst), "l"(map), "r"(c0), "r"(c1), "r"(bar) : "memory");
-}
-
-// Programmatic dependent launch: the next kernel on the stream may be scheduled as soon as every
-// CTA of this one has said so (it still cannot take an SM before a CTA here exits), and a kernel
-// must call pdl_wait() before it reads what its predecessor wrote or writes what its
-// predecessor may still read.
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-// One lane of a converged warp; the caller keeps every operand warp-uniform so that the
-// single-thread instructions (bulk copies, MMAs, commits) take uniform registers directly.
-__device__ __forceinline__ bool elect_one() {
-  uint32_t pred;
-  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(pred));
-  return pred != 0;
-}
-
-// D[tmem] (+)= A_sparse[smem] * B[smem] with the 2-bit metadata at e_tmem.  The shared-memory
-// descriptors are passed as their low words (start address field) and one common high word each.
-__device__ __forceinline__ void umma_sp_f16(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
-                                            uint32_t e_tmem, uint32_t idesc, uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
-      "setp.ne.b32 p, %7, 0;\n\t"
-      "mov.b64 da, {%1, %2};\n\t"
-      "mov.b64 db, {%3, %4};\n\t"
-      "tcgen05.mma.sp.cta_group::1.kind::f16 [%0], da, db, [%5], %6, p;\n\t}"
-      ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(e_tmem), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-// Positions in a block are bank-major slot coordinates u = bank << 8 | slot-in-window << 7 | row,
-// where bank is the 32-bit word of the 128-byte (swizzled) row that holds the slot's window.  The
-// byte offset of slot u inside the 128 x 128-byte K-major image is therefore a bit-field move:
-// row * 128 + bank * 4 + slot-in-window * 2.  The packer orders both PDD streams by u and gives
-// lane l of a decode warp a chain whose empty slots all lie in bank l.
-__device__ __forceinline__ uint32_t swizzled_offset(uint32_t u) { return ((u & 0x7Fu) << 7) | ((u >> 6) & 0x7Eu); }
-
-// Epilogue of tl3_spmm_ex: y = act(sum + bias), in fp32, before the rounding to fp16.  A real
-// call, not inlined: it is used from many unrolled places, and a kernel image that grows by tens of
-// kilobytes costs every launch time at its start.
-__device__ __noinline__ float finish(float v, float bias, int act) {
-  v += bias;
-  if (act == TL3_ACT_RELU) return fmaxf(v, 0.f);
-  if (act == TL3_ACT_SILU) return v / (1.f + __expf(-v));
-  if (act == TL3_ACT_GELU_TANH) return 0.5f * v * (1.f + tanhf(0.7978845608f * (v + 0.044715f * v * v * v)));
-  return v;
-}
-
-template <int NPAD> struct TmemLd;
-template <> struct TmemLd<16> {
-  static __device__ __forceinline__ void ld(uint32_t taddr, uint32_t* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                 : "r"(taddr) : "memory");
-  }
-};
-template <> struct TmemLd<32> {
-  static __device__ __forceinline__ void ld(uint32_t taddr, uint32_t* v) {
-    TmemLd<16>::ld(taddr, v);
-    TmemLd<16>::ld(taddr + 16, v + 16);
-  }
-};
-template <> struct TmemLd<64> {
-  static __device__ __forceinline__ void ld(uint32_t taddr, uint32_t* v) {
-    TmemLd<32>::ld(taddr, v);
-    TmemLd<32>::ld(taddr + 32, v + 32);
-  }
-};
-
-// CTA c of G owns tiles [c*T/G, (c+1)*T/G); the CTA that owns tile t.  In 32 bits: the launcher
-// refuses matrices with (G + 1) * T >= 2^32 (hundreds of gigabytes), and a 64-bit division costs a
-// CTA 0.15 us each at its cold start, where there are three of them.
-__device__ __forceinline__ uint32_t range_begin(uint32_t c, uint32_t T, uint32_t G) { return c * T / G; }
-__device__ __forceinline__ int owner_of(uint32_t t, uint32_t T, uint32_t G) { return static_cast<int>(((t + 1u) * G - 1u) / T); }
-
-// ---------------------------------------------------------------------------------------------
 // The kernel
 // ---------------------------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
-  uint32_t v;
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ uint32_t lds_u16(uint32_t addr) {
-  uint16_t v;
-  asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(addr));
-  return v;
-}
-__device__ __forceinline__ void sts_u16(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.u16 [%0], %1;" ::"r"(addr), "h"(static_cast<uint16_t>(v)) : "memory");
-}
-__device__ __forceinline__ void sts_zero16B(uint32_t addr) {
-  asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(addr), "r"(0u) : "memory");
-}
-
-// Algorithm 1 for one chain, one code word (four delta bytes) at a time.  `pos` carries offset_t in
-// its low and offset_r in its high 16 bits (both as bank-major coordinates u), so one add advances
-// both cursors and two shift/mask pairs form both byte offsets.  Within a round all positions are
-// formed first, then all W_t loads are issued, then all stores, so that the shared-memory round
-// trips of different entries overlap.  (Rounds of two code words, and a software-pipelined loop
-// that issues the next round's loads before this round's stores, both measured slower.)
-
-// packed byte offsets (W_t offset low, W_r offset high) of the packed positions `pos`
-__device__ __forceinline__ uint32_t swizzled_offset2(uint32_t pos) { return ((pos & 0x007F007Fu) << 7) | ((pos >> 6) & 0x007E007Eu); }
-
-// Positions are checked (< 8192 slots per tile) before they become addresses; a violation is
-// reported in *bad and the entry is skipped.  The code words of a tile are stored transposed
-// (word k of chain slot j at (k * 128 + j) * 4) and every chain has `n_words` of them (<= 3, padded
-// with zero bytes = dummy points), so the loads are conflict free and the loop is warp-uniform.
-__device__ __forceinline__ void decode_chain(uint32_t stage, uint32_t wr, uint32_t hdr, uint32_t code_addr, uint32_t n_words, uint32_t* bad) {
-  if (hdr == 0xFFFFFFFFu) return;                       // empty chain
-  if (hdr & 0xE000E000u) { *bad = 1u; return; }
-  uint32_t pos = hdr;
-  uint32_t w[3] = {0u, 0u, 0u};
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    if (static_cast<uint32_t>(k) < n_words) w[k] = lds_u32(code_addr + k * 512);
-  {                                                     // first pair: absolute 16-bit positions
-    const uint32_t off2 = swizzled_offset2(pos);
-    const uint32_t at = stage + (off2 & 0xFFFFu);
-    const uint32_t v = lds_u16(at);
-    sts_u16(at, 0);                                     // the slot it was parked in is empty again
-    sts_u16(wr + (off2 >> 16), v);                      // the value goes to its own position in W_r
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {                         // one code word = four delta bytes
-    if (static_cast<uint32_t>(k) >= n_words) break;
-    const uint32_t bytes = w[k];
-    uint32_t off2[4], val[4];
-    bool real[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const uint32_t bt = __byte_perm(bytes, 0u, 0x4440u + q);    // delta byte q
-      const uint32_t delta = (bt * 0x1001u) & 0x000F000Fu;        // t delta | r delta << 16
-      pos += delta;
-      real[q] = ((delta - 0x00010001u) & 0x80008000u) == 0u;      // both nibbles non-zero (else a dummy point)
-      off2[q] = swizzled_offset2(pos);
-    }
-    // both cursors only grow, so the last position of the round bounds them all
-    if (pos & 0xE000E000u) {
-      *bad = 2u;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) real[q] = false;
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (real[q]) val[q] = lds_u16(stage + (off2[q] & 0xFFFFu));
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-      if (real[q]) { sts_u16(stage + (off2[q] & 0xFFFFu), 0); sts_u16(wr + (off2[q] >> 16), val[q]); }
-  }
-}
-
 // XT: the activations are given as X^T (N x K row-major, the [batch, hidden] layout of an inference
 // stack, Sec. 2.1) and the result is written as Y^T (N x M row-major).  The X tile then arrives as
 // two boxes of 64 k-values (128 bytes per row, 128-byte swizzle) and is a K-major B operand.
@@ -896,13 +623,7 @@ __global__ void bounded_wait_probe_kernel(unsigned int* status, unsigned int* ou
 // ---------------------------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------------------------
-struct DeviceInfo {
-  int sm_count = 0;
-  int cc_major = 0;
-  bool ok = false;
-};
-
-static int device_info(DeviceInfo* out) {
+int device_info(DeviceInfo* out) {
   int dev = 0;
   TL3_CUDA(cudaGetDevice(&dev));
   static std::mutex mu;
@@ -919,11 +640,7 @@ static int device_info(DeviceInfo* out) {
   return TL3_OK;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
-                                  const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_tiled_fn() {
+EncodeTiledFn encode_tiled_fn() {
   static EncodeTiledFn fn = []() -> EncodeTiledFn {
     void* p = nullptr;
     cudaDriverEntryPointQueryResult q;
@@ -937,15 +654,15 @@ static EncodeTiledFn encode_tiled_fn() {
 
 static inline int n_pad_of(int N) { return N <= 16 ? 16 : N <= 32 ? 32 : 64; }
 
-struct WorkspaceLayout {
-  size_t status_off = 0, flags_off = 256, partials_off = 0, total = 0;
-};
-
-static WorkspaceLayout workspace_layout(const tl3_matrix* m, int n_pad, int sm_count) {
+// Up to 64 columns a CTA has two partial-sum slots of n_pad columns.  The wide kernel uses one per CTA
+// (only a CTA that begins inside a row-tile hands a partial sum on) of as many columns as a pass may
+// have; 128 of those are as many bytes as the two slots of 64.
+WorkspaceLayout workspace_layout(int N, int sm_count) {
   WorkspaceLayout w;
-  (void)m;
   w.partials_off = (256 + static_cast<size_t>(2) * sm_count * 4 + 4095) / 4096 * 4096;
-  w.total = w.partials_off + static_cast<size_t>(2) * sm_count * n_pad * 128 * sizeof(float);
+  int columns = 2 * n_pad_of(N);
+  if (N > 128) columns = N < kWideColumns ? (N + 15) / 16 * 16 : kWideColumns;
+  w.total = w.partials_off + static_cast<size_t>(columns) * sm_count * 128 * sizeof(float);
   return w;
 }
 
@@ -1031,7 +748,7 @@ size_t tl3_workspace_bytes(const tl3_matrix* m, int N) {
   if (!m || N < 1 || N > TL3_MAX_N) return 0;
   tl3::DeviceInfo di;
   if (tl3::device_info(&di) != TL3_OK) return 0;
-  return tl3::workspace_layout(m, tl3::n_pad_of(N), di.sm_count).total;
+  return tl3::workspace_layout(N, di.sm_count).total;
 }
 
 int tl3_workspace_init(void* workspace, size_t bytes, void* stream) {
@@ -1095,7 +812,7 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   const long long total = m->n_tiles;
   const int grid = static_cast<int>(total < di.sm_count ? total : di.sm_count);
   if (static_cast<unsigned long long>(total) * static_cast<unsigned long long>(grid + 1) >= (1ull << 32)) return TL3_ERR_UNSUPPORTED;   // the kernel splits the tiles in 32-bit arithmetic
-  const WorkspaceLayout wl = workspace_layout(m, n_pad, di.sm_count);
+  const WorkspaceLayout wl = workspace_layout(N, di.sm_count);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   KernelArgs args;
   args.blob = static_cast<const uint8_t*>(m->dptr);
@@ -1155,9 +872,12 @@ int tl3_spmm_ex(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_
   if (!m->dptr) return TL3_ERR_NOT_UPLOADED;
   if (N < 1 || N > TL3_MAX_N) return TL3_ERR_UNSUPPORTED;
   if (ldx < N || ldy < N) return TL3_ERR_INVALID_ARG;
-  // Wider activation blocks are processed 64 columns at a time; every block streams W again, so
-  // beyond N = 64 the time grows in proportion to N (this kernel targets the decode phase; the
-  // paper, too, loses to the dense GEMM at large N, Sec. 6).
+  if (N > 64) {
+    const int rc = tl3::spmm_wide(m, X, ldx, Y, ldy, N, ep, false, workspace, stream);
+    if (rc != tl3::kWideNoPlan) return rc;
+  }
+  // One launch of up to 64 columns; a wider product gets here only with blocks so large that the wide
+  // kernel's buffers do not fit beside them.
   for (int n0 = 0; n0 < N; n0 += 64) {
     const int nb = N - n0 < 64 ? N - n0 : 64;
     const int rc = spmm_block(m, static_cast<const uint16_t*>(X) + n0, ldx, static_cast<uint16_t*>(Y) + n0, ldy, nb, ep, false, workspace, stream);
@@ -1175,6 +895,10 @@ int tl3_spmm_nt(const tl3_matrix* m, const void* Xt, int64_t ldxt, void* Yt, int
   if (!m->dptr) return TL3_ERR_NOT_UPLOADED;
   if (N < 1 || N > TL3_MAX_N) return TL3_ERR_UNSUPPORTED;
   if (ldxt < m->K || ldyt < m->M) return TL3_ERR_INVALID_ARG;
+  if (N > 64) {
+    const int rc = tl3::spmm_wide(m, Xt, ldxt, Yt, ldyt, N, ep, true, workspace, stream);
+    if (rc != tl3::kWideNoPlan) return rc;
+  }
   for (int n0 = 0; n0 < N; n0 += 64) {                           // 64 rows of X^T (= columns of X) per launch
     const int nb = N - n0 < 64 ? N - n0 : 64;
     const int rc = spmm_block(m, static_cast<const uint16_t*>(Xt) + static_cast<int64_t>(n0) * ldxt, ldxt,
@@ -1237,7 +961,7 @@ int tl3_spmm_static_scratch(const tl3_matrix* m, const void* X, int64_t ldx, voi
   if (N < 1 || N > TL3_MAX_N) return TL3_ERR_UNSUPPORTED;
   tl3::DeviceInfo di;
   if (int rc = tl3::device_info(&di)) return rc;
-  const tl3::WorkspaceLayout wl = tl3::workspace_layout(m, tl3::n_pad_of(N), di.sm_count);
+  const tl3::WorkspaceLayout wl = tl3::workspace_layout(N, di.sm_count);
   if (wl.total > TL3_STATIC_SCRATCH_BYTES) return TL3_ERR_SCRATCH_LIMIT;
   void* scratch = nullptr;
   if (int rc = tl3::static_scratch_address(&scratch)) return rc;

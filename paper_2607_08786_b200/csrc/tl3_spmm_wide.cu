@@ -1,0 +1,631 @@
+// SpMM for more than 64 columns (a prompt, a wide batch), sm_100a: W is streamed and decoded once for
+// up to 256 columns.
+//
+// The pieces are those of tl3_spmm.cu (bulk copies of the packed blocks, Algorithm 1 by decode warps
+// into a second 2:4 operand W_r, tcgen05.mma.sp on W_t and W_r into one fp32 accumulator, split-K over
+// contiguous tile ranges with one reduction at the end), arranged for an accumulator of up to 256
+// columns:
+//   * the blocks and X have rings of their own: X arrives in slices of 64 k-values x n_pad columns
+//     (one TMA box when X is [batch, hidden], one per 64 columns when it is [hidden, batch]) that are
+//     given back half a tile at a time, so that shared memory holds more of the blocks;
+//   * one launch covers all columns: a row-tile is worked on once per group of n_pad columns, the
+//     groups of a row-tile directly after one another (its blocks then come from L2);
+//   * two accumulators while they fit tensor memory beside the metadata, else one.
+#include <cuda.h>
+#include <cuda_runtime.h>
+#include <cuda_fp16.h>
+
+#include <cstdint>
+#include <mutex>
+#include <vector>
+
+#include "tl3_device.cuh"
+#include "tl3_internal.h"
+
+namespace tl3 {
+namespace {
+
+constexpr int kGroups = 3;                // decode groups of four warps
+constexpr int kProducerWarp = 0;          // packed blocks
+constexpr int kMmaWarp = 1;
+constexpr int kClearWarp = 2;             // clears W_r; owns the tensor-memory allocation
+constexpr int kXWarp = 3;                 // X slices
+constexpr int kDecodeWarp0 = 4;
+constexpr int kEpilogueWarp0 = kDecodeWarp0 + 4 * kGroups;
+constexpr int kThreads = (kEpilogueWarp0 + 4) * 32;
+constexpr int kEpilogueBarrier = 1;
+constexpr int kMaxRing = 8;
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kColMetaT = 480;       // + 4 * (W_r buffer)
+constexpr uint32_t kColMetaR = 496;
+constexpr uint32_t kTurnPitch = 36;       // bytes per row of a warp's turning area (16 halves, odd number of words)
+constexpr uint32_t kTurnBytes = 32u * kTurnPitch;
+constexpr uint32_t kSlack = 1024u + 4u * kTurnBytes + 1024u;   // barriers, the epilogue warps' turning areas, alignment
+
+struct WideArgs {
+  const uint8_t* blob;
+  const DirEntry* dir;
+  uint32_t tiles, tiles_k, chunks;        // tiles of W, groups of n_pad columns
+  int M, N, n_pad;
+  long long ldy;
+  __half* Y;
+  const __half* bias;
+  int act;
+  float* partials;                        // [gridDim.x][n_pad][128]
+  unsigned int* flags;                    // [gridDim.x]
+  unsigned int* status;
+  uint32_t block_area, slice_bytes;       // multiples of 1024
+  int n_w, n_x, n_wr;                     // ring sizes: blocks (>= n_wr), X slices, W_r buffers
+  int n_acc;
+};
+
+// barriers, one 64-bit word each
+enum : uint32_t {
+  kBarFull = 0, kBarWFree = 8, kBarDec = 16, kBarXFull = 24, kBarXFree = 32, kBarWrReady = 40, kBarWrFree = 44,
+  kBarAccFull = 48, kBarReduce = 50, kBarAccEmpty = 51, kBarCount = 53, kTmemSlot = 53, kAbort = 54
+};
+
+// Bias and activation of 16 sums of one row.  One branch per 16 columns, the functions inlined: a
+// call per element (as in tl3_spmm.cu, where a small kernel image matters more) took 50 us of 181 on
+// 20480 x 5120, N = 512 with bias and ReLU.
+__device__ __forceinline__ void apply_epilogue(uint32_t (&v)[16], float bias, int act) {
+#pragma unroll
+  for (int c = 0; c < 16; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) + bias);
+  if (act == TL3_ACT_RELU) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] = __float_as_uint(fmaxf(__uint_as_float(v[c]), 0.f));
+  } else if (act != TL3_ACT_NONE) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) v[c] = __float_as_uint(finish(__uint_as_float(v[c]), 0.f, act));
+  }
+}
+
+// Columns c_begin, c_begin + c_step, ... (16 at a time) of one row of a row-tile: accumulator (+ the
+// partial sums of the n_others CTAs after this one, in ascending order whatever the order they came
+// in), bias, activation, rounding, Y.  Executed by whole warps, `et` is the row, 32 * (warp % 4) + lane.
+// `turn`: kTurnBytes of shared memory of the warp's own.  A thread holds a row, so rows of Y that
+// 16-byte stores do not fit are turned there first: stored by their rows' threads, two bytes each a
+// row pitch apart, they took 6 us of 25 on 4096 x 4096, N = 65.
+template <bool XT>
+__device__ __noinline__ void write_columns(const WideArgs& a, uint32_t acc_tmem, int et, uint32_t vrow, int c_begin, int c_step, int n_others, uint32_t turn) {
+  constexpr int CH = 16;
+  const int row = static_cast<int>(vrow / a.chunks) * kTileM + et;
+  const int n0 = static_cast<int>(vrow % a.chunks) * a.n_pad;
+  const int cols = a.N - n0 < a.n_pad ? a.N - n0 : a.n_pad;
+  const bool plain = a.bias == nullptr && a.act == TL3_ACT_NONE;
+  const float bias = a.bias != nullptr && row < a.M ? __half2float(__ldg(a.bias + row)) : 0.f;
+  const bool vec_ok = !XT && (a.ldy & 7) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0;
+  const size_t slot = static_cast<size_t>(a.n_pad) * 128;
+#pragma unroll 1
+  for (int c0 = c_begin; c0 < cols; c0 += c_step) {
+    uint32_t v[CH];
+    TmemLd<CH>::ld(acc_tmem + c0, v);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    const float* p = a.partials + slot * (blockIdx.x + 1) + c0 * 128 + et;
+    for (int k = 0; k < n_others; k += 2, p += 2 * slot) {         // two slots' loads in flight
+      float p0[CH], p1[CH];
+      const bool second = k + 1 < n_others;
+#pragma unroll
+      for (int c = 0; c < CH; ++c) { p0[c] = __ldcg(p + c * 128); p1[c] = second ? __ldcg(p + slot + c * 128) : 0.f; }
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        float x = __uint_as_float(v[c]) + p0[c];
+        if (second) x += p1[c];
+        v[c] = __float_as_uint(x);
+      }
+    }
+    if (!plain) apply_epilogue(v, bias, a.act);
+    if constexpr (XT) {
+      if (row >= a.M) continue;
+      __half* y = a.Y + static_cast<long long>(n0 + c0) * a.ldy + row;
+#pragma unroll
+      for (int c = 0; c < CH; ++c, y += a.ldy)
+        if (c0 + c < cols) *y = __float2half_rn(__uint_as_float(v[c]));
+    } else {
+      uint32_t o[CH / 2];
+#pragma unroll
+      for (int c = 0; c < CH / 2; ++c) {
+        const __half2 h = __floats2half2_rn(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]));
+        o[c] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      if (vec_ok && c0 + CH <= cols) {
+        if (row >= a.M) continue;
+        uint4* y = reinterpret_cast<uint4*>(a.Y + static_cast<long long>(row) * a.ldy + n0 + c0);
+        y[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        y[1] = make_uint4(o[4], o[5], o[6], o[7]);
+      } else {
+        const int lane = et & 31, col = lane & 15;
+        __syncwarp();
+#pragma unroll
+        for (int c = 0; c < CH / 2; ++c) sts_u32(turn + static_cast<uint32_t>(lane) * kTurnPitch + 4u * c, o[c]);
+        __syncwarp();
+        const int row0 = row - lane + (lane >> 4);                 // half a warp writes one row
+        __half* y = a.Y + static_cast<long long>(row0) * a.ldy + n0 + c0 + col;
+#pragma unroll 4
+        for (int i = 0; i < 16; ++i, y += 2 * a.ldy) {
+          const uint32_t h = lds_u16(turn + static_cast<uint32_t>(2 * i + (lane >> 4)) * kTurnPitch + 2u * col);
+          if (row0 + 2 * i < a.M && c0 + col < cols) *reinterpret_cast<uint16_t*>(y) = static_cast<uint16_t>(h);
+        }
+      }
+    }
+  }
+}
+
+// XT as in tl3_spmm.cu: activations and result transposed ([batch, hidden]).
+template <bool XT>
+__global__ void __launch_bounds__(kThreads, 1)
+tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ WideArgs a) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  const uint32_t w_base = smem_u32(smem);
+  const uint32_t x_base = w_base + static_cast<uint32_t>(a.n_w) * a.block_area;
+  const uint32_t wr_base = x_base + static_cast<uint32_t>(a.n_x) * a.slice_bytes;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (wr_base - w_base) + static_cast<uint32_t>(a.n_wr) * kWrBytes);
+  const uint32_t bar0 = smem_u32(bars);
+  auto bar = [&](uint32_t which, int i) -> uint32_t { return bar0 + 8u * (which + static_cast<uint32_t>(i)); };
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kTmemSlot);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + kAbort);
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // Tile v of the launch: row-tile v / tiles_k of tiles_m * chunks (row-tile major, column group
+  // minor), k-tile v % tiles_k.
+  const uint32_t T = a.tiles * a.chunks, G = gridDim.x, TK = a.tiles_k;
+  const uint32_t t_begin = range_begin(blockIdx.x, T, G), t_end = range_begin(blockIdx.x + 1, T, G);
+  const int n_tiles = static_cast<int>(t_end - t_begin);
+  const uint32_t kt_begin = t_begin % TK, vrow_begin = t_begin / TK;
+  const int AG = a.n_wr < kGroups ? a.n_wr : kGroups;   // decode groups in use: see the waits of the decode warps
+
+  if (warp == kProducerWarp) {
+    if (lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&x_map) : "memory");
+    for (int i = lane; i < static_cast<int>(kBarCount); i += 32) {
+      const uint32_t u = static_cast<uint32_t>(i);
+      const uint32_t count = (u >= kBarDec && u < kBarXFull) || u >= kBarAccEmpty ? 128u : (u >= kBarWrReady && u < kBarWrFree) ? 32u : 1u;
+      mbar_init(bar0 + 8u * u, count);
+    }
+    if (lane == 0) *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == kClearWarp) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  const WaitCtx wctx{abort_flag, a.status};
+  pdl_launch_dependents();
+
+  if (warp == kProducerWarp) {
+    // ------------------------------------------------------------------ packed blocks
+    // (never written by the kernel before this one: no wait for it)
+    int issued = 0, s = 0;
+    uint32_t ph = 0, kt = kt_begin, vrow = vrow_begin;
+    bool alive = true;
+    for (int base = 0; base < n_tiles && alive; base += 32) {
+      // directory entries of the next 32 tiles, one per lane
+      uint4 mine = make_uint4(0, 0, 0, 0);
+      if (base + lane < n_tiles) {
+        uint32_t k = kt + static_cast<uint32_t>(lane), v = vrow;
+        while (k >= TK) { k -= TK; ++v; }
+        mine = __ldg(reinterpret_cast<const uint4*>(a.dir + static_cast<size_t>(v / a.chunks) * TK + k));
+      }
+      const int cnt = n_tiles - base < 32 ? n_tiles - base : 32;
+      for (int j = 0; j < cnt; ++j) {
+        const uint32_t off16 = __shfl_sync(0xFFFFFFFFu, mine.x, j), bytes = __shfl_sync(0xFFFFFFFFu, mine.y, j);
+        if (base + j >= a.n_w) alive = __all_sync(0xFFFFFFFFu, mbar_wait(bar(kBarWFree, s), ph ^ 1u, wctx, kStProducer));
+        if (!alive) break;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(bar(kBarFull, s), bytes);
+          bulk_copy_g2s(w_base + static_cast<uint32_t>(s) * a.block_area, a.blob + static_cast<size_t>(off16) * 16, bytes, bar(kBarFull, s));
+        }
+        __syncwarp();
+        issued = base + j + 1;
+        if (++s == a.n_w) { s = 0; ph ^= 1u; }
+        if (++kt == TK) { kt = 0; ++vrow; }
+      }
+    }
+    if (lane == 0 && *abort_flag) {
+      // let the copies still in flight land before the CTA goes away
+      for (int i = issued > a.n_w ? issued - a.n_w : 0; i < issued; ++i) {
+        const unsigned long long t1 = global_timer();
+        while (!mbar_try_wait(bar(kBarFull, i % a.n_w), (i / a.n_w) & 1)) {
+          if (global_timer() - t1 > kWaitLimitNs / 4) { atomicCAS(a.status, 0u, (uint32_t)kStDrain); break; }
+        }
+      }
+    }
+  } else if (warp == kXWarp) {
+    // ------------------------------------------------------------------ X slices, two per tile
+    int issued = 0, s = 0;
+    uint32_t ph = 0, kt = kt_begin, vrow = vrow_begin;
+    bool alive = true;
+    pdl_wait();                                                   // the kernel before this one may have written X
+    for (int i = 0; i < n_tiles && alive; ++i) {
+      const int n0 = static_cast<int>(vrow % a.chunks) * a.n_pad;
+      for (int h = 0; h < 2; ++h) {
+        if (issued >= a.n_x) alive = __all_sync(0xFFFFFFFFu, mbar_wait(bar(kBarXFree, s), ph ^ 1u, wctx, kStProducer));
+        if (!alive) break;
+        if (elect_one()) {
+          const uint32_t full = bar(kBarXFull, s), dst = x_base + static_cast<uint32_t>(s) * a.slice_bytes;
+          const int k0 = static_cast<int>(kt) * kTileK + 64 * h;
+          mbar_arrive_expect_tx(full, a.slice_bytes);
+          if (XT) {
+            tma_load_2d(dst, &x_map, k0, n0, full);
+          } else {
+            for (uint32_t c = 0; c * 8192u < a.slice_bytes; ++c) tma_load_2d(dst + c * 8192u, &x_map, n0 + static_cast<int>(64u * c), k0, full);
+          }
+        }
+        __syncwarp();
+        ++issued;
+        if (++s == a.n_x) { s = 0; ph ^= 1u; }
+      }
+      if (++kt == TK) { kt = 0; ++vrow; }
+    }
+    if (lane == 0 && *abort_flag) {
+      for (int i = issued > a.n_x ? issued - a.n_x : 0; i < issued; ++i) {
+        const unsigned long long t1 = global_timer();
+        while (!mbar_try_wait(bar(kBarXFull, i % a.n_x), (i / a.n_x) & 1)) {
+          if (global_timer() - t1 > kWaitLimitNs / 4) { atomicCAS(a.status, 0u, (uint32_t)kStDrain); break; }
+        }
+      }
+    }
+  } else if (warp == kClearWarp) {
+    // ------------------------------------------------------------------ W_r clearing
+    int wb = 0, use = 0;
+    for (int i = 0; i < n_tiles; ++i) {
+      bool ok = true;
+      if (use >= 1) ok = mbar_wait(bar(kBarWrFree, wb), (use - 1) & 1, wctx, kStClearWrFree);
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
+      const uint32_t wr = wr_base + static_cast<uint32_t>(wb) * kWrBytes;
+#pragma unroll
+      for (int c = 0; c < 32; ++c) sts_zero16B(wr + (c * 32 + lane) * 16);
+      fence_proxy_async_smem();
+      mbar_arrive(bar(kBarWrReady, wb));
+      if (++wb == a.n_wr) { wb = 0; ++use; }
+    }
+  } else if (warp == kMmaWarp) {
+    // ------------------------------------------------------------------ MMA issuer
+    // Descriptors as in tl3_spmm.cu.  B: with XT n_pad rows x 128 bytes, K-major, 8-row groups 1024 B
+    // apart, a k-block is 64 bytes of a row; otherwise blocks of 64 k-rows x 128 bytes (64 columns),
+    // MN-major, 8-row groups 1024 B apart (stride field), the blocks 8192 B (leading-offset field), a
+    // k-block is 32 rows.
+    const uint32_t idesc = (1u << 2) | (1u << 4) | (XT ? 0u : (1u << 16)) | (static_cast<uint32_t>(a.n_pad >> 3) << 17) | (8u << 24);
+    constexpr uint32_t kHi = (1024u >> 4) | (1u << 14) | (2u << 29);
+    constexpr uint32_t kLboA = 1u << 16, kLboB = XT ? (1u << 16) : ((8192u >> 4) << 16);
+    constexpr uint32_t kBStep = (XT ? 64u : 4096u) >> 4;
+    int seg = 0, s = 0, sx = 0, wb = 0;
+    uint32_t ph = 0, phx = 0, kt = kt_begin;
+    for (int i = 0; i < n_tiles; ++i) {
+      const bool first_of_seg = (i == 0) || (kt == 0);
+      const bool last_of_seg = (i == n_tiles - 1) || (kt == TK - 1);
+      const int b = a.n_acc == 2 ? seg & 1 : 0, b_use = a.n_acc == 2 ? seg >> 1 : seg;
+      bool ok = true;
+      if (first_of_seg && b_use >= 1) ok = mbar_wait(bar(kBarAccEmpty, b), (b_use - 1) & 1, wctx, kStMmaAccEmpty);
+      ok = ok && mbar_wait(bar(kBarDec, s), ph, wctx, kStMmaDecoded);
+      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(b * a.n_pad);
+      const uint32_t e_t = tmem_base + kColMetaT + 4 * wb, e_r = tmem_base + kColMetaR;
+      const uint32_t a_lo = ((w_base + static_cast<uint32_t>(s) * a.block_area) >> 4) | kLboA;
+      const uint32_t r_lo = ((wr_base + static_cast<uint32_t>(wb) * kWrBytes) >> 4) | kLboA;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        ok = ok && mbar_wait(bar(kBarXFull, sx), phx, wctx, kStMmaX);
+        if (!__all_sync(0xFFFFFFFFu, ok)) break;
+        tc_fence_after();
+        const uint32_t b_lo = ((x_base + static_cast<uint32_t>(sx) * a.slice_bytes) >> 4) | kLboB;
+        const uint32_t xfree = bar(kBarXFree, sx), wfree = bar(kBarWFree, s), wrfree = bar(kBarWrFree, wb), acc = bar(kBarAccFull, b);
+        if (elect_one()) {
+#pragma unroll
+          for (int q = 0; q < 2; ++q) {
+            const uint32_t kb = 2u * h + q, id = idesc | static_cast<uint32_t>(q);
+            umma_sp_f16(d_tmem, a_lo + kb * 2u, kHi, b_lo + q * kBStep, kHi, e_t + 2u * h, id, (first_of_seg && kb == 0) ? 0u : 1u);
+            umma_sp_f16(d_tmem, r_lo + kb * 2u, kHi, b_lo + q * kBStep, kHi, e_r, id, 1u);
+          }
+          umma_commit(xfree);
+          if (h == 1) {
+            umma_commit(wfree);
+            umma_commit(wrfree);
+            if (last_of_seg) umma_commit(acc);
+          }
+        }
+        __syncwarp();
+        if (++sx == a.n_x) { sx = 0; phx ^= 1u; }
+      }
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
+      if (last_of_seg) ++seg;
+      if (++s == a.n_w) { s = 0; ph ^= 1u; }
+      if (++kt == TK) kt = 0;
+      if (++wb == a.n_wr) wb = 0;
+    }
+  } else if (warp >= kDecodeWarp0 && warp < kEpilogueWarp0) {
+    // ------------------------------------------------------------------ decode (Algorithm 1)
+    const int g = (warp - kDecodeWarp0) >> 2;
+    const int r = tid - (kDecodeWarp0 + 4 * g) * 32;            // chain / row / tensor-memory lane 0..127
+    const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    if (g == 0) {   // constant metadata of W_r: every window selects in-window positions {2, 3}
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};"
+                   ::"r"(tmem_base + lane_base + kColMetaR), "r"(0xEEEEEEEEu), "r"(0xEEEEEEEEu) : "memory");
+    }
+    // Tile i goes to group i % AG, W_r buffer i % n_wr, block stage i % n_w, AG <= n_wr <= n_w.  Parity
+    // waits cannot tell phases two apart; here they need not: when tile i is waited for, this group
+    // has finished tile i - AG, whose buffer was opened after that of tile i - n_wr (they open in
+    // order), so the buffer is at most one phase behind; and once it is open the MMAs of tile
+    // i - n_wr are done, so the stage's last user i - n_w has been loaded and consumed.
+    int wb = g, use = 0;
+    int s = g;
+    uint32_t ph = 0;
+    for (int i = g, j = 0; g < AG && i < n_tiles; i += AG, ++j) {
+      const int cr = (r + 32 * (j & 3)) & 127;                  // chain handled by this thread (lengths differ by warp: rotated)
+      const uint32_t wr = wr_base + static_cast<uint32_t>(wb) * kWrBytes;
+      bool ok = mbar_wait(bar(kBarWrReady, wb), use & 1, wctx, kStDecodeWrReady);
+      ok = ok && mbar_wait(bar(kBarFull, s), ph, wctx, kStDecodeFull);
+      const uint32_t stage = w_base + static_cast<uint32_t>(s) * a.block_area;
+      uint32_t m0 = 0, m1 = 0, m2 = 0, m3 = 0, n_words = 0, hdr = 0xFFFFFFFFu, pdd_len = 0, res_cnt = 0;
+      if (ok) {
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(m0), "=r"(m1), "=r"(m2), "=r"(m3) : "r"(stage + kMetaOff + r * 16));
+        n_words = lds_u32(stage + kInfoOff + 8);
+        hdr = lds_u32(stage + kHdrOff + cr * 4);
+        pdd_len = lds_u32(stage + kInfoOff);
+        res_cnt = lds_u32(stage + kInfoOff + 4);
+      }
+      if (!__all_sync(0xFFFFFFFFu, ok)) break;
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};"
+                   ::"r"(tmem_base + lane_base + kColMetaT + 4 * wb), "r"(m0), "r"(m1), "r"(m2), "r"(m3) : "memory");
+      uint32_t bad = 0;
+      const uint32_t room = a.block_area - kPddOff;             // bytes a block may use after its fixed part
+      const bool lens_ok = pdd_len <= room && res_cnt <= room / 4 && ((pdd_len + 3u) & ~3u) + 4u * res_cnt <= room &&
+                           n_words <= 3u && pdd_len == n_words * 512u;
+      if (lens_ok) decode_chain(stage, wr, hdr, stage + kPddOff + cr * 4, n_words, &bad);
+      else bad = 3u;
+      __syncwarp();
+      if (lens_ok) {                                              // Residual layer: (position, value) entries go to W_r too
+        const uint32_t res = stage + kPddOff + ((pdd_len + 3u) & ~3u);
+        for (uint32_t k = r; k < res_cnt; k += 128) {
+          const uint32_t rv = lds_u32(res + 4 * k);
+          if ((rv & 0xFFFFu) < 8192u) sts_u16(wr + swizzled_offset(rv & 0xFFFFu), rv >> 16);
+          else bad = 4u;
+        }
+      }
+      if (bad) atomicCAS(a.status, 0u, kStBadBlock | (bad << 8) | (static_cast<uint32_t>(i) << 12));
+      fence_proxy_async_smem();                                   // generic-proxy writes -> MMA reads
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      tc_fence_before();
+      mbar_arrive(bar(kBarDec, s));
+      s += AG;
+      while (s >= a.n_w) { s -= a.n_w; ph ^= 1u; }
+      wb += AG;
+      while (wb >= a.n_wr) { wb -= a.n_wr; ++use; }
+    }
+    // The last row-tile of this CTA's range, if other CTAs finish it: the decode warps, idle by now, read
+    // the partial sums together with the epilogue warps (an accumulator is as wide as 256 columns, and
+    // four warps alone had 16 us of loads in a row in front of them on 4096 x 4096, N = 128).
+    const uint32_t vrow = (t_end - 1) / TK;
+    if (vrow * TK >= t_begin && (vrow + 1) * TK > t_end && !*abort_flag) {
+      if (__all_sync(0xFFFFFFFFu, mbar_wait(bar(kBarReduce, 0), 0, wctx, kStEpilogueTail))) {
+        tc_fence_after();
+        __threadfence();
+        const int last_seg = static_cast<int>(vrow - vrow_begin);
+        const uint32_t acc = tmem_base + lane_base + static_cast<uint32_t>((a.n_acc == 2 ? last_seg & 1 : 0) * a.n_pad);
+        write_columns<XT>(a, acc, r, vrow, 16 * (g + 1), 16 * (kGroups + 1), owner_of((vrow + 1) * TK - 1, T, G) - static_cast<int>(blockIdx.x),
+                          wr_base + static_cast<uint32_t>(warp - kDecodeWarp0) * kTurnBytes);   // (the W_r buffers are idle too)
+      }
+    }
+  } else if (warp >= kEpilogueWarp0) {
+    // ------------------------------------------------------------------ epilogue
+    const int et = tid - kEpilogueWarp0 * 32;                    // row of the tile = tensor-memory lane
+    const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
+    int seg = 0;
+    uint32_t t = t_begin;
+    pdl_wait();   // Y, the partial sums and their flags may still be in use by the previous kernel
+    while (t < t_end) {
+      const uint32_t vrow = t / TK;
+      const uint32_t row_begin = vrow * TK, row_end = row_begin + TK;
+      const uint32_t seg_end = row_end < t_end ? row_end : t_end;
+      const bool complete = (t == row_begin) && (seg_end == row_end);
+      const int b = a.n_acc == 2 ? seg & 1 : 0, b_use = a.n_acc == 2 ? seg >> 1 : seg;
+      const int c_first = owner_of(row_begin, T, G), c_last = owner_of(row_end - 1, T, G);
+      // A shared row-tile is finished by the CTA that owns its first tile; for that CTA it is the last segment.
+      const bool reducer = !complete && static_cast<int>(blockIdx.x) == c_first;
+      const int n_others = c_last - c_first;
+      if (!named_bar_all(kEpilogueBarrier, 128, mbar_wait(bar(kBarAccFull, b), b_use & 1, wctx, kStEpilogueAccFull))) break;
+      tc_fence_after();
+      const uint32_t acc_tmem = tmem_base + lane_base + static_cast<uint32_t>(b * a.n_pad);
+      bool ready = true;
+      if (reducer) {
+        // The contributors (the CTAs after this one) store their partial sums and raise their flags;
+        // the sum runs in ascending CTA order, so the result does not depend on timing.  Every
+        // contributor holds an SM or gets one without waiting for this CTA; the wait is bounded.
+        bool ok = true;
+        if (et < 32) {
+          for (int base = 0; base < n_others && ok; base += 32) {
+            bool pending = base + et < n_others;
+            const int c_id = c_first + 1 + base + et;
+            unsigned long long t_slow = 0;
+            for (uint32_t it = 0; __any_sync(0xFFFFFFFFu, pending); ++it) {
+              if (pending) {
+                unsigned int up;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(up) : "l"(a.flags + c_id) : "memory");
+                if (up != 0u) {
+                  pending = false;
+                  a.flags[c_id] = 0u;                             // leave the workspace cleared
+                }
+              }
+              if ((it & 15u) == 15u) {
+                const unsigned long long now = global_timer();
+                if (t_slow == 0) t_slow = now;
+                const bool out = *abort_flag != 0 || now - t_slow > kWaitLimitNs;
+                if (__any_sync(0xFFFFFFFFu, out)) {
+                  if (et == 0) { atomicCAS(a.status, 0u, static_cast<uint32_t>(kStEpilogueFlags)); *abort_flag = 1; }
+                  ok = false;
+                  break;
+                }
+              }
+            }
+          }
+          __syncwarp();
+        }
+        if (et == 0 && ok) mbar_arrive(bar(kBarReduce, 0));       // the decode warps take part
+        ready = named_bar_all(kEpilogueBarrier, 128, ok);
+        __threadfence();                                          // the others' partial sums, after their flags
+      }
+      if (ready) {
+        if (complete || reducer) {
+          write_columns<XT>(a, acc_tmem, et, vrow, 0, reducer ? 16 * (kGroups + 1) : 16, reducer ? n_others : 0,
+                            bar0 + 1024u + static_cast<uint32_t>(warp & 3) * kTurnBytes);
+        } else {
+          float* mine = a.partials + static_cast<size_t>(a.n_pad) * 128 * blockIdx.x + et;
+#pragma unroll 1
+          for (int c0 = 0; c0 < a.n_pad; c0 += 16) {
+            uint32_t v[16];
+            TmemLd<16>::ld(acc_tmem + c0, v);
+            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+            for (int c = 0; c < 16; ++c) __stcg(mine + (c0 + c) * 128, __uint_as_float(v[c]));
+          }
+        }
+      }
+      tc_fence_before();
+      mbar_arrive(bar(kBarAccEmpty, b));
+      if (!complete && !reducer) {
+        __threadfence();                                          // the partial sums, before the flag
+        named_bar_sync(kEpilogueBarrier, 128);
+        if (et == 0) asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(a.flags + blockIdx.x), "r"(1u) : "memory");
+      }
+      ++seg;
+      t = seg_end;
+    }
+  }
+
+  // ------------------------------------------------------------------ teardown
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kClearWarp) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+  }
+}
+
+template <bool XT>
+int launch_wide(const CUtensorMap& map, const WideArgs& args, int grid, uint32_t smem_bytes, cudaStream_t stream) {
+  {
+    int dev = 0;
+    TL3_CUDA(cudaGetDevice(&dev));
+    static std::mutex mu;
+    static std::vector<char> configured;                          // per device, as in tl3_spmm.cu
+    std::lock_guard<std::mutex> lock(mu);
+    if (static_cast<size_t>(dev) >= configured.size()) configured.resize(dev + 1, 0);
+    if (!configured[dev]) {
+      TL3_CUDA(cudaFuncSetAttribute(tl3_spmm_wide_kernel<XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemLimit)));
+      configured[dev] = 1;
+    }
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = smem_bytes;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see pdl_wait() in the kernel
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_spmm_wide_kernel<XT>, map, args));
+  TL3_CUDA(cudaGetLastError());
+  return TL3_OK;
+}
+
+}  // namespace
+
+// Columns per pass.  More of them decode W less often, fewer give a small matrix more row-tiles to
+// share out and less to add up at the end.  The estimate of a launch, in us, from measured launches: a
+// tile costs 0.45 (its decode) + 0.0036 per column; the CTAs that share a row-tile hand over n_pad
+// columns each at 0.008 per column and CTA.  (1024 x 1024, N = 500: 23 us in 2 passes, 17 in 3, 13 in 4;
+// 20480 x 5120, N = 512: 125 in 2, 142 in 3, 160 in 4.)
+static int wide_columns(const tl3_matrix* m, int N, int sm_count) {
+  double best = 0;
+  int best_n = 0;
+  for (int passes = (N + 255) / 256; passes <= (N + 63) / 64; ++passes) {
+    const int n_pad = ((N + passes - 1) / passes + 15) / 16 * 16;
+    const double rows = static_cast<double>(m->tiles_m) * ((N + n_pad - 1) / n_pad);
+    const double per_cta = rows * m->tiles_k / sm_count;
+    const double ctas = per_cta < 1 ? static_cast<double>(m->tiles_k) : sm_count / rows;   // that share a row-tile
+    const double t = (per_cta < 1 ? 1.0 : per_cta) * (0.45 + 0.0036 * n_pad) + 0.008 * n_pad * (ctas > 1 ? ctas : 1.0);
+    if (best_n == 0 || t < best) { best = t; best_n = n_pad; }
+  }
+  return best_n;
+}
+
+int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t ldy, int N, const tl3_epilogue* ep, bool xt,
+              void* workspace, void* stream) {
+  if ((ldx & 7) != 0 || (reinterpret_cast<uintptr_t>(X) & 15) != 0 || (reinterpret_cast<uintptr_t>(Y) & 1) != 0 ||
+      (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
+    return TL3_ERR_INVALID_ARG;
+  DeviceInfo di;
+  if (int rc = device_info(&di)) return rc;
+  if (di.cc_major != 10) return TL3_ERR_UNSUPPORTED;
+
+  WideArgs a{};
+  a.n_pad = wide_columns(m, N, di.sm_count);
+  a.chunks = static_cast<uint32_t>((N + a.n_pad - 1) / a.n_pad);
+  a.block_area = (m->max_block_bytes + 1023u) / 1024u * 1024u;
+  a.slice_bytes = xt ? static_cast<uint32_t>(a.n_pad) * 128u : static_cast<uint32_t>((a.n_pad + 63) / 64) * 8192u;
+  a.n_acc = 2 * a.n_pad <= static_cast<int>(kColMetaT) ? 2 : 1;
+  {
+    // Three W_r buffers (one being cleared, one decoded into, one multiplied: 131 us against 122 with two
+    // on 20480 x 5120, N = 512), three X slices, at least as many blocks as W_r buffers; with large blocks
+    // less, down to two of each; with small ones what is left goes to blocks (five are enough), then to X.
+    const uint32_t room = kSmemLimit - kSlack;
+    auto blocks = [&]() -> int {
+      const uint32_t fixed = a.n_wr * kWrBytes + a.n_x * a.slice_bytes;
+      return fixed < room ? static_cast<int>((room - fixed) / a.block_area) : 0;
+    };
+    a.n_wr = 3; a.n_x = 3;
+    if (blocks() < a.n_wr) a.n_x = 2;
+    if (blocks() < a.n_wr) { a.n_wr = 2; a.n_x = 3; }
+    if (blocks() < a.n_wr) a.n_x = 2;
+    while (a.n_x < kMaxRing) {
+      ++a.n_x;
+      if (blocks() < 5) { --a.n_x; break; }
+    }
+    a.n_w = blocks();
+    if (a.n_w > kMaxRing) a.n_w = kMaxRing;
+    if (a.n_w < a.n_wr) return kWideNoPlan;
+  }
+  const uint32_t smem_bytes = a.n_w * a.block_area + a.n_x * a.slice_bytes + a.n_wr * kWrBytes + kSlack;
+
+  EncodeTiledFn encode = encode_tiled_fn();
+  if (!encode) return TL3_ERR_UNSUPPORTED;
+  CUtensorMap map;
+  // dims {N, K}, box {64 columns, 64 k}; transposed: dims {K, N}, box {64 k, n_pad rows}.  What lies beyond reads as zero.
+  const cuuint64_t dims[2] = {static_cast<cuuint64_t>(xt ? m->K : N), static_cast<cuuint64_t>(xt ? N : m->K)};
+  const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ldx) * 2};
+  const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(xt ? a.n_pad : 64)};
+  const cuuint32_t elem_strides[2] = {1, 1};
+  const CUresult cr = encode(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, elem_strides,
+                             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (cr != CUDA_SUCCESS) { set_cuda_error(static_cast<int>(cr)); return TL3_ERR_CUDA; }
+
+  const unsigned long long total = static_cast<unsigned long long>(m->n_tiles) * a.chunks;
+  const int grid = static_cast<int>(total < static_cast<unsigned long long>(di.sm_count) ? total : di.sm_count);
+  if (total * static_cast<unsigned long long>(grid + 1) >= (1ull << 32)) return kWideNoPlan;   // the kernel splits the tiles in 32-bit arithmetic
+  const WorkspaceLayout wl = workspace_layout(N, di.sm_count);
+  uint8_t* ws = static_cast<uint8_t*>(workspace);
+  a.blob = static_cast<const uint8_t*>(m->dptr);
+  a.dir = reinterpret_cast<const DirEntry*>(a.blob + m->dir_offset);
+  a.tiles = static_cast<uint32_t>(m->n_tiles);
+  a.tiles_k = static_cast<uint32_t>(m->tiles_k);
+  a.M = static_cast<int>(m->M);
+  a.N = N;
+  a.ldy = ldy;
+  a.Y = static_cast<__half*>(Y);
+  a.bias = ep ? static_cast<const __half*>(ep->bias) : nullptr;
+  a.act = ep ? ep->activation : TL3_ACT_NONE;
+  a.partials = reinterpret_cast<float*>(ws + wl.partials_off);
+  a.flags = reinterpret_cast<unsigned int*>(ws + wl.flags_off);
+  a.status = reinterpret_cast<unsigned int*>(ws + wl.status_off);
+  m->last_ctas = grid; m->last_stages = a.n_w; m->last_smem = static_cast<int>(smem_bytes);
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  return xt ? launch_wide<true>(map, a, grid, smem_bytes, st) : launch_wide<false>(map, a, grid, smem_bytes, st);
+}
+
+}  // namespace tl3

@@ -147,6 +147,11 @@ def _stream_ptr(stream) -> int:
     return int(getattr(stream, "cuda_stream", stream))
 
 
+def _scratch_class(N: int) -> int:
+    """The width whose workspace a product of N columns uses: sizes change at these."""
+    return 16 if N <= 16 else 32 if N <= 32 else 128 if N <= 128 else 256
+
+
 class Matrix:
     """Handle of one encoded weight matrix (``tl3_matrix``)."""
 
@@ -280,6 +285,10 @@ class Matrix:
         _check(lib().tl3_workspace_init(ws.data_ptr(), n, _stream_ptr(stream)), "tl3_workspace_init")
         return ws
 
+    def _too_small(self, workspace, N: int) -> bool:
+        """A workspace made for fewer columns: the product is then taken 64 columns at a time."""
+        return workspace.numel() * workspace.element_size() < self.workspace_bytes(N)
+
     def spmm(self, X, Y=None, workspace=None, stream=None, bias=None, activation=None):
         """``Y = W X`` on the GPU, or ``Y = act(W X + bias)`` when a bias (torch.float16, M entries, on
         the device) and / or an activation ("relu", "silu", "gelu_tanh") is given.
@@ -294,10 +303,14 @@ class Matrix:
         if Y is None:
             Y = torch.empty((M, N), dtype=torch.float16, device=X.device)
         if workspace is None:
-            key = 16 if N <= 16 else 32 if N <= 32 else 64        # wider blocks reuse the 64-column scratch
+            key = _scratch_class(N)
             workspace = self._workspaces.get(key)
             if workspace is None:
-                workspace = self._workspaces[key] = self.new_workspace(N, stream)
+                workspace = self._workspaces[key] = self.new_workspace(key, stream)
+        elif N > 128 and self._too_small(workspace, N):
+            for n in range(0, N, 64):
+                self.spmm(X[:, n:n + 64], Y[:, n:n + 64], workspace, stream, bias, activation)
+            return Y
         if bias is None and activation is None:
             _check(lib().tl3_spmm(self._h, X.data_ptr(), X.stride(0), Y.data_ptr(), Y.stride(0), N,
                                   workspace.data_ptr(), _stream_ptr(stream)), "tl3_spmm")
@@ -322,10 +335,14 @@ class Matrix:
         if Yt is None:
             Yt = torch.empty((N, M), dtype=torch.float16, device=Xt.device)
         if workspace is None:
-            key = 16 if N <= 16 else 32 if N <= 32 else 64
+            key = _scratch_class(N)
             workspace = self._workspaces.get(key)
             if workspace is None:
-                workspace = self._workspaces[key] = self.new_workspace(N, stream)
+                workspace = self._workspaces[key] = self.new_workspace(key, stream)
+        elif N > 128 and self._too_small(workspace, N):
+            for n in range(0, N, 64):
+                self.spmm_nt(Xt[n:n + 64], Yt[n:n + 64], workspace, stream, bias, activation)
+            return Yt
         if bias is not None and (bias.dtype != torch.float16 or bias.numel() != M or not bias.is_contiguous()):
             raise ValueError("bias must be a contiguous float16 tensor with one entry per row of W")
         ep = Epilogue(bias.data_ptr() if bias is not None else None, ACTIVATIONS[activation])
