@@ -112,7 +112,7 @@ int tl3_encode(const uint16_t* W, int64_t M, int64_t K, const tl3_params* params
  * (tl3_decode, tl3_upload, tl3_serialize ... work on it as on any other).
  *   dW: device, fp16 bits, row-major M x K, leading dimension ldw >= K, already masked.
  *   Tile 128 x 128, maxd 15 only.  The call allocates and frees device scratch of about the size
- *   of the container (cudaMalloc), runs on `stream` and waits for it.
+ *   of W (cudaMalloc), runs on `stream` and waits for it.
  * Errors: INVALID_ARG, UNSUPPORTED (more than 4 GiB of PDD bytes), CUDA, NO_MEMORY. */
 int tl3_encode_device(const void* dW, int64_t M, int64_t K, int64_t ldw, void* stream, tl3_matrix** out);
 /* The same conversion for a matrix that is only going to be multiplied: the container stays on the

@@ -456,12 +456,17 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
 
   int rc = TL3_OK;
   uint8_t* scratch = nullptr;               // everything the kernels write, in one allocation
-  uint8_t* var = nullptr;                   // PDD bytes and Residual entries (sized after the count pass)
+  uint8_t* extra = nullptr;                 // PDD bytes and Residual entries that do not fit it
   unsigned long long totals[2] = {0, 0}, stats[6] = {0, 0, 0, 0, 0, 0};
   // layout of `scratch` (every part 256-byte aligned)
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  // One allocation serves the whole conversion (cudaMalloc and cudaFree of more than 2 MB take 0.35 ms
+  // each, whatever the size: more than all kernels of a 5120 x 5120 matrix): the arrays of known size,
+  // the packer's scratch, and a guess at the PDD bytes and Residual entries that holds down to 40 %
+  // sparsity; only a matrix that needs more has them allocated when their sizes are known.
   const size_t o_vals = 0, o_meta = o_vals + up(n_vals * 2), o_tau = o_meta + up(n_meta), o_rho = o_tau + up(n_chain * 2),
-               o_len = o_rho + up(n_chain * 2), o_dir = o_len + up(n_chain), o_stats = o_dir + up(n_dir * 4), total = o_stats + 256;
+               o_len = o_rho + up(n_chain * 2), o_dir = o_len + up(n_chain), o_stats = o_dir + up(n_dir * 4), o_pack = o_stats + 256,
+               o_var = o_pack + up(pack_scratch_bytes(m->n_tiles)), guess = static_cast<size_t>(m->n_tiles) * 10240, total = o_var + guess;
   EncodeArgs a{};
   {
     TL3_ENC_CUDA(cudaMalloc(reinterpret_cast<void**>(&scratch), total));
@@ -485,7 +490,11 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
     TL3_ENC_CUDA(cudaStreamSynchronize(st));
     if (totals[0] > 0xFFFFFFFFull || totals[1] > 0xFFFFFFFFull) { rc = TL3_ERR_UNSUPPORTED; goto done; }   // 32-bit directory offsets
     const size_t o_res_rho = up(totals[0]), o_res_val = o_res_rho + up(totals[1] * 2), var_total = o_res_val + up(totals[1] * 2) + 256;
-    TL3_ENC_CUDA(cudaMalloc(reinterpret_cast<void**>(&var), var_total));
+    uint8_t* var = scratch + o_var;
+    if (var_total > guess) {
+      TL3_ENC_CUDA(cudaMalloc(reinterpret_cast<void**>(&extra), var_total));
+      var = extra;
+    }
     a.pdd_bytes = var;
     a.res_rho = reinterpret_cast<uint16_t*>(var + o_res_rho);
     a.res_val = reinterpret_cast<uint16_t*>(var + o_res_val);
@@ -499,13 +508,13 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
       m->n_res = static_cast<int64_t>(stats[3]); m->n_dummy = static_cast<int64_t>(stats[4]); m->n_slots_unused = static_cast<int64_t>(stats[5]);
       DeviceCanon* c = new (std::nothrow) DeviceCanon();
       if (!c) { rc = TL3_ERR_NO_MEMORY; goto done; }
-      *c = DeviceCanon{a.tc_vals, a.tc_meta, a.chain_tau0, a.chain_rho0, a.chain_len, a.pdd_bytes, a.tile_dir, a.res_rho, a.res_val, {scratch, var}};
+      *c = DeviceCanon{a.tc_vals, a.tc_meta, a.chain_tau0, a.chain_rho0, a.chain_len, a.pdd_bytes, a.tile_dir, a.res_rho, a.res_val, scratch + o_pack, {scratch, extra}};
       m->device_canon = c;
       m->release_device_canon = release_encoded;
       m->host_arrays = false;
       m->canon_bytes = static_cast<int64_t>(n_vals * 2 + n_meta + n_chain * 5 + n_dir * 4 + totals[0] + totals[1] * 4);
       scratch = nullptr;                                            // owned by the handle from here on
-      var = nullptr;
+      extra = nullptr;
       goto done;
     }
     try {
@@ -532,7 +541,7 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
   }
 done:
   if (scratch) cudaFree(scratch);
-  if (var) cudaFree(var);
+  if (extra) cudaFree(extra);
   if (rc == TL3_OK && keep_on_device) rc = tl3_plan_device(m, stream);   // sizes of the packed blocks: tl3_device_bytes() is valid on return
   if (rc != TL3_OK) { tl3_free(m); return rc; }
   *out = m;

@@ -67,8 +67,10 @@ namespace tl3 {
 struct DeviceCanon {
   const uint16_t* tc_vals; const uint8_t* tc_meta; const uint16_t* chain_tau0; const uint16_t* chain_rho0;
   const uint8_t* chain_len; const uint8_t* pdd_bytes; const uint32_t* tile_dir; const uint16_t* res_rho; const uint16_t* res_val;
+  void* pack_scratch;                        // pack_scratch_bytes(): sizes of the packed blocks, then their offsets
   void* alloc[2];                            // what to cudaFree
 };
+inline size_t pack_scratch_bytes(int64_t n_tiles) { return static_cast<size_t>(n_tiles + 1) * 12; }
 
 // ---- device blob layout ------------------------------------------------------------------
 // [0, 256)                 header (magic, shape; informational)
@@ -106,6 +108,7 @@ struct DirEntry {
 size_t plan_device_layout(const tl3_matrix* m);           // fills device_bytes, offsets, max block (once, thread-safe)
 void pack_device_blob(const tl3_matrix* m, uint8_t* out); // out: device_bytes bytes, host
 void set_device_layout(const tl3_matrix* m, const uint32_t* sizes);   // layout from per-tile sizes computed on the GPU
+// (block_off: one entry per tile, and the end of the last block)
 void blob_header_and_offsets(const tl3_matrix* m, uint8_t* header256, std::vector<unsigned long long>* block_off);
 
 void set_cuda_error(int e);

@@ -307,12 +307,13 @@ void blob_header_and_offsets(const tl3_matrix* m, uint8_t* header256, std::vecto
   struct { uint32_t magic, version; int64_t M, K, M_pad, K_pad, n_tiles; uint64_t dir_off, blocks_off; uint32_t max_block; } hdr{
       0x33334C54u, 2, m->M, m->K, m->M_pad, m->K_pad, m->n_tiles, m->dir_offset, m->blocks_offset, m->max_block_bytes};
   std::memcpy(header256, &hdr, sizeof(hdr));
-  block_off->resize(static_cast<size_t>(m->n_tiles));
+  block_off->resize(static_cast<size_t>(m->n_tiles) + 1);
   size_t off = m->blocks_offset;
   for (int64_t t = 0; t < m->n_tiles; ++t) {
     (*block_off)[t] = off;
     off += align_up(block_bytes(m->dev_sizes[2 * t], m->dev_sizes[2 * t + 1]), kBlockAlign);
   }
+  (*block_off)[static_cast<size_t>(m->n_tiles)] = off;
 }
 
 void pack_device_blob(const tl3_matrix* m, uint8_t* out) {

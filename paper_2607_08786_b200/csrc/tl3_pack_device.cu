@@ -390,16 +390,17 @@ int canon_to_device(tl3_matrix* m, cudaStream_t st, PackArgs* out) {
   size_t off[10];
   off[0] = 0;
   for (int i = 0; i < 9; ++i) off[i + 1] = off[i] + up(sz[i] + 16);
+  const size_t o_pack = off[9];
   if (!m->device_canon) {
     if (!m->host_arrays) return TL3_ERR_UNSUPPORTED;           // a device-only handle whose container has been packed and released
     void* p = nullptr;
-    TL3_PK_CUDA(cudaMalloc(&p, off[9]));
+    TL3_PK_CUDA(cudaMalloc(&p, o_pack + pack_scratch_bytes(m->n_tiles)));
     DeviceCanon* c = new (std::nothrow) DeviceCanon();
     if (!c) { cudaFree(p); return TL3_ERR_NO_MEMORY; }
     uint8_t* b = static_cast<uint8_t*>(p);
     *c = DeviceCanon{reinterpret_cast<const uint16_t*>(b + off[0]), b + off[1], reinterpret_cast<const uint16_t*>(b + off[2]),
                      reinterpret_cast<const uint16_t*>(b + off[3]), b + off[4], b + off[5], reinterpret_cast<const uint32_t*>(b + off[6]),
-                     reinterpret_cast<const uint16_t*>(b + off[7]), reinterpret_cast<const uint16_t*>(b + off[8]), {p, nullptr}};
+                     reinterpret_cast<const uint16_t*>(b + off[7]), reinterpret_cast<const uint16_t*>(b + off[8]), b + o_pack, {p, nullptr}};
     m->device_canon = c;
     m->release_device_canon = release_canon;
     for (int i = 0; i < 9; ++i)
@@ -444,18 +445,15 @@ extern "C" int tl3_plan_device(tl3_matrix* m, void* stream) {
   if (int rc = configure_pack_kernel()) return rc;
   PackArgs a{};
   if (int rc = canon_to_device(m, st, &a)) return rc;
-  uint32_t* d_sizes = nullptr;
-  TL3_PK_CUDA(cudaMalloc(reinterpret_cast<void**>(&d_sizes), static_cast<size_t>(m->n_tiles) * 12));
-  a.sizes = d_sizes;
+  a.sizes = static_cast<uint32_t*>(static_cast<DeviceCanon*>(m->device_canon)->pack_scratch);
   a.emit = 0;
   tl3_pack_kernel<<<static_cast<unsigned>(m->n_tiles), kPackThreads, sizeof(PackSmem), st>>>(a);
   std::vector<uint32_t> sizes;
   int rc = TL3_OK;
   try { sizes.resize(static_cast<size_t>(m->n_tiles) * 3); } catch (const std::bad_alloc&) { rc = TL3_ERR_NO_MEMORY; }
   cudaError_t e = cudaGetLastError();
-  if (rc == TL3_OK && e == cudaSuccess) e = cudaMemcpyAsync(sizes.data(), d_sizes, sizes.size() * 4, cudaMemcpyDeviceToHost, st);
+  if (rc == TL3_OK && e == cudaSuccess) e = cudaMemcpyAsync(sizes.data(), a.sizes, sizes.size() * 4, cudaMemcpyDeviceToHost, st);
   if (rc == TL3_OK && e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFree(d_sizes);
   if (rc != TL3_OK) return rc;
   if (e != cudaSuccess) { set_cuda_error(static_cast<int>(e)); return TL3_ERR_CUDA; }
   set_device_layout(m, sizes.data());
@@ -474,10 +472,13 @@ extern "C" int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream) {
   uint8_t header[256];
   std::vector<unsigned long long> block_off;
   try { blob_header_and_offsets(m, header, &block_off); } catch (const std::bad_alloc&) { return TL3_ERR_NO_MEMORY; }
-  unsigned long long* d_off = nullptr;
-  TL3_PK_CUDA(cudaMalloc(reinterpret_cast<void**>(&d_off), block_off.size() * 8));
+  unsigned long long* d_off = static_cast<unsigned long long*>(static_cast<DeviceCanon*>(m->device_canon)->pack_scratch);
   cudaError_t e = cudaMemcpyAsync(d_off, block_off.data(), block_off.size() * 8, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dptr, 0, m->device_bytes, st);
+  // zeros where no block is: before the first and behind the last (a block's padding is the kernel's)
+  const size_t blocks_end = block_off.back();
+  if (e == cudaSuccess) e = cudaMemsetAsync(dptr, 0, m->blocks_offset, st);
+  if (e == cudaSuccess && blocks_end < m->device_bytes)
+    e = cudaMemsetAsync(static_cast<uint8_t*>(dptr) + blocks_end, 0, m->device_bytes - blocks_end, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(dptr, header, 256, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
     a.blob = static_cast<uint8_t*>(dptr);
@@ -488,7 +489,6 @@ extern "C" int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream) {
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);          // header, offsets and the canonical copies are released below
-  cudaFree(d_off);
   if (m->device_canon) { release_canon(m->device_canon); m->device_canon = nullptr; }
   if (e != cudaSuccess) { set_cuda_error(static_cast<int>(e)); return TL3_ERR_CUDA; }
   m->dptr = dptr;
