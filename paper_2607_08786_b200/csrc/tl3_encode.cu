@@ -523,6 +523,8 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
       m->tile_dir.resize(n_dir);
       m->pdd_bytes.resize(totals[0]); m->res_rho.resize(totals[1]); m->res_val.resize(totals[1]);
     } catch (const std::bad_alloc&) { rc = TL3_ERR_NO_MEMORY; goto done; }
+    prefault(m->tc_vals.data(), n_vals * 2);                       // while the kernel runs
+    prefault(m->tc_meta.data(), n_meta);
     TL3_ENC_CUDA(cudaMemcpyAsync(m->tc_vals.data(), a.tc_vals, n_vals * 2, cudaMemcpyDeviceToHost, st));
     TL3_ENC_CUDA(cudaMemcpyAsync(m->tc_meta.data(), a.tc_meta, n_meta, cudaMemcpyDeviceToHost, st));
     TL3_ENC_CUDA(cudaMemcpyAsync(m->chain_tau0.data(), a.chain_tau0, n_chain * 2, cudaMemcpyDeviceToHost, st));

@@ -1,12 +1,54 @@
 // Internal definitions shared by the host-side and CUDA-side translation units of libtl3.
 #pragma once
+#include <sys/mman.h>
+
 #include <atomic>
 #include <cstdint>
 #include <cstddef>
+#include <cstdlib>
 #include <mutex>
+#include <new>
+#include <utility>
 #include <vector>
 
 #include "tl3.h"
+
+namespace tl3 {
+
+// Memory of the container's arrays: not cleared (every byte is written after a resize), and large
+// arrays on huge pages.  A first copy into 132 MB of fresh memory takes one thread 62 ms on 4 KB pages
+// and 28 ms on huge ones; eight threads 8.5 and 4.4 ms.
+template <class T> struct RawAllocator {
+  using value_type = T;
+  static constexpr size_t kHuge = size_t{2} << 20;
+  RawAllocator() = default;
+  template <class U> RawAllocator(const RawAllocator<U>&) {}
+  T* allocate(size_t n) {
+    if (n > (static_cast<size_t>(-1) - kHuge) / sizeof(T)) throw std::bad_alloc();
+    const size_t bytes = n * sizeof(T);
+    void* p;
+    if (bytes >= 2 * kHuge) {
+      p = std::aligned_alloc(kHuge, (bytes + kHuge - 1) / kHuge * kHuge);
+      if (p) madvise(p, bytes, MADV_HUGEPAGE);                      // (advice: a refusal costs time only)
+    } else {
+      p = std::malloc(bytes ? bytes : 1);
+    }
+    if (!p) throw std::bad_alloc();
+    return static_cast<T*>(p);
+  }
+  void deallocate(T* p, size_t) { std::free(p); }
+  template <class U> void construct(U* p) { ::new (static_cast<void*>(p)) U; }
+  template <class U, class... A> void construct(U* p, A&&... a) { ::new (static_cast<void*>(p)) U(std::forward<A>(a)...); }
+  template <class U> bool operator==(const RawAllocator<U>&) const { return true; }
+  template <class U> bool operator!=(const RawAllocator<U>&) const { return false; }
+};
+template <class T> using raw_vector = std::vector<T, RawAllocator<T>>;
+
+// Large copies and first touches of fresh memory, shared out over up to eight threads (tl3_host.cpp).
+void parallel_copy(void* dst, const void* src, size_t bytes);
+void prefault(void* p, size_t bytes);                        // fresh memory that a copy engine is about to fill
+
+}  // namespace tl3
 
 struct tl3_matrix {
   int64_t M = 0, K = 0, M_pad = 0, K_pad = 0;
@@ -14,13 +56,13 @@ struct tl3_matrix {
   tl3_params p{128, 128, 15};
 
   // canonical container (Sec. 3.2)
-  std::vector<uint16_t> tc_vals;
-  std::vector<uint8_t> tc_meta;
-  std::vector<uint16_t> chain_tau0, chain_rho0;
-  std::vector<uint8_t> chain_len;
-  std::vector<uint8_t> pdd_bytes;
-  std::vector<uint32_t> tile_dir;      // 4 per tile: pdd_off, pdd_len, res_off, res_cnt
-  std::vector<uint16_t> res_rho, res_val;
+  tl3::raw_vector<uint16_t> tc_vals;
+  tl3::raw_vector<uint8_t> tc_meta;
+  tl3::raw_vector<uint16_t> chain_tau0, chain_rho0;
+  tl3::raw_vector<uint8_t> chain_len;
+  tl3::raw_vector<uint8_t> pdd_bytes;
+  tl3::raw_vector<uint32_t> tile_dir;      // 4 per tile: pdd_off, pdd_len, res_off, res_cnt
+  tl3::raw_vector<uint16_t> res_rho, res_val;
 
   // layer statistics
   int64_t nnz = 0, n_tc = 0, n_sf = 0, n_res = 0, n_dummy = 0, n_slots_unused = 0;

@@ -17,9 +17,13 @@
 // banks, the two passes took 181 + 247 us on 5120 x 5120 at 50 % sparsity; now 57 + 77 us.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <cstdint>
 #include <cstring>
+#include <mutex>
 #include <new>
+#include <thread>
 #include <vector>
 
 #include "tl3_internal.h"
@@ -379,6 +383,81 @@ void release_canon(void* p) {
     }                                                         \
   } while (0)
 
+struct HostPiece {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+
+// Pageable host memory to the device, complete on return.  The runtime's own copy moves 11 GB/s, one
+// thread of its filling one staging buffer; here six threads fill a pinned megabyte each (6 MB kept for
+// the life of the process: pinning it costs more than a copy of 100 MB; one caller at a time uses it,
+// another one that comes meanwhile takes the runtime's way).  132 MB: 12.2 -> 5 ms.
+cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st) {
+  constexpr int kSlots = 6;
+  constexpr size_t kSlotBytes = size_t{1} << 20;
+  static std::mutex mu;
+  static uint8_t* ring = nullptr;
+  size_t total = 0;
+  for (const HostPiece& p : arrays) total += p.bytes;
+  std::unique_lock<std::mutex> lock(mu, std::defer_lock);
+  cudaStream_t own = nullptr;
+  int dev = 0;
+  bool staged = total >= (size_t{8} << 20) && lock.try_lock() && cudaGetDevice(&dev) == cudaSuccess;
+  if (staged && !ring && cudaHostAlloc(reinterpret_cast<void**>(&ring), kSlots * kSlotBytes, cudaHostAllocPortable) != cudaSuccess) {
+    ring = nullptr;
+    staged = false;
+    cudaGetLastError();
+  }
+  // (a stream of its own: the caller's may be one that means another stream in another thread)
+  if (staged && cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) != cudaSuccess) { staged = false; cudaGetLastError(); }
+  if (!staged) {
+    for (const HostPiece& p : arrays) {
+      if (!p.bytes) continue;
+      if (cudaError_t e = cudaMemcpyAsync(p.dst, p.src, p.bytes, cudaMemcpyHostToDevice, st)) return e;
+    }
+    return cudaStreamSynchronize(st);
+  }
+  std::vector<HostPiece> pieces;
+  std::vector<std::thread> pool;
+  std::atomic<size_t> next{0};
+  std::atomic<int> failed{cudaSuccess};
+  auto worker = [&](int slot) {
+    uint8_t* buf = ring + static_cast<size_t>(slot) * kSlotBytes;
+    cudaEvent_t done = nullptr;
+    cudaError_t e = cudaSetDevice(dev);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+    bool busy = false;
+    while (e == cudaSuccess && failed.load(std::memory_order_relaxed) == cudaSuccess) {
+      const size_t i = next.fetch_add(1);
+      if (i >= pieces.size()) break;
+      if (busy) e = cudaEventSynchronize(done);
+      if (e != cudaSuccess) break;
+      std::memcpy(buf, pieces[i].src, pieces[i].bytes);
+      e = cudaMemcpyAsync(pieces[i].dst, buf, pieces[i].bytes, cudaMemcpyHostToDevice, own);
+      if (e == cudaSuccess) e = cudaEventRecord(done, own);
+      busy = true;
+    }
+    if (done) cudaEventDestroy(done);
+    if (e != cudaSuccess) failed.store(e, std::memory_order_relaxed);
+  };
+  bool listed = false;
+  try {
+    for (const HostPiece& p : arrays)
+      for (size_t at = 0; at < p.bytes; at += kSlotBytes)
+        pieces.push_back({static_cast<uint8_t*>(p.dst) + at, static_cast<const uint8_t*>(p.src) + at, std::min(kSlotBytes, p.bytes - at)});
+    listed = true;
+    for (int t = 1; t < kSlots; ++t) pool.emplace_back(worker, t);
+  } catch (const std::exception&) {                              // fewer threads, or no list at all
+  }
+  if (!listed) failed.store(cudaErrorMemoryAllocation);
+  worker(0);
+  for (auto& th : pool) th.join();
+  const cudaError_t e = cudaStreamSynchronize(own);              // the ring is free again, whatever happened
+  cudaStreamDestroy(own);
+  return failed.load() != cudaSuccess ? static_cast<cudaError_t>(failed.load()) : e;
+}
+
 // Copies the canonical arrays of the handle to the device (one allocation, kept in the handle) and
 // fills the kernel arguments that point into it.
 int canon_to_device(tl3_matrix* m, cudaStream_t st, PackArgs* out) {
@@ -403,8 +482,19 @@ int canon_to_device(tl3_matrix* m, cudaStream_t st, PackArgs* out) {
                      reinterpret_cast<const uint16_t*>(b + off[7]), reinterpret_cast<const uint16_t*>(b + off[8]), b + o_pack, {p, nullptr}};
     m->device_canon = c;
     m->release_device_canon = release_canon;
-    for (int i = 0; i < 9; ++i)
-      if (sz[i]) TL3_PK_CUDA(cudaMemcpyAsync(b + off[i], src[i], sz[i], cudaMemcpyHostToDevice, st));
+    std::vector<HostPiece> arrays;
+    cudaError_t e = cudaErrorMemoryAllocation;
+    try {
+      for (int i = 0; i < 9; ++i) arrays.push_back({b + off[i], src[i], sz[i]});
+      e = copy_from_host(arrays, st);
+    } catch (const std::bad_alloc&) {
+    }
+    if (e != cudaSuccess) {                                        // nothing half-copied stays with the handle
+      m->device_canon = nullptr;
+      release_canon(c);
+      set_cuda_error(static_cast<int>(e));
+      return TL3_ERR_CUDA;
+    }
   }
   const DeviceCanon* c = static_cast<const DeviceCanon*>(m->device_canon);
   PackArgs a{};

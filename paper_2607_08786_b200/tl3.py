@@ -140,9 +140,28 @@ def _u16(a) -> np.ndarray:
     return np.ascontiguousarray(a)
 
 
+_new_bytes = ctypes.PYFUNCTYPE(ctypes.py_object, ctypes.c_char_p, ctypes.c_ssize_t)(("PyBytes_FromStringAndSize", ctypes.pythonapi))
+
+_torch = None
+_raw_stream = _device = None       # torch's C entries behind torch.cuda.current_stream(), where it has them
+
+
+def _torch_module():
+    """torch, imported when a call needs it (an import statement in every call costs a third of a microsecond)."""
+    global _torch, _raw_stream, _device
+    if _torch is None:
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        _device = getattr(torch._C, "_cuda_getDevice", None)
+        _torch = torch
+    return _torch
+
+
 def _stream_ptr(stream) -> int:
     if stream is None:
-        import torch
+        torch = _torch_module()
+        if _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device())          # 0.3 us; the Stream object of the line below costs 3
         return torch.cuda.current_stream().cuda_stream
     return int(getattr(stream, "cuda_stream", stream))
 
@@ -155,8 +174,9 @@ def _scratch_class(N: int) -> int:
 class Matrix:
     """Handle of one encoded weight matrix (``tl3_matrix``)."""
 
-    def __init__(self, handle: int):
+    def __init__(self, handle: int, shape=None):
         self._h = ctypes.c_void_p(handle)
+        self._shape = shape        # fixed for the life of a handle
         self._blob = None          # torch.uint8 tensor holding the device blob
         self._workspaces = {}
 
@@ -170,7 +190,7 @@ class Matrix:
         p = Params(tile_m, tile_k, maxd)
         _check(lib().tl3_encode(W.ctypes.data, W.shape[0], W.shape[1], ctypes.byref(p), ctypes.byref(h)),
                "tl3_encode")
-        return cls(h.value)
+        return cls(h.value, W.shape)
 
     @classmethod
     def encode_on_device(cls, W, stream=None, device_only: bool = False) -> "Matrix":
@@ -182,13 +202,18 @@ class Matrix:
         h = ctypes.c_void_p()
         fn = lib().tl3_encode_device_only if device_only else lib().tl3_encode_device
         _check(fn(W.data_ptr(), W.shape[0], W.shape[1], W.stride(0), _stream_ptr(stream), ctypes.byref(h)), "tl3_encode_device")
-        return cls(h.value)
+        return cls(h.value, (W.shape[0], W.shape[1]))
 
     @classmethod
     def deserialize(cls, data: bytes) -> "Matrix":
         h = ctypes.c_void_p()
-        buf = (ctypes.c_char * len(data)).from_buffer_copy(data)
-        _check(lib().tl3_deserialize(ctypes.addressof(buf), len(data), ctypes.byref(h)), "tl3_deserialize")
+        try:
+            buf = np.frombuffer(data, dtype=np.uint8)              # the library copies what it keeps
+            address = buf.ctypes.data
+        except (TypeError, ValueError):
+            buf = (ctypes.c_char * len(data)).from_buffer_copy(data)
+            address = ctypes.addressof(buf)
+        _check(lib().tl3_deserialize(address, len(data), ctypes.byref(h)), "tl3_deserialize")
         return cls(h.value)
 
     def close(self) -> None:
@@ -212,8 +237,10 @@ class Matrix:
 
     @property
     def shape(self):
-        s = self.stats()
-        return s["M"], s["K"]
+        if self._shape is None:
+            s = self.stats()
+            self._shape = (s["M"], s["K"])
+        return self._shape
 
     def decode(self) -> np.ndarray:
         M, K = self.shape
@@ -236,9 +263,10 @@ class Matrix:
         fn = lib().tl3_serialize_compact if compact else lib().tl3_serialize
         n = ctypes.c_size_t()
         _check(fn(self._h, None, ctypes.byref(n)), "tl3_serialize")
-        buf = ctypes.create_string_buffer(n.value)
-        _check(fn(self._h, buf, ctypes.byref(n)), "tl3_serialize")
-        return buf.raw[:n.value]
+        # the library writes into the bytes object itself
+        data = _new_bytes(None, n.value)
+        _check(fn(self._h, ctypes.cast(ctypes.c_char_p(data), ctypes.c_void_p), ctypes.byref(n)), "tl3_serialize")
+        return data[:n.value]
 
     # -- device side -------------------------------------------------------------------------
     def device_bytes(self) -> int:
@@ -293,12 +321,12 @@ class Matrix:
         """``Y = W X`` on the GPU, or ``Y = act(W X + bias)`` when a bias (torch.float16, M entries, on
         the device) and / or an activation ("relu", "silu", "gelu_tanh") is given.
         X: torch.float16 (K x N, last dim contiguous) on the device."""
-        import torch
+        torch = _torch_module()
         if X.dtype != torch.float16 or X.dim() != 2 or X.stride(1) != 1:
             raise ValueError("X must be a 2-D float16 tensor with contiguous rows")
         M, K = self.shape
-        N = X.shape[1]
-        if X.shape[0] != K:
+        rows, N = X.shape
+        if rows != K:
             raise ValueError("X has the wrong number of rows")
         if Y is None:
             Y = torch.empty((M, N), dtype=torch.float16, device=X.device)
@@ -325,12 +353,12 @@ class Matrix:
     def spmm_nt(self, Xt, Yt=None, workspace=None, stream=None, bias=None, activation=None):
         """``Yt = Xt W^T`` (+ bias, activation): activations in the [batch, hidden] layout.
         Xt: torch.float16 (N x K, last dim contiguous) on the device; Yt: N x M."""
-        import torch
+        torch = _torch_module()
         if Xt.dtype != torch.float16 or Xt.dim() != 2 or Xt.stride(1) != 1:
             raise ValueError("Xt must be a 2-D float16 tensor with contiguous rows")
         M, K = self.shape
-        N = Xt.shape[0]
-        if Xt.shape[1] != K:
+        N, columns = Xt.shape
+        if columns != K:
             raise ValueError("Xt has the wrong number of columns")
         if Yt is None:
             Yt = torch.empty((N, M), dtype=torch.float16, device=Xt.device)
@@ -345,8 +373,10 @@ class Matrix:
             return Yt
         if bias is not None and (bias.dtype != torch.float16 or bias.numel() != M or not bias.is_contiguous()):
             raise ValueError("bias must be a contiguous float16 tensor with one entry per row of W")
-        ep = Epilogue(bias.data_ptr() if bias is not None else None, ACTIVATIONS[activation])
-        _check(lib().tl3_spmm_nt(self._h, Xt.data_ptr(), Xt.stride(0), Yt.data_ptr(), Yt.stride(0), N, ctypes.byref(ep),
+        ep = None
+        if bias is not None or activation is not None:
+            ep = ctypes.byref(Epilogue(bias.data_ptr() if bias is not None else None, ACTIVATIONS[activation]))
+        _check(lib().tl3_spmm_nt(self._h, Xt.data_ptr(), Xt.stride(0), Yt.data_ptr(), Yt.stride(0), N, ep,
                                  workspace.data_ptr(), _stream_ptr(stream)), "tl3_spmm_nt")
         return Yt
 
