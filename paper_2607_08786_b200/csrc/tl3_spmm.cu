@@ -666,6 +666,56 @@ WorkspaceLayout workspace_layout(int N, int sm_count) {
   return w;
 }
 
+// X with N columns, N no multiple of eight, from pinned host memory to rows of ldx elements: a thread
+// reads 16 bytes over PCIe and stores eight elements.  The copy engine moves such rows of a few bytes
+// one by one (a product with X and Y on the host, 5001 x 3003, N = 5: 95 us, with this kernel 39; 8000 x
+// 7000, N = 33: 464 and 73).
+__global__ void __launch_bounds__(256)
+tl3_spread_rows_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst, long long total, unsigned int N, long long ldx) {
+  pdl_launch_dependents();                                         // (the product's CTAs may start; they wait before they read X)
+  const long long e0 = (static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) * 8;
+  if (e0 >= total) return;
+  uint16_t v[8];
+  const int n = total - e0 < 8 ? static_cast<int>(total - e0) : 8;
+  if (n == 8) {
+    *reinterpret_cast<uint4*>(v) = *reinterpret_cast<const uint4*>(src + e0);
+  } else {
+    for (int i = 0; i < n; ++i) v[i] = src[e0 + i];
+  }
+  long long row = e0 / N;
+  unsigned int col = static_cast<unsigned int>(e0 - row * N);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    if (i < n) dst[row * ldx + col] = v[i];
+    if (++col == N) { col = 0; ++row; }
+  }
+}
+
+// The address under which kernels read [p, p + bytes), if all of it lies in one pinned allocation (or
+// registration) and on 16 bytes; else null.
+static const void* pinned_address(const void* p, size_t bytes) {
+  typedef CUresult (*AttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
+  static AttributesFn fn = []() -> AttributesFn {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+      return nullptr;
+    return reinterpret_cast<AttributesFn>(f);
+  }();
+  if (!fn) return nullptr;
+  unsigned int type = 0, managed = 0;
+  CUdeviceptr dev = 0, start = 0;
+  size_t size = 0;
+  CUpointer_attribute which[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void* out[5] = {&type, &managed, &dev, &start, &size};
+  if (fn(5, which, out, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return nullptr;
+  if (type != CU_MEMORYTYPE_HOST || managed || !dev || (dev & 15) != 0) return nullptr;
+  if (dev != reinterpret_cast<CUdeviceptr>(p)) return nullptr;     // (a mapping at another address: the range is not in its terms)
+  if (dev < start || bytes > size || dev - start > size - bytes) return nullptr;
+  return reinterpret_cast<const void*>(dev);
+}
+
 // Process-wide launch tuning (tl3_set_tuning); the default is what measured best on B200.
 static std::atomic<int> g_decode_before_x{TL3_DEFAULT_DECODE_BEFORE_X};
 
@@ -914,8 +964,14 @@ int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // device copy of X with a leading dimension that satisfies the 16-byte rule
   const int64_t ldx = (N + 7) / 8 * 8;
+  const size_t x_bytes = static_cast<size_t>(m->K) * N * 2;
   if (ldx == N) {
-    TL3_CUDA(cudaMemcpyAsync(dX, X, static_cast<size_t>(m->K) * N * 2, cudaMemcpyHostToDevice, st));
+    TL3_CUDA(cudaMemcpyAsync(dX, X, x_bytes, cudaMemcpyHostToDevice, st));
+  } else if (const void* src = tl3::pinned_address(X, x_bytes)) {
+    const long long total = m->K * N;
+    tl3::tl3_spread_rows_kernel<<<static_cast<unsigned>((total + 2047) / 2048), 256, 0, st>>>(static_cast<const uint16_t*>(src), static_cast<uint16_t*>(dX),
+                                                                                            total, static_cast<unsigned>(N), ldx);
+    TL3_CUDA(cudaGetLastError());
   } else {
     TL3_CUDA(cudaMemcpy2DAsync(dX, static_cast<size_t>(ldx) * 2, X, static_cast<size_t>(N) * 2, static_cast<size_t>(N) * 2,
                                static_cast<size_t>(m->K), cudaMemcpyHostToDevice, st));
