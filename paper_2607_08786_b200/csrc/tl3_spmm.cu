@@ -661,7 +661,7 @@ WorkspaceLayout workspace_layout(int N, int sm_count) {
   WorkspaceLayout w;
   w.partials_off = (256 + static_cast<size_t>(2) * sm_count * 4 + 4095) / 4096 * 4096;
   int columns = 2 * n_pad_of(N);
-  if (N > 128) columns = N < kWideColumns ? (N + 15) / 16 * 16 : kWideColumns;
+  if (N > 128) columns = N < kWideColumns ? (N + 31) / 32 * 32 : kWideColumns;
   w.total = w.partials_off + static_cast<size_t>(columns) * sm_count * 128 * sizeof(float);
   return w;
 }
