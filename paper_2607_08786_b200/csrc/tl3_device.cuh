@@ -23,6 +23,8 @@ namespace tl3 {
 
 constexpr uint32_t kWrBytes = 16384;      // one W_r buffer
 constexpr uint32_t kSmemLimit = 232448;   // 227 KB
+constexpr uint32_t kTurnPitch = 36;       // bytes per row of a warp's turning area (16 halves, odd number of words)
+constexpr uint32_t kTurnBytes = 32u * kTurnPitch;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s without progress, per wait
 #ifndef TL3_TRYWAIT_HINT_NS
 #define TL3_TRYWAIT_HINT_NS 20000u

@@ -76,6 +76,7 @@ struct KernelArgs {
   uint32_t x_offset;         // offset of the X tile inside a stage, multiple of 1024
   int num_stages;
   int num_wr;                // W_r buffers (4 or 5)
+  uint32_t turn_offset;      // turning areas of the epilogue warps, from the start of shared memory (0: none)
   uint32_t opts;             // kOpt* bits
   long long* timing;         // time-stamp records (debug builds), else null
 };
@@ -428,39 +429,58 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
       tc_fence_after();
       constexpr int CH = NPAD < 32 ? NPAD : 32;                 // columns handled per round (register budget)
       __half* y = XT ? a.Y + row : a.Y + static_cast<long long>(row) * a.ldy;   // XT: element (row, c) at y[c * ldy]
-      // 16-byte stores when the columns fill them (N = 8 runs in the 16-column kernel)
-      const bool vec_ok = !XT && (NPAD == 16 ? (a.N & 7) == 0 : a.N == NPAD) && (a.ldy & 7) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0;
+      // Rows of Y that 16-byte stores fit are stored eight columns at a time, others turned in shared memory
+      // first (below): a thread holds a row, and two-byte stores a row pitch apart took 2-15 us of a
+      // launch (20480 x 5120, N = 63: 51 -> 35; 5120 x 5120, N = 40: 19 -> 15).
+      const bool vec_ok = !XT && (a.ldy & 7) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0;
+      const uint32_t turn = smem_base + a.turn_offset + static_cast<uint32_t>(warp & 3) * kTurnBytes;
       const bool plain = a.bias == nullptr && a.act == TL3_ACT_NONE;
-      auto fin = [](uint32_t bits) { return __uint_as_float(bits); };
       auto store_y = [&](uint32_t* v, int c0) {                 // (bias, activation,) fp32 -> fp16 (round to nearest even) -> Y
-        if (row >= a.M) return;
         if (!plain) {                                             // one test per call, not one per element
 #pragma unroll
           for (int c = 0; c < CH; ++c) v[c] = __float_as_uint(finish(__uint_as_float(v[c]), bias_v, a.act));
         }
-        if (vec_ok) {
+        if constexpr (XT) {
+          if (row >= a.M) return;
+          __half* yc = y + static_cast<long long>(c0) * a.ldy;          // column c0 of this row: Yt[c0][row]
 #pragma unroll
-          for (int c = 0; c < CH; c += 8) {
-            if (NPAD == 16 && c0 + c >= a.N) break;
-            uint4 o;
-            __half2 h0 = __floats2half2_rn(fin(v[c + 0]), fin(v[c + 1]));
-            __half2 h1 = __floats2half2_rn(fin(v[c + 2]), fin(v[c + 3]));
-            __half2 h2 = __floats2half2_rn(fin(v[c + 4]), fin(v[c + 5]));
-            __half2 h3 = __floats2half2_rn(fin(v[c + 6]), fin(v[c + 7]));
-            o.x = *reinterpret_cast<uint32_t*>(&h0); o.y = *reinterpret_cast<uint32_t*>(&h1);
-            o.z = *reinterpret_cast<uint32_t*>(&h2); o.w = *reinterpret_cast<uint32_t*>(&h3);
-            *reinterpret_cast<uint4*>(y + c0 + c) = o;
-          }
+          for (int c = 0; c < CH; ++c, yc += a.ldy)
+            if (c0 + c < a.N) *yc = __float2half_rn(__uint_as_float(v[c]));
         } else {
-          if (XT) {
-            __half* yc = y + static_cast<long long>(c0) * a.ldy;          // column c0 of this row: Yt[c0][row]
+          uint32_t o[CH / 2];
 #pragma unroll
-            for (int c = 0; c < CH; ++c, yc += a.ldy)
-              if (c0 + c < a.N) *yc = __float2half_rn(fin(v[c]));
-          } else {
+          for (int c = 0; c < CH / 2; ++c) {
+            const __half2 h = __floats2half2_rn(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]));
+            o[c] = *reinterpret_cast<const uint32_t*>(&h);
+          }
+          if (vec_ok && (a.N & 7) == 0) {
+            if (row >= a.M) return;
+#pragma unroll
+            for (int c = 0; c < CH; c += 8)
+              if (c0 + c < a.N) *reinterpret_cast<uint4*>(y + c0 + c) = make_uint4(o[c / 2], o[c / 2 + 1], o[c / 2 + 2], o[c / 2 + 3]);
+          } else if (a.turn_offset) {
+            // 16 columns at a time: every lane puts down its row, half a warp picks up one
+            const int col = lane & 15, row0 = row - lane + (lane >> 4);
+#pragma unroll
+            for (int g = 0; g < CH; g += 16) {
+              if (c0 + g >= a.N) break;
+              __syncwarp();
+#pragma unroll
+              for (int c = 0; c < 8; ++c) sts_u32(turn + static_cast<uint32_t>(lane) * kTurnPitch + 4u * c, o[g / 2 + c]);
+              __syncwarp();
+              uint16_t* yt = reinterpret_cast<uint16_t*>(a.Y) + static_cast<long long>(row0) * a.ldy + c0 + g + col;
+              const bool in = c0 + g + col < a.N;
+#pragma unroll 4
+              for (int i = 0; i < 16; ++i, yt += 2 * a.ldy) {
+                const uint32_t h = lds_u16(turn + static_cast<uint32_t>(2 * i + (lane >> 4)) * kTurnPitch + 2u * col);
+                if (in && row0 + 2 * i < a.M) *yt = static_cast<uint16_t>(h);
+              }
+            }
+          } else if (row < a.M) {
+            uint16_t* ys = reinterpret_cast<uint16_t*>(y) + c0;
 #pragma unroll
             for (int c = 0; c < CH; ++c)
-              if (c0 + c < a.N) y[c0 + c] = __float2half_rn(fin(v[c]));
+              if (c0 + c < a.N) ys[c] = static_cast<uint16_t>(o[c / 2] >> (16 * (c & 1)));
           }
         }
       };
@@ -842,7 +862,13 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   }
   if (stages < 2) return TL3_ERR_UNSUPPORTED;
   if (stages > kMaxStages) stages = kMaxStages;
-  const uint32_t smem_bytes = fixed + static_cast<uint32_t>(stages) * stage_stride;
+  uint32_t smem_bytes = fixed + static_cast<uint32_t>(stages) * stage_stride;
+  // the epilogue's turning areas behind everything else, where they cost no stage (four and a half KB)
+  uint32_t turn_offset = 0;
+  if (!xt && smem_bytes + 4 * kTurnBytes <= kSmemLimit) {
+    turn_offset = smem_bytes - 1024u;                              // (the last 1024 bytes are for the alignment of the first)
+    smem_bytes += 4 * kTurnBytes;
+  }
 
   // tensor map of X: dims {N, K}, box {n_pad, 128}; columns >= N and rows >= K read as zero
   EncodeTiledFn encode = encode_tiled_fn();
@@ -883,6 +909,7 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   args.x_offset = block_area;
   args.num_stages = stages;
   args.num_wr = num_wr;
+  args.turn_offset = turn_offset;
   // Decoding ahead of X pays where a launch is short (a tile or a few per CTA: most of its time is
   // the start) and measured level or slightly worse on longer ones.
   const int dbx = g_decode_before_x.load(std::memory_order_relaxed);

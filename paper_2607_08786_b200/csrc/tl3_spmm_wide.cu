@@ -46,8 +46,6 @@ constexpr int kMaxRing = 8;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kColMetaT = 480;       // + 4 * (W_r buffer)
 constexpr uint32_t kColMetaR = 496;
-constexpr uint32_t kTurnPitch = 36;       // bytes per row of a warp's turning area (16 halves, odd number of words)
-constexpr uint32_t kTurnBytes = 32u * kTurnPitch;
 constexpr uint32_t kSlack = 1024u + 4u * kTurnBytes + 1024u;   // barriers, the epilogue warps' turning areas, alignment
 
 struct WideArgs {
