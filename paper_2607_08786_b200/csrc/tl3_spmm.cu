@@ -888,6 +888,20 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   const long long total = m->n_tiles;
   const int grid = static_cast<int>(total < di.sm_count ? total : di.sm_count);
   if (static_cast<unsigned long long>(total) * static_cast<unsigned long long>(grid + 1) >= (1ull << 32)) return TL3_ERR_UNSUPPORTED;   // the kernel splits the tiles in 32-bit arithmetic
+  // A row-tile shared by so many CTAs that their partial sums do not fit the stages is added up from
+  // global memory by the four epilogue warps here; the wide kernel has its decode warps help.  Staged, this
+  // kernel's reducer is the faster one.  With 16 KB slots a few reducers above the limit are no loss yet.
+  // (us here / there: 1024 x 1024, N = 64 15.3 / 9.4; 4096 x 4096, N = 64 17.4 / 14.3; 1024 x 4096, N = 32 16.9 /
+  // 13.4; staged: 5120 x 5120, N = 64 14.9 / 17.0; 2000 x 8000, N = 32 11.2 / 14.5.  8 KB slots: 700 x 24000, N = 16,
+  // 27 CTAs per row-tile, 18.2 / 19.4.)
+  if (n_pad > 16) {
+    const unsigned long long sharing = (static_cast<unsigned long long>(m->tiles_k) * grid + total - 1) / total;   // CTAs per row-tile
+    const unsigned long long staging = static_cast<unsigned long long>(stages) * stage_stride;
+    if (sharing * (n_pad * 512ull) > (n_pad == 32 ? staging + staging / 4 : staging)) {
+      const int rc = spmm_wide(m, X, ldx, Y, ldy, N, ep, xt, workspace, stream);
+      if (rc != kWideNoPlan) return rc;
+    }
+  }
   const WorkspaceLayout wl = workspace_layout(N, di.sm_count);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   KernelArgs args;

@@ -26,10 +26,12 @@ def _within(oracle_mod, W, X, Y):
 
 # Column counts around the edges of a pass (one and two accumulators, one and two passes, a ragged last
 # one), shapes with one tile, ragged tiles, many CTAs per row-tile and many row-tiles per CTA, blocks
-# so large that fewer buffers fit (dense) and every pitch of Y that 16-byte stores can not take.
+# so large that fewer buffers fit (dense), every pitch of Y that 16-byte stores can not take, and up to
+# 64 columns with many CTAs per row-tile.
 @pytest.mark.parametrize("M,K,N,sparsity", [(128, 128, 65, 0.5), (7, 8, 80, 0.5), (300, 2000, 129, 0.6), (1000, 1096, 96, 0.4),
                                             (2048, 4096, 240, 0.5), (2048, 4096, 241, 0.5), (700, 3000, 256, 0.5),
-                                            (9000, 640, 257, 0.5), (640, 9000, 300, 0.7), (512, 640, 512, 0.0), (20000, 256, 200, 0.5)])
+                                            (9000, 640, 257, 0.5), (640, 9000, 300, 0.7), (512, 640, 512, 0.0), (20000, 256, 200, 0.5),
+                                            (1024, 1024, 64, 0.5), (1024, 1024, 33, 0.5), (700, 6000, 24, 0.5), (1300, 1300, 32, 0.6)])
 def test_wide_products(tl3, oracle_mod, M, K, N, sparsity):
     import torch
     case = wl.Case(0, "wide", M, K, N, 300 + N, sparsity, "magnitude")
