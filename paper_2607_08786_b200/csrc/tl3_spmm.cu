@@ -894,10 +894,14 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   // (us here / there: 1024 x 1024, N = 64 15.3 / 9.4; 4096 x 4096, N = 64 17.4 / 14.3; 1024 x 4096, N = 32 16.9 /
   // 13.4; staged: 5120 x 5120, N = 64 14.9 / 17.0; 2000 x 8000, N = 32 11.2 / 14.5.  8 KB slots: 700 x 24000, N = 16,
   // 27 CTAs per row-tile, 18.2 / 19.4.)
+  // Blocks so large that fewer stages than decode groups fit go there from six CTAs per row-tile on, at N > 32
+  // (1024 x 1024 at 40 %, N = 64 15.4 / 9.4); below that the gain is smaller (4096 x 2048 at 40 %, N = 64, five
+  // CTAs, 14.9 / 12.3; 2048 x 2048 dense, N = 32 14.1 / 12.7) and this kernel keeps its case of a short ring.
   if (n_pad > 16) {
     const unsigned long long sharing = (static_cast<unsigned long long>(m->tiles_k) * grid + total - 1) / total;   // CTAs per row-tile
     const unsigned long long staging = static_cast<unsigned long long>(stages) * stage_stride;
-    if (sharing * (n_pad * 512ull) > (n_pad == 32 ? staging + staging / 4 : staging)) {
+    const bool unstaged = sharing * (n_pad * 512ull) > (n_pad == 32 ? staging + staging / 4 : staging);
+    if (unstaged && (stages >= kGroups || (n_pad == 64 && sharing > 5))) {
       const int rc = spmm_wide(m, X, ldx, Y, ldy, N, ep, xt, workspace, stream);
       if (rc != kWideNoPlan) return rc;
     }
