@@ -173,21 +173,6 @@ enum : uint32_t {
   kBarAccFull = 48, kBarReduce = 50, kBarAccEmpty = 51, kBarCount = 53, kTmemSlot = 53, kAbort = 54
 };
 
-// Bias and activation of 16 sums of one row.  One branch per 16 columns, the functions inlined: a
-// call per element (as in tl3_spmm.cu, where a small kernel image matters more) took 50 us of 181 on
-// 20480 x 5120, N = 512 with bias and ReLU.
-__device__ __forceinline__ void apply_epilogue(uint32_t (&v)[16], float bias, int act) {
-#pragma unroll
-  for (int c = 0; c < 16; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) + bias);
-  if (act == TL3_ACT_RELU) {
-#pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] = __float_as_uint(fmaxf(__uint_as_float(v[c]), 0.f));
-  } else if (act != TL3_ACT_NONE) {
-#pragma unroll
-    for (int c = 0; c < 16; ++c) v[c] = __float_as_uint(finish(__uint_as_float(v[c]), 0.f, act));
-  }
-}
-
 // Columns c_begin, c_begin + c_step, ... (16 at a time) of one row of a row-tile: accumulator (+ the
 // partial sums of the n_others CTAs after this one, in ascending order whatever the order they came
 // in), bias, activation, rounding, Y.  Executed by whole warps, `et` is the row, 32 * (warp % 4) + lane.
@@ -236,7 +221,7 @@ __device__ __noinline__ void write_columns(const WideArgs& a, uint32_t acc_tmem,
         }
       }
     }
-    if (!plain) apply_epilogue(v, bias, a.act);
+    if (!plain) apply_epilogue<CH>(v, bias, a.act, cols - c0);
     uint32_t o[CH / 2];
 #pragma unroll
     for (int c = 0; c < CH / 2; ++c) {
