@@ -192,10 +192,11 @@ int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream);
 int tl3_bind(tl3_matrix* m, void* dptr);
 
 /* Scratch the kernel needs for N columns: split-K partial sums, one arrival flag per partial-sum
- * slot, a status word.  Depends on the current device's SM count.  The caller allocates it (device,
- * 256-byte aligned), clears it once with tl3_workspace_init(), and may then reuse it for any number
+ * slot, a status word.  Depends on the current device's SM count and grows with N up to 256 columns (9.7 MB
+ * from N = 33 on, 19.4 MB from N = 225 on, with 148 SMs).  The caller allocates it (device, 256-byte aligned),
+ * clears it once with tl3_workspace_init(), and may then reuse it for any number
  * of calls that do not overlap on the GPU (the kernel leaves it cleared; after a call that ended
- * with a non-zero status, clear it again). */
+ * with a non-zero status, clear it again).  tl3_workspace_init() also records `bytes` in it. */
 size_t tl3_workspace_bytes(const tl3_matrix* m, int N);
 int tl3_workspace_init(void* workspace, size_t bytes, void* stream);
 
@@ -210,8 +211,8 @@ int tl3_workspace_init(void* workspace, size_t bytes, void* stream);
  *   with an element of X).
  * Asynchronous on `stream`; allocates nothing; does not synchronise.  Calls that share a
  * workspace must not overlap on the GPU; the workspace must hold tl3_workspace_bytes(m, N) bytes
- * for THIS N (it grows with N up to 256: that many columns of partial sums per CTA), the call cannot
- * check that.  Calls on different streams, each with its own workspace, may be in flight together.
+ * for THIS N, which the call cannot check; only from 33 columns on does one made for fewer serve
+ * any N (more than 128 columns are then taken at half as many a pass).  Calls on different streams, each with its own workspace, may be in flight together.
  * A row-tile shared by several CTAs is finished by the CTA that owns its first tile, which waits
  * (bounded, status code 11) for CTAs with a higher index; that those get to run while other
  * kernels hold SMs rests on the GPU dispatching the blocks of a grid in index order.

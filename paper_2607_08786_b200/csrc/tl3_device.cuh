@@ -333,12 +333,13 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 EncodeTiledFn encode_tiled_fn();
 
 struct WorkspaceLayout {
-  size_t status_off = 0, flags_off = 256, partials_off = 0, total = 0;
+  size_t status_off = 0, flags_off = 256, room_off = 0, partials_off = 0, total = 0;
 };
 WorkspaceLayout workspace_layout(int N, int sm_count);
 
 // ---- tl3_spmm_wide.cu: N > 64 columns in one launch
 constexpr int kWideColumns = 256;                               // most columns of one pass over W
+constexpr int kRoomUnit = 16;                                   // unit of the workspace's record of its size, in columns per CTA
 int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t ldy, int N, const tl3_epilogue* ep, bool xt,
               void* workspace, void* stream);                   // kWideNoPlan: blocks too large for it
 

@@ -25,6 +25,7 @@
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cstdint>
 #include <cstring>
@@ -678,7 +679,8 @@ static inline int n_pad_of(int N) { return N <= 16 ? 16 : N <= 32 ? 32 : 64; }
 // have; 128 of those are as many bytes as the two slots of 64.
 WorkspaceLayout workspace_layout(int N, int sm_count) {
   WorkspaceLayout w;
-  w.partials_off = (256 + static_cast<size_t>(2) * sm_count * 4 + 4095) / 4096 * 4096;
+  w.room_off = (256 + static_cast<size_t>(2) * sm_count * 4 + 4095) / 4096 * 4096;
+  w.partials_off = w.room_off + 256;
   int columns = 2 * n_pad_of(N);
   if (N > 128) columns = N < kWideColumns ? (N + 31) / 32 * 32 : kWideColumns;
   w.total = w.partials_off + static_cast<size_t>(columns) * sm_count * 128 * sizeof(float);
@@ -823,6 +825,16 @@ size_t tl3_workspace_bytes(const tl3_matrix* m, int N) {
 int tl3_workspace_init(void* workspace, size_t bytes, void* stream) {
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) != 0) return TL3_ERR_INVALID_ARG;
   TL3_CUDA(cudaMemsetAsync(workspace, 0, bytes, static_cast<cudaStream_t>(stream)));
+  // how many columns of partial sums per CTA there is room for: what a product of more than 128 columns
+  // goes by (a memory that was only zeroed counts as the smallest)
+  tl3::DeviceInfo di;
+  if (int rc = tl3::device_info(&di)) return rc;
+  const tl3::WorkspaceLayout wl = tl3::workspace_layout(1, di.sm_count);
+  if (bytes > wl.partials_off) {
+    const size_t columns = (bytes - wl.partials_off) / (static_cast<size_t>(di.sm_count) * 128 * sizeof(float));
+    const size_t room = std::min<size_t>(columns / tl3::kRoomUnit, 255);
+    TL3_CUDA(cudaMemsetAsync(static_cast<uint8_t*>(workspace) + wl.room_off, static_cast<int>(room), 1, static_cast<cudaStream_t>(stream)));
+  }
   return TL3_OK;
 }
 

@@ -51,8 +51,11 @@ constexpr uint32_t kSlack = 1024u + 4u * kTurnBytes + 1024u;   // barriers, the 
 struct WideArgs {
   const uint8_t* blob;
   const DirEntry* dir;
-  uint32_t tiles_m, tiles_k, chunks;      // tiles of W, groups of n_pad columns
-  int M, N, n_pad;
+  uint32_t tiles_m, tiles_k;              // tiles of W
+  int M, N;
+  int n_pad[2];                           // columns of a pass; for pairs also: in a workspace made for 128 columns or fewer
+  uint32_t chunks[2];                     // groups of so many columns
+  const unsigned char* room;              // columns of partial sums per CTA that the workspace holds, / kRoomUnit
   long long ldy;
   __half* Y;
   const __half* bias;
@@ -180,15 +183,18 @@ enum : uint32_t {
 // 16-byte stores do not fit are turned there first: stored by their rows' threads, two bytes each a
 // row pitch apart, they took 6 us of 25 on 4096 x 4096, N = 65.
 template <bool XT, int S, bool kShared>
-__device__ __noinline__ void write_columns(const WideArgs& a, uint32_t acc_tmem, int et, uint32_t vrow, int c_begin, int c_step, int n_others, uint32_t turn) {
+__device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t acc_tmem, int et, uint32_t vrow, int c_begin, int c_step, int n_others,
+                                           uint32_t turn) {
   constexpr int CH = 16;
-  const int row = static_cast<int>(S * (vrow / a.chunks) + blockIdx.x % S) * kTileM + et;
-  const int n0 = static_cast<int>(vrow % a.chunks) * a.n_pad;
-  const int cols = a.N - n0 < a.n_pad ? a.N - n0 : a.n_pad;
+  const int n_pad = a.n_pad[less];
+  const uint32_t chunks = a.chunks[less];
+  const int row = static_cast<int>(S * (vrow / chunks) + blockIdx.x % S) * kTileM + et;
+  const int n0 = static_cast<int>(vrow % chunks) * n_pad;
+  const int cols = a.N - n0 < n_pad ? a.N - n0 : n_pad;
   const bool plain = a.bias == nullptr && a.act == TL3_ACT_NONE;
   const float bias = a.bias != nullptr && row < a.M ? __half2float(__ldg(a.bias + row)) : 0.f;
   const bool vec_ok = !XT && (a.ldy & 7) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 15) == 0;
-  const size_t slot = static_cast<size_t>(a.n_pad) * 128;
+  const size_t slot = static_cast<size_t>(n_pad) * 128;
   const int lane = et & 31;
   // XT: four lanes hand each other their values, so that a thread stores four rows of one column
   const bool quads = XT && row - lane + 32 <= a.M && (a.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 7) == 0;
@@ -307,7 +313,12 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
   // group minor), k-tile v % tiles_k.  An odd last row-tile is done by both CTAs of a pair (the second
   // one's rows lie beyond M and are not stored).
   const uint32_t rank = blockIdx.x % S, unit = blockIdx.x / S;
-  const uint32_t TK = a.tiles_k, T = (a.tiles_m + S - 1) / S * a.chunks * TK, G = gridDim.x / S;
+  // The partial sums of a pair are up to 256 columns per CTA.  A workspace made for fewer, which
+  // tl3_workspace_init() recorded in it, gets passes of half the columns: the slices of X are then loaded
+  // as wide as ever and used in part.  (The record is older than anything a kernel before this one does:
+  // no wait for it.)
+  const int less = S == 2 && static_cast<int>(__ldcg(a.room)) * kRoomUnit < a.n_pad[0] ? 1 : 0;
+  const uint32_t TK = a.tiles_k, T = (a.tiles_m + S - 1) / S * a.chunks[less] * TK, G = gridDim.x / S;
   const uint32_t t_begin = range_begin(unit, T, G), t_end = range_begin(unit + 1, T, G);
   const int n_tiles = static_cast<int>(t_end - t_begin);
   const uint32_t kt_begin = t_begin % TK, vrow_begin = t_begin / TK;
@@ -345,7 +356,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
       if (base + lane < n_tiles) {
         uint32_t k = kt + static_cast<uint32_t>(lane), v = vrow;
         while (k >= TK) { k -= TK; ++v; }
-        const uint32_t mt = S * (v / a.chunks) + rank;
+        const uint32_t mt = S * (v / a.chunks[less]) + rank;
         mine = __ldg(reinterpret_cast<const uint4*>(a.dir + static_cast<size_t>(mt < a.tiles_m ? mt : a.tiles_m - 1) * TK + k));
       }
       const int cnt = n_tiles - base < 32 ? n_tiles - base : 32;
@@ -378,7 +389,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
     uint32_t kt = kt_begin, vrow = vrow_begin;
     pdl_wait();                                                    // the kernel before this one may have written X
     for (int j = 0; j < 2 * n_tiles; ++j) {
-      const int n0 = static_cast<int>(vrow % a.chunks) * a.n_pad + static_cast<int>(rank) * (a.n_pad / S);
+      const int n0 = static_cast<int>(vrow % a.chunks[less]) * a.n_pad[less] + static_cast<int>(rank) * (a.n_pad[less] / S);
       const int last = j - a.n_x;                                  // the slice that was here before
       if (last >= 0 && !__all_sync(0xFFFFFFFFu, (last & 1) ? wait_done(last >> 1, wctx, kStProducer) : wait_half(last >> 1, wctx, kStProducer))) break;
       if (elect_one()) {
@@ -415,7 +426,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
     // apart, a k-block is 64 bytes of a row; otherwise blocks of 64 k-rows x 128 bytes (64 columns),
     // MN-major, 8-row groups 1024 B apart (stride field), the blocks 8192 B (leading-offset field), a
     // k-block is 32 rows.
-    const uint32_t idesc = (1u << 2) | (1u << 4) | (XT ? 0u : (1u << 16)) | (static_cast<uint32_t>(a.n_pad >> 3) << 17) | (8u * S << 24);
+    const uint32_t idesc = (1u << 2) | (1u << 4) | (XT ? 0u : (1u << 16)) | (static_cast<uint32_t>(a.n_pad[less] >> 3) << 17) | (8u * S << 24);
     constexpr uint32_t kHi = (1024u >> 4) | (1u << 14) | (2u << 29);
     constexpr uint32_t kLboA = 1u << 16, kLboB = XT ? (1u << 16) : ((8192u >> 4) << 16);
     constexpr uint32_t kBStep = (XT ? 64u : 4096u) >> 4;
@@ -426,7 +437,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
       const bool first_of_seg = (i == 0) || (kt == 0);
       const bool last_of_seg = (i == n_tiles - 1) || (kt == TK - 1);
       const int b = a.n_acc == 2 ? seg & 1 : 0, b_use = a.n_acc == 2 ? seg >> 1 : seg;
-      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(b * a.n_pad);
+      const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(b * a.n_pad[less]);
       const uint32_t e_t = tmem_base + kColMetaT + 4 * wb, e_r = tmem_base + kColMetaR;
       const uint32_t a_lo = ((w_base + static_cast<uint32_t>(s) * a.block_area) >> 4) | kLboA;
       const uint32_t r_lo = ((wr_base + static_cast<uint32_t>(wb) * kWrBytes) >> 4) | kLboA;
@@ -528,8 +539,8 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
         tc_fence_after();
         __threadfence();
         const int last_seg = static_cast<int>(vrow - vrow_begin);
-        const uint32_t acc = tmem_base + lane_base + static_cast<uint32_t>((a.n_acc == 2 ? last_seg & 1 : 0) * a.n_pad);
-        write_columns<XT, S, true>(a, acc, r, vrow, 16 * (g + 1), 16 * (kGroups + 1), owner_of((vrow + 1) * TK - 1, T, G) - static_cast<int>(unit),
+        const uint32_t acc = tmem_base + lane_base + static_cast<uint32_t>((a.n_acc == 2 ? last_seg & 1 : 0) * a.n_pad[less]);
+        write_columns<XT, S, true>(a, less, acc, r, vrow, 16 * (g + 1), 16 * (kGroups + 1), owner_of((vrow + 1) * TK - 1, T, G) - static_cast<int>(unit),
                           wr_base + static_cast<uint32_t>(warp - kDecodeWarp0) * kTurnBytes);   // (the W_r buffers are idle too)
       }
     }
@@ -552,7 +563,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
       const int n_others = c_last - c_first;
       if (!named_bar_all(kEpilogueBarrier, 128, mbar_wait_unit<S>(bar(kBarAccFull, b), b_use & 1, wctx, kStEpilogueAccFull))) break;
       tc_fence_after();
-      const uint32_t acc_tmem = tmem_base + lane_base + static_cast<uint32_t>(b * a.n_pad);
+      const uint32_t acc_tmem = tmem_base + lane_base + static_cast<uint32_t>(b * a.n_pad[less]);
       bool ready = true;
       if (reducer) {
         // The contributors (the CTAs after this one, or its counterparts in the pairs after this one) store their partial sums and raise their flags;
@@ -594,13 +605,13 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
       if (ready) {
         const uint32_t turn = bar0 + 1024u + static_cast<uint32_t>(warp & 3) * kTurnBytes;
         if (complete) {
-          write_columns<XT, S, false>(a, acc_tmem, et, vrow, 0, 16, 0, turn);
+          write_columns<XT, S, false>(a, less, acc_tmem, et, vrow, 0, 16, 0, turn);
         } else if (reducer) {
-          write_columns<XT, S, true>(a, acc_tmem, et, vrow, 0, 16 * (kGroups + 1), n_others, turn);
+          write_columns<XT, S, true>(a, less, acc_tmem, et, vrow, 0, 16 * (kGroups + 1), n_others, turn);
         } else {
-          float* mine = a.partials + static_cast<size_t>(a.n_pad) * 128 * blockIdx.x + et;
+          float* mine = a.partials + static_cast<size_t>(a.n_pad[less]) * 128 * blockIdx.x + et;
 #pragma unroll 1
-          for (int c0 = 0; c0 < a.n_pad; c0 += 16) {
+          for (int c0 = 0; c0 < a.n_pad[less]; c0 += 16) {
             uint32_t v[16];
             TmemLd<16>::ld(acc_tmem + c0, v);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
@@ -701,12 +712,14 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   if (di.cc_major != 10) return TL3_ERR_UNSUPPORTED;
 
   WideArgs a{};
-  a.n_pad = wide_columns(m, N, di.sm_count);
-  a.chunks = static_cast<uint32_t>((N + a.n_pad - 1) / a.n_pad);
+  const int n_pad = wide_columns(m, N, di.sm_count);
   a.block_area = (m->max_block_bytes + 1023u) / 1024u * 1024u;
-  const int S = a.n_pad > kAloneColumns ? 2 : 1;
-  a.x_bytes = xt ? static_cast<uint32_t>(a.n_pad / S) * 128u : static_cast<uint32_t>((a.n_pad / S + 63) / 64) * 8192u;   // per CTA
-  a.n_acc = 2 * a.n_pad <= static_cast<int>(kColMetaT) ? 2 : 1;
+  const int S = n_pad > kAloneColumns ? 2 : 1;
+  a.n_pad[0] = n_pad;
+  a.n_pad[1] = S == 1 ? n_pad : (n_pad / 2 + 31) / 32 * 32;         // (an MMA of 256 rows takes multiples of 32)
+  for (int i = 0; i < 2; ++i) a.chunks[i] = static_cast<uint32_t>((N + a.n_pad[i] - 1) / a.n_pad[i]);
+  a.x_bytes = xt ? static_cast<uint32_t>(n_pad / S) * 128u : static_cast<uint32_t>((n_pad / S + 63) / 64) * 8192u;   // per CTA
+  a.n_acc = 2 * n_pad <= static_cast<int>(kColMetaT) ? 2 : 1;
   {
     // A W_r buffer per decode group (with two of them instead of three 20480 x 5120, N = 512 took 131 us, not
     // 122, with three instead of four, in pairs, 113, not 108), at least as many blocks, and four X slices, three
@@ -739,16 +752,18 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   // dims {N, K}, box {64 columns, 64 k}; transposed: dims {K, N}, box {64 k, n_pad / S rows}.  What lies beyond reads as zero.
   const cuuint64_t dims[2] = {static_cast<cuuint64_t>(xt ? m->K : N), static_cast<cuuint64_t>(xt ? N : m->K)};
   const cuuint64_t strides[1] = {static_cast<cuuint64_t>(ldx) * 2};
-  const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(xt ? a.n_pad / S : 64)};
+  const cuuint32_t box[2] = {64, static_cast<cuuint32_t>(xt ? n_pad / S : 64)};
   const cuuint32_t elem_strides[2] = {1, 1};
   const CUresult cr = encode(&map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(X), dims, strides, box, elem_strides,
                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (cr != CUDA_SUCCESS) { set_cuda_error(static_cast<int>(cr)); return TL3_ERR_CUDA; }
 
-  const unsigned long long total = static_cast<unsigned long long>((m->tiles_m + S - 1) / S) * m->tiles_k * a.chunks;
+  const unsigned long long total = static_cast<unsigned long long>((m->tiles_m + S - 1) / S) * m->tiles_k * a.chunks[0];
   const int units = static_cast<int>(total < static_cast<unsigned long long>(di.sm_count / S) ? total : di.sm_count / S);
-  if (total * static_cast<unsigned long long>(units + 1) >= (1ull << 32)) return kWideNoPlan;   // the kernel splits the tiles in 32-bit arithmetic
+  // the kernel splits the tiles in 32-bit arithmetic, whichever the columns of a pass
+  const unsigned long long most = total / a.chunks[0] * a.chunks[1];
+  if (most * static_cast<unsigned long long>(units + 1) >= (1ull << 32)) return kWideNoPlan;
   const int grid = S * units;
   const WorkspaceLayout wl = workspace_layout(N, di.sm_count);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
@@ -765,6 +780,7 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   a.partials = reinterpret_cast<float*>(ws + wl.partials_off);
   a.flags = reinterpret_cast<unsigned int*>(ws + wl.flags_off);
   a.status = reinterpret_cast<unsigned int*>(ws + wl.status_off);
+  a.room = ws + wl.room_off;
   m->last_ctas = grid; m->last_stages = a.n_w; m->last_smem = static_cast<int>(smem_bytes);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (S == 2) return xt ? launch_wide<true, 2>(map, a, grid, smem_bytes, st) : launch_wide<false, 2>(map, a, grid, smem_bytes, st);

@@ -313,10 +313,6 @@ class Matrix:
         _check(lib().tl3_workspace_init(ws.data_ptr(), n, _stream_ptr(stream)), "tl3_workspace_init")
         return ws
 
-    def _too_small(self, workspace, N: int) -> bool:
-        """A workspace made for fewer columns: the product is then taken 64 columns at a time."""
-        return workspace.numel() * workspace.element_size() < self.workspace_bytes(N)
-
     def spmm(self, X, Y=None, workspace=None, stream=None, bias=None, activation=None):
         """``Y = W X`` on the GPU, or ``Y = act(W X + bias)`` when a bias (torch.float16, M entries, on
         the device) and / or an activation ("relu", "silu", "gelu_tanh") is given.
@@ -335,10 +331,6 @@ class Matrix:
             workspace = self._workspaces.get(key)
             if workspace is None:
                 workspace = self._workspaces[key] = self.new_workspace(key, stream)
-        elif N > 128 and self._too_small(workspace, N):
-            for n in range(0, N, 64):
-                self.spmm(X[:, n:n + 64], Y[:, n:n + 64], workspace, stream, bias, activation)
-            return Y
         if bias is None and activation is None:
             _check(lib().tl3_spmm(self._h, X.data_ptr(), X.stride(0), Y.data_ptr(), Y.stride(0), N,
                                   workspace.data_ptr(), _stream_ptr(stream)), "tl3_spmm")
@@ -367,10 +359,6 @@ class Matrix:
             workspace = self._workspaces.get(key)
             if workspace is None:
                 workspace = self._workspaces[key] = self.new_workspace(key, stream)
-        elif N > 128 and self._too_small(workspace, N):
-            for n in range(0, N, 64):
-                self.spmm_nt(Xt[n:n + 64], Yt[n:n + 64], workspace, stream, bias, activation)
-            return Yt
         if bias is not None and (bias.dtype != torch.float16 or bias.numel() != M or not bias.is_contiguous()):
             raise ValueError("bias must be a contiguous float16 tensor with one entry per row of W")
         ep = None

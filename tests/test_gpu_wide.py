@@ -85,8 +85,7 @@ def test_wide_bias_and_activation(tl3, activation):
 
 
 def test_a_workspace_for_fewer_columns_still_serves_wide_products(tl3):
-    """The binding sees the size of the workspace it is given; one that was made for 64 columns is used
-    64 columns at a time."""
+    """One that was made for 64 columns; more of them in test_gpu_workspace.py."""
     import torch
     case = wl.Case(0, "wide_ws", 900, 700, 300, 10, 0.5, "magnitude")
     W, X = case.make_W(), case.make_X()
