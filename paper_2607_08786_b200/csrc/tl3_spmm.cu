@@ -556,7 +556,7 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
           for (int c0 = 0; c0 < NPAD; c0 += CH) {
             uint32_t v[CH];
             TmemLd<CH>::ld(acc_tmem + c0, v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            tmem_wait_ld<CH>(v);
             // own part first (lowest CTA), then the others in ascending order.  Two loops: in one
             // loop the slot arithmetic of the unstaged case (a 64-bit division per contributor)
             // was computed on the staged path too, 0.25 us on a reducer's way out.
@@ -591,7 +591,7 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
       for (int c0 = 0; c0 < NPAD; c0 += CH) {
         uint32_t v[CH];
         TmemLd<CH>::ld(acc_tmem + c0, v);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        tmem_wait_ld<CH>(v);
         if (complete) {
           store_y(v, c0);
         } else {

@@ -206,13 +206,13 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
   for (int c0 = c_begin; c0 < cols; c0 += c_step) {
     uint32_t v[CH];
     if (!kShared) {
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      tmem_wait_ld<CH>(next);
 #pragma unroll
       for (int c = 0; c < CH; ++c) v[c] = next[c];
       if (c0 + c_step < cols) TmemLd<CH>::ld(acc_tmem + c0 + c_step, next);
     } else {
       TmemLd<CH>::ld(acc_tmem + c0, v);
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      tmem_wait_ld<CH>(v);
       const float* p = a.partials + slot * (blockIdx.x + S) + c0 * 128 + et;   // the next CTA, or the same one of the next pair
       for (int k = 0; k < n_others; k += 2, p += 2 * S * slot) {
         float p0[CH], p1[CH];
@@ -284,7 +284,6 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
       }
     }
   }
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
 // XT as in tl3_spmm.cu: activations and result transposed ([batch, hidden]).
@@ -614,7 +613,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
           for (int c0 = 0; c0 < a.n_pad[less]; c0 += 16) {
             uint32_t v[16];
             TmemLd<16>::ld(acc_tmem + c0, v);
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            tmem_wait_ld<16>(v);
 #pragma unroll
             for (int c = 0; c < 16; ++c) __stcg(mine + (c0 + c) * 128, __uint_as_float(v[c]));
           }
