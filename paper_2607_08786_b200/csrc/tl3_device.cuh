@@ -26,6 +26,9 @@ constexpr uint32_t kSmemLimit = 232448;   // 227 KB
 constexpr uint32_t kTurnPitch = 36;       // bytes per row of a warp's turning area (16 halves, odd number of words)
 constexpr uint32_t kTurnBytes = 32u * kTurnPitch;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // 2 s without progress, per wait
+// A wait behind several others of the same CTA, each with its own 2 s (the last MMAs, an accumulator, the
+// contributors' flags): one that gives up raises the abort flag, this one ends with it and reports nothing.
+constexpr unsigned long long kHandOverLimitNs = 4 * kWaitLimitNs;
 #ifndef TL3_TRYWAIT_HINT_NS
 #define TL3_TRYWAIT_HINT_NS 20000u
 #endif
@@ -85,7 +88,7 @@ struct WaitCtx {
 // The limit runs from the moment THIS wait began to look slow (its sixteenth unsuccessful probe), not
 // from the start of the kernel: a wait that completes is progress, so a long launch, or one whose
 // context was switched out for a while earlier on, does not use up the allowance of later waits.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& w, uint32_t code) {
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const WaitCtx& w, uint32_t code, unsigned long long limit = kWaitLimitNs) {
   unsigned long long t_slow = 0;
   for (uint32_t it = 0;; ++it) {
     if (mbar_try_wait(bar, parity)) return true;
@@ -93,7 +96,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, const W
       if (*w.abort_flag) return false;
       const unsigned long long now = global_timer();
       if (t_slow == 0) t_slow = now;
-      if (now - t_slow > kWaitLimitNs) {
+      if (now - t_slow > limit) {
         atomicCAS(w.status, 0u, code);
         *w.abort_flag = 1;
         return false;

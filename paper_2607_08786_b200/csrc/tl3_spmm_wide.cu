@@ -533,8 +533,8 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
     // the partial sums together with the epilogue warps (an accumulator is as wide as 256 columns, and
     // four warps alone had 16 us of loads in a row in front of them on 4096 x 4096, N = 128).
     const uint32_t vrow = (t_end - 1) / TK;
-    if (vrow * TK >= t_begin && (vrow + 1) * TK > t_end && !*abort_flag) {
-      if (__all_sync(0xFFFFFFFFu, mbar_wait(bar(kBarReduce, 0), 0, wctx, kStEpilogueTail))) {
+    if (vrow * TK >= t_begin && (vrow + 1) * TK > t_end) {
+      if (__all_sync(0xFFFFFFFFu, mbar_wait(bar(kBarReduce, 0), 0, wctx, kStEpilogueTail, kHandOverLimitNs))) {
         tc_fence_after();
         __threadfence();
         const int last_seg = static_cast<int>(vrow - vrow_begin);

@@ -15,3 +15,15 @@ def test_tensor_memory_waits_name_the_registers():
     assert waits
     for name, operands in waits:
         assert operands.count('"+r"') in (16, 32), (name, operands)
+
+
+def test_the_hand_over_outlasts_the_waits_it_depends_on():
+    """The decode warps of the wide kernel wait for the epilogue, whose own waits (2 s each) have to be the
+    ones that give up: a missing contributor is status 11.  And no lane leaves on its own reading of the
+    abort flag, in front of votes of the whole warp."""
+    device, wide = (CSRC / "tl3_device.cuh").read_text(), (CSRC / "tl3_spmm_wide.cu").read_text()
+    assert int(re.search(r"kHandOverLimitNs = (\d+) \* kWaitLimitNs", device)[1]) >= 4
+    waits = re.findall(r"mbar_wait\(bar\(kBarReduce, 0\)[^;]*?\)\)", wide)
+    assert len(waits) == 1 and "kHandOverLimitNs" in waits[0]
+    decode = wide[wide.index("decode (Algorithm 1)"):wide.index("} else if (warp >= kEpilogueWarp0)")]
+    assert "abort_flag" not in decode
