@@ -269,6 +269,9 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
         *reinterpret_cast<uint4*>(y) = odd ? make_uint4(other[0], other[1], other[2], other[3]) : make_uint4(o[0], o[1], o[2], o[3]);
       if (r0 + 1 < a.M)
         *reinterpret_cast<uint4*>(y + a.ldy) = odd ? make_uint4(o[4], o[5], o[6], o[7]) : make_uint4(other[0], other[1], other[2], other[3]);
+    } else if (vec_ok && cols - c0 == 8) {
+      // half a step at the end (20480 x 128, N = 72 turned 9.5 us, so 8.2; 20480 x 5120, N = 88 46.2 and 45.0)
+      if (row < a.M) *reinterpret_cast<uint4*>(a.Y + static_cast<long long>(row) * a.ldy + n0 + c0) = make_uint4(o[0], o[1], o[2], o[3]);
     } else {
       const int col = lane & 15;
       __syncwarp();

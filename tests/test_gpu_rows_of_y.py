@@ -1,5 +1,5 @@
-"""Rows of Y that 16-byte stores fit and rows that are turned in shared memory first, at up to 64 columns
-(needs a B200): every pitch gives the same bits, nothing beyond the columns is touched, and the values are
+"""Rows of Y that 16-byte stores fit, rows that are turned in shared memory first and rows that are stored as
+they are, at up to 64 columns and with half a step of the wider kernel at the end (needs a B200): every pitch gives the same bits, nothing beyond the columns is touched, and the values are
 those of the float64 product within the tolerance of tests/test_gpu_spmm.py."""
 import numpy as np
 import pytest
@@ -9,7 +9,7 @@ from paper_2607_08786_b200 import build, tl3, workloads as wl
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("N", [1, 5, 8, 15, 17, 24, 31, 33, 40, 56, 63, 64])
+@pytest.mark.parametrize("N", [1, 5, 8, 15, 17, 24, 31, 33, 40, 56, 63, 64, 72, 136])
 @pytest.mark.parametrize("M,K", [(1100, 500), (130, 1300)])
 def test_every_pitch(oracle_mod, M, K, N):
     import torch
