@@ -71,7 +71,7 @@ struct KernelArgs {
   const __half* bias;        // per output row, added before the activation (null: none)
   int act;                   // TL3_ACT_*
   float* partials;           // [2 * gridDim.x][n_pad][128]
-  unsigned int* flags;       // [2 * gridDim.x] one per partial-sum slot: 1 = written and not yet collected
+  unsigned int* flags;       // [2 * gridDim.x] one per slot (2 * CTA): 1 = written and not yet collected
   unsigned int* status;      // status word
   uint32_t stage_stride;     // bytes per stage (block area + X tile), multiple of 1024
   uint32_t x_offset;         // offset of the X tile inside a stage, multiple of 1024
@@ -485,7 +485,8 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
         }
       };
       const uint32_t acc_tmem = tmem_base + lane_base + static_cast<uint32_t>(b * NPAD);
-      // partial sums of a shared row-tile: slot 2*cta + (this row-tile is not the first one of my range)
+      // partial sums of a shared row-tile: slot 2*cta + (this row-tile is not the first one of my range).  (Only
+      // a CTA that begins inside a row-tile hands a partial sum on, so the slots in use are the even ones.)
       const int slot = 2 * blockIdx.x + (t_begin < row_tile_begin ? 1 : 0);
       float* mine = a.partials + static_cast<size_t>(slot) * NPAD * 128 + et;
       if (reducer) {
@@ -557,9 +558,7 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
             uint32_t v[CH];
             TmemLd<CH>::ld(acc_tmem + c0, v);
             tmem_wait_ld<CH>(v);
-            // own part first (lowest CTA), then the others in ascending order.  Two loops: in one
-            // loop the slot arithmetic of the unstaged case (a 64-bit division per contributor)
-            // was computed on the staged path too, 0.25 us on a reducer's way out.
+            // own part first (lowest CTA), then the others in ascending order
             if (staged) {
               uint32_t p = smem_base + static_cast<uint32_t>(et) * 4u + static_cast<uint32_t>(c0) * 512u;
               for (int k = 0; k < n_others; ++k, p += NPAD * 512u) {
@@ -570,12 +569,17 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
                 for (int c = 0; c < CH; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) + __uint_as_float(w[c]));
               }
             } else {
-              for (int k = 0; k < n_others; ++k) {
-                const int c_id = c_first + 1 + k;
-                const int sl = 2 * c_id + (range_begin(c_id, T, G) < row_tile_begin ? 1 : 0);
-                const float* p = a.partials + static_cast<size_t>(sl) * NPAD * 128 + et;
+              // The contributors' slots are the even ones (a division for each of them, to tell, stood
+              // between the loads; 700 x 6000, N = 16, 25 CTAs per row-tile, 13.8 -> 11.4 us, 128 x 20480, N = 16, 148 of them,
+              // 49 -> 39.5).
+              // (16 columns: one pointer that moves on.  With 32 in hand that costs the staged sums above as much as
+              // it saves here, 1024 x 1024, N = 32 6.1 -> 6.5: there the address is formed anew.)
+              auto at = [&](int k) { return a.partials + static_cast<size_t>(2 * (c_first + 1 + k)) * NPAD * 128 + c0 * 128 + et; };
+              const float* p = at(0);
+              for (int k = 0; k < n_others; ++k, p += 2 * NPAD * 128) {
+                if constexpr (NPAD > 16) p = at(k);
 #pragma unroll
-                for (int c = 0; c < CH; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) + __ldcg(p + (c0 + c) * 128));
+                for (int c = 0; c < CH; ++c) v[c] = __float_as_uint(__uint_as_float(v[c]) + __ldcg(p + c * 128));
               }
             }
             store_y(v, c0);

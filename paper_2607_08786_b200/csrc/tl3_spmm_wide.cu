@@ -186,8 +186,8 @@ template <bool XT, int S, bool kShared>
 __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t acc_tmem, int et, uint32_t vrow, int c_begin, int c_step, int n_others,
                                            uint32_t turn) {
   constexpr int CH = 16;
-  const int n_pad = a.n_pad[less];
-  const uint32_t chunks = a.chunks[less];
+  const int n_pad = S == 1 ? a.n_pad[0] : a.n_pad[less];
+  const uint32_t chunks = S == 1 ? a.chunks[0] : a.chunks[less];
   const int row = static_cast<int>(S * (vrow / chunks) + blockIdx.x % S) * kTileM + et;
   const int n0 = static_cast<int>(vrow % chunks) * n_pad;
   const int cols = a.N - n0 < n_pad ? a.N - n0 : n_pad;
