@@ -21,8 +21,8 @@ static void run_parallel(int64_t n, unsigned most, const F& f) {
   auto worker = [&]() {
     for (int64_t i = next.fetch_add(1); i < n; i = next.fetch_add(1)) f(i);
   };
-  const unsigned hw = std::thread::hardware_concurrency();
-  const int64_t threads = std::min<int64_t>(std::min<int64_t>(hw ? hw : 1, most), n);
+  int64_t threads = std::min<int64_t>(most, n);
+  if (threads > 1) threads = std::min<int64_t>(threads, std::max(1u, std::thread::hardware_concurrency()));   // (asking takes 2 us)
   std::vector<std::thread> pool;
   try {
     for (int64_t t = 1; t < threads; ++t) pool.emplace_back(worker);

@@ -207,13 +207,17 @@ class Matrix:
     @classmethod
     def deserialize(cls, data: bytes) -> "Matrix":
         h = ctypes.c_void_p()
-        try:
-            buf = np.frombuffer(data, dtype=np.uint8)              # the library copies what it keeps
-            address = buf.ctypes.data
-        except (TypeError, ValueError):
-            buf = (ctypes.c_char * len(data)).from_buffer_copy(data)
-            address = ctypes.addressof(buf)
-        _check(lib().tl3_deserialize(address, len(data), ctypes.byref(h)), "tl3_deserialize")
+        # read where it lies (the library copies what it keeps): bytes, else a writable buffer, else any other
+        source = data
+        if type(data) is not bytes:
+            try:
+                source = (ctypes.c_char * len(data)).from_buffer(data)
+            except (TypeError, ValueError):
+                try:
+                    source = np.frombuffer(data, dtype=np.uint8).ctypes.data_as(ctypes.c_void_p)
+                except (TypeError, ValueError):
+                    source = (ctypes.c_char * len(data)).from_buffer_copy(data)
+        _check(lib().tl3_deserialize(source, len(data), ctypes.byref(h)), "tl3_deserialize")
         return cls(h.value)
 
     def close(self) -> None:
@@ -265,7 +269,7 @@ class Matrix:
         _check(fn(self._h, None, ctypes.byref(n)), "tl3_serialize")
         # the library writes into the bytes object itself
         data = _new_bytes(None, n.value)
-        _check(fn(self._h, ctypes.cast(ctypes.c_char_p(data), ctypes.c_void_p), ctypes.byref(n)), "tl3_serialize")
+        _check(fn(self._h, data, ctypes.byref(n)), "tl3_serialize")
         return data[:n.value]
 
     # -- device side -------------------------------------------------------------------------
