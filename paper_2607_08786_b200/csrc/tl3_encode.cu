@@ -466,10 +466,17 @@ static int encode_device_impl(const void* dW, int64_t M, int64_t K, int64_t ldw,
   // sparsity; only a matrix that needs more has them allocated when their sizes are known.
   const size_t o_vals = 0, o_meta = o_vals + up(n_vals * 2), o_tau = o_meta + up(n_meta), o_rho = o_tau + up(n_chain * 2),
                o_len = o_rho + up(n_chain * 2), o_dir = o_len + up(n_chain), o_stats = o_dir + up(n_dir * 4), o_pack = o_stats + 256,
-               o_var = o_pack + up(pack_scratch_bytes(m->n_tiles)), guess = static_cast<size_t>(m->n_tiles) * 10240, total = o_var + guess;
+               o_var = o_pack + up(pack_scratch_bytes(m->n_tiles));
+  size_t guess = static_cast<size_t>(m->n_tiles) * 10240;
   EncodeArgs a{};
   {
-    TL3_ENC_CUDA(cudaMalloc(reinterpret_cast<void**>(&scratch), total));
+    cudaError_t got = cudaMalloc(reinterpret_cast<void**>(&scratch), o_var + guess);
+    if (got == cudaErrorMemoryAllocation) {                         // a device that is nearly full: without the guess, which is twice
+      cudaGetLastError();                                           // to five times what a matrix needs
+      guess = 0;
+      got = cudaMalloc(reinterpret_cast<void**>(&scratch), o_var);
+    }
+    TL3_ENC_CUDA(got);
     TL3_ENC_CUDA(cudaMemsetAsync(scratch + o_stats, 0, 256, st));
     a.W = static_cast<const uint16_t*>(dW);
     a.M = M; a.K = K; a.ldw = ldw; a.K_pad = m->K_pad; a.tiles_k = static_cast<int>(m->tiles_k);

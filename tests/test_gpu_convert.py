@@ -55,3 +55,28 @@ def test_conversion_of_awkward_sources(tl3, W, pitch, shift):
     only = tl3.Matrix.encode_on_device(src, device_only=True)
     assert np.array_equal(only.upload_packed_on_device().cpu().numpy(), want)
     assert only.stats()["canonical_bytes"] == ref.stats()["canonical_bytes"]
+
+
+def test_conversion_on_a_nearly_full_device(tl3):
+    """Room for the container, its bytes and entries as they are, but not for the allocation that serves any
+    matrix down to 40 % sparsity at once (29 KB per tile)."""
+    import torch
+    W = torch.from_numpy(_random(8192, 4096, 0.5)).cuda()
+    tiles, MB = 64 * 32, 1 << 20
+    ref = tl3.Matrix.encode_on_device(W, device_only=True)
+    want = ref.upload_packed_on_device().clone()
+    blob = torch.empty_like(want)
+    ref.close()
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    room = 52 * MB
+    assert 19200 * tiles + 5 * MB < room < 29000 * tiles
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8, device="cuda")
+    assert abs(torch.cuda.mem_get_info()[0] - room) <= 3 * MB
+    m = tl3.Matrix.encode_on_device(W, device_only=True)
+    stream = torch.cuda.current_stream().cuda_stream
+    assert m.device_bytes() == want.numel()
+    assert tl3.lib().tl3_upload_device(m._h, blob.data_ptr(), stream) == tl3.OK
+    del filler
+    torch.cuda.empty_cache()
+    assert torch.equal(blob, want)
