@@ -25,7 +25,6 @@
 // walked by a thread per row, 57 + 89 us.
 #include <cuda_runtime.h>
 
-#include <atomic>
 #include <cstdint>
 #include <new>
 #include <vector>
@@ -414,15 +413,10 @@ tl3_encode_scan_kernel(uint32_t* tile_dir, long long n_tiles, unsigned long long
 
 namespace tl3 {
 namespace {
-// More than 48 KB of dynamic shared memory is opted into once per device (a repeated call sets the same value).
+// More than 48 KB of dynamic shared memory is opted into.  On every call, like the packer's (a microsecond
+// of a millisecond): an opt-in that is remembered per device does not outlive a cudaDeviceReset().
 cudaError_t configure_encode_kernel() {
-  static std::atomic<bool> done[64] = {};
-  int dev = 0;
-  if (cudaError_t e = cudaGetDevice(&dev)) return e;
-  if (dev < 64 && done[dev].load(std::memory_order_acquire)) return cudaSuccess;
-  if (cudaError_t e = cudaFuncSetAttribute(tl3_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(EncodeSmem)))) return e;
-  if (dev < 64) done[dev].store(true, std::memory_order_release);
-  return cudaSuccess;
+  return cudaFuncSetAttribute(tl3_encode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(EncodeSmem)));
 }
 
 void release_encoded(void* p) {

@@ -15,6 +15,7 @@
 // What bounds it is the latency of a tile's serial steps (the chains), hidden by three tiles per SM.
 // With two-byte copies, a thread per 64 coordinates tested one by one and one thread sharing out the
 // banks, the two passes took 181 + 247 us on 5120 x 5120 at 50 % sparsity; now 57 + 77 us.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -389,26 +390,69 @@ struct HostPiece {
   size_t bytes;
 };
 
+// The pinned memory of copy_from_host(): 6 MB that stay between calls (pinning them costs more than a copy
+// of 100 MB) until tl3_trim(), for one caller at a time.  Somebody's cudaDeviceReset() takes such memory
+// away, and its address may then be another allocation's: what is kept is used only while the driver
+// still knows it by the number that it gave it.
+constexpr int kRingSlots = 6;
+constexpr size_t kRingSlotBytes = size_t{1} << 20;
+
+template <class Fn> Fn driver_entry(const char* name) {
+  void* f = nullptr;
+  cudaDriverEntryPointQueryResult q;
+  if (cudaGetDriverEntryPoint(name, &f, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) return nullptr;
+  return reinterpret_cast<Fn>(f);
+}
+
+unsigned long long buffer_id(const void* p) {                    // 0: not an allocation of the driver's
+  static const auto fn = driver_entry<CUresult (*)(void*, CUpointer_attribute, CUdeviceptr)>("cuPointerGetAttribute");
+  unsigned long long id = 0;
+  if (!fn || !p || fn(&id, CU_POINTER_ATTRIBUTE_BUFFER_ID, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return 0;
+  return id;
+}
+
+struct PinnedRing {
+  std::mutex mu;
+  uint8_t* base = nullptr;
+  unsigned long long id = 0;
+
+  uint8_t* get() {                                               // (mu held) the memory, or null
+    if (base && buffer_id(base) == id) return base;
+    void* p = nullptr;
+    base = nullptr;
+    if (cudaHostAlloc(&p, kRingSlots * kRingSlotBytes, cudaHostAllocPortable) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    id = buffer_id(p);
+    if (id == 0) { cudaFreeHost(p); return nullptr; }
+    return base = static_cast<uint8_t*>(p);
+  }
+  cudaError_t release() {                                        // (mu held)
+    const bool there = base && buffer_id(base) == id;
+    uint8_t* p = base;
+    base = nullptr;
+    return there ? cudaFreeHost(p) : cudaSuccess;
+  }
+};
+PinnedRing& ring_of_process() {
+  static PinnedRing* r = new PinnedRing();                       // (never destroyed: a thread may still copy while the process exits)
+  return *r;
+}
+
 // Pageable host memory to the device, complete on return.  The runtime's own copy moves 11 GB/s, one
-// thread of its filling one staging buffer; here six threads fill a pinned megabyte each (6 MB kept for
-// the life of the process: pinning it costs more than a copy of 100 MB; one caller at a time uses it,
-// another one that comes meanwhile takes the runtime's way).  132 MB: 12.2 -> 5 ms.
+// thread of its filling one staging buffer; here six threads fill a pinned megabyte each (one caller at a
+// time; another one that comes meanwhile takes the runtime's way).  132 MB: 12.2 -> 5 ms.
 cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st) {
-  constexpr int kSlots = 6;
-  constexpr size_t kSlotBytes = size_t{1} << 20;
-  static std::mutex mu;
-  static uint8_t* ring = nullptr;
   size_t total = 0;
   for (const HostPiece& p : arrays) total += p.bytes;
-  std::unique_lock<std::mutex> lock(mu, std::defer_lock);
+  PinnedRing& pinned = ring_of_process();
+  std::unique_lock<std::mutex> lock(pinned.mu, std::defer_lock);
   cudaStream_t own = nullptr;
-  int dev = 0;
-  bool staged = total >= (size_t{8} << 20) && lock.try_lock() && cudaGetDevice(&dev) == cudaSuccess;
-  if (staged && !ring && cudaHostAlloc(reinterpret_cast<void**>(&ring), kSlots * kSlotBytes, cudaHostAllocPortable) != cudaSuccess) {
-    ring = nullptr;
-    staged = false;
-    cudaGetLastError();
-  }
+  // the caller's context, which need not be its device's primary one, for the threads
+  static const auto get_context = driver_entry<CUresult (*)(CUcontext*)>("cuCtxGetCurrent");
+  static const auto set_context = driver_entry<CUresult (*)(CUcontext)>("cuCtxSetCurrent");
+  CUcontext context = nullptr;
+  uint8_t* ring = nullptr;
+  bool staged = total >= (size_t{8} << 20) && get_context && set_context && lock.try_lock() && (ring = pinned.get()) != nullptr &&
+                get_context(&context) == CUDA_SUCCESS && context;
   // (a stream of its own: the caller's may be one that means another stream in another thread)
   if (staged && cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking) != cudaSuccess) { staged = false; cudaGetLastError(); }
   if (!staged) {
@@ -423,9 +467,9 @@ cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st
   std::atomic<size_t> next{0};
   std::atomic<int> failed{cudaSuccess};
   auto worker = [&](int slot) {
-    uint8_t* buf = ring + static_cast<size_t>(slot) * kSlotBytes;
+    uint8_t* buf = ring + static_cast<size_t>(slot) * kRingSlotBytes;
     cudaEvent_t done = nullptr;
-    cudaError_t e = cudaSetDevice(dev);
+    cudaError_t e = set_context(context) == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
     bool busy = false;
     while (e == cudaSuccess && failed.load(std::memory_order_relaxed) == cudaSuccess) {
@@ -444,10 +488,10 @@ cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st
   bool listed = false;
   try {
     for (const HostPiece& p : arrays)
-      for (size_t at = 0; at < p.bytes; at += kSlotBytes)
-        pieces.push_back({static_cast<uint8_t*>(p.dst) + at, static_cast<const uint8_t*>(p.src) + at, std::min(kSlotBytes, p.bytes - at)});
+      for (size_t at = 0; at < p.bytes; at += kRingSlotBytes)
+        pieces.push_back({static_cast<uint8_t*>(p.dst) + at, static_cast<const uint8_t*>(p.src) + at, std::min(kRingSlotBytes, p.bytes - at)});
     listed = true;
-    for (int t = 1; t < kSlots; ++t) pool.emplace_back(worker, t);
+    for (int t = 1; t < kRingSlots; ++t) pool.emplace_back(worker, t);
   } catch (const std::exception&) {                              // fewer threads, or no list at all
   }
   if (!listed) failed.store(cudaErrorMemoryAllocation);
@@ -514,12 +558,7 @@ int canon_to_device(tl3_matrix* m, cudaStream_t st, PackArgs* out) {
 }
 
 int configure_pack_kernel() {
-  static bool done[64] = {};
-  int dev = 0;
-  TL3_PK_CUDA(cudaGetDevice(&dev));
-  if (dev < 64 && done[dev]) return TL3_OK;
   TL3_PK_CUDA(cudaFuncSetAttribute(tl3_pack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(PackSmem))));
-  if (dev < 64) done[dev] = true;
   return TL3_OK;
 }
 
@@ -582,5 +621,13 @@ extern "C" int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream) {
   if (m->device_canon) { release_canon(m->device_canon); m->device_canon = nullptr; }
   if (e != cudaSuccess) { set_cuda_error(static_cast<int>(e)); return TL3_ERR_CUDA; }
   m->dptr = dptr;
+  return TL3_OK;
+}
+
+extern "C" int tl3_trim(void) {
+  using namespace tl3;
+  PinnedRing& pinned = ring_of_process();
+  std::lock_guard<std::mutex> lock(pinned.mu);                   // (waits for a copy under way)
+  TL3_PK_CUDA(pinned.release());
   return TL3_OK;
 }

@@ -29,7 +29,7 @@ _CANONICAL_DTYPES = (np.uint16, np.uint8, np.uint16, np.uint16, np.uint8, np.uin
                      np.uint16, np.uint16, np.uint32, np.uint16, np.uint8, np.uint32, np.uint16, np.uint8)
 
 # every symbol include/tl3.h declares
-SYMBOLS = ("tl3_encode", "tl3_encode_device", "tl3_encode_device_only", "tl3_decode", "tl3_canonical", "tl3_stats", "tl3_serialize", "tl3_serialize_compact", "tl3_deserialize",
+SYMBOLS = ("tl3_encode", "tl3_encode_device", "tl3_encode_device_only", "tl3_decode", "tl3_canonical", "tl3_stats", "tl3_serialize", "tl3_serialize_compact", "tl3_deserialize", "tl3_trim",
            "tl3_free", "tl3_device_bytes", "tl3_pack", "tl3_upload", "tl3_bind", "tl3_plan_device", "tl3_upload_device", "tl3_workspace_bytes", "tl3_workspace_init",
            "tl3_spmm", "tl3_spmm_ex", "tl3_spmm_nt", "tl3_spmm_host", "tl3_spmm_host_async", "tl3_spmm_static_scratch", "tl3_static_scratch_status", "tl3_status", "tl3_status_word", "tl3_selftest_bounded_wait", "tl3_last_launch", "tl3_strerror",
            "tl3_last_cuda_error", "tl3_get_tuning", "tl3_set_tuning")
@@ -423,6 +423,11 @@ class Matrix:
 
 def encode(W, **kw) -> Matrix:
     return Matrix.encode(W, **kw)
+
+
+def trim() -> None:
+    """Gives back the pinned host memory that the library keeps between uploads (``tl3_trim``)."""
+    _check(lib().tl3_trim(), "tl3_trim")
 
 
 def get_tuning() -> dict:
