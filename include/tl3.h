@@ -121,7 +121,9 @@ int tl3_encode_device(const void* dW, int64_t M, int64_t K, int64_t ldw, void* s
  * of the container; tl3_spmm*, tl3_bind, tl3_stats (layer counts; the sizes of the compact forms
  * read -1), tl3_workspace_bytes and tl3_free work as on any handle.  The calls that need the
  * container on the host -- tl3_decode, tl3_canonical, tl3_serialize*, tl3_pack, tl3_upload --
- * return UNSUPPORTED.  dW, ldw, stream, errors: as for tl3_encode_device. */
+ * return UNSUPPORTED.  Until it is packed the handle holds about 29 KB of device memory per tile whatever
+ * the sparsity (0.9 of W; 19 KB and what the container needs, where that is more or where the device has
+ * no more).  dW, ldw, stream, errors: as for tl3_encode_device. */
 int tl3_encode_device_only(const void* dW, int64_t M, int64_t K, int64_t ldw, void* stream, tl3_matrix** out);
 
 /* Decode back to dense: Algorithm 1 run on the host, then the 2:4 expansion and the Residual
@@ -209,7 +211,8 @@ int tl3_workspace_init(void* workspace, size_t bytes, void* stream);
  *   X: device, fp16, K x N row-major, leading dimension ldx >= N, ldx % 8 == 0, 16-byte aligned.
  *   Y: device, fp16, M x N row-major, leading dimension ldy >= N; fully overwritten.
  *   1 <= N <= TL3_MAX_N.  One kernel launch; W is streamed and decoded once for up to 64 columns (the
- *   decode phase), beyond that once for every 64 to 256 columns.  fp32 accumulation, fp16
+ *   decode phase), beyond that once for every 48 to 256 columns (tl3_last_pass()).  (A matrix of more than
+ *   2^32 / (SMs + 1) tiles times such groups is done in ceil(N / 64) launches.)  fp32 accumulation, fp16
  *   round-to-nearest-even output.  W and X are assumed finite (an empty slot multiplies an exact zero
  *   with an element of X).
  * Asynchronous on `stream`; allocates nothing; does not synchronise.  Calls that share a
@@ -295,15 +298,17 @@ int tl3_static_scratch_status(void* stream);
 int tl3_status(const tl3_matrix* m, void* workspace, void* stream);
 int tl3_status_word(void* workspace, void* stream, uint32_t* word);
 
-/* Self-test of the kernels' bounded waits (every wait inside the kernels gives up after 2 s,
- * records a code in the status word and lets the kernel return).  Enqueues a one-CTA kernel that
+/* Self-test of the kernels' bounded waits (every wait inside the kernels gives up after 2 s, one that
+ * sits behind others after 8 s, records a code in the status word and lets the kernel return).  Enqueues a one-CTA kernel that
  * waits on a barrier nothing ever arrives at; about 2 s after it starts, tl3_status() on the
  * same workspace reports DEVICE_TIMEOUT (code 1), the second word of the workspace holds 2
  * ("gave up"; 1 would mean the wait completed), and the device is usable as before.  Clear the
  * workspace with tl3_workspace_init() before using it for a product again. */
 int tl3_selftest_bounded_wait(void* workspace, void* stream);
 
-/* (No counterpart in the paper.)  Launch tuning, process-wide, read by every later tl3_spmm* call.
+/* (No counterpart in the paper.)  Launch tuning, process-wide, read by every later tl3_spmm* call that
+ * takes the kernel for up to 64 columns (the other one, for N > 64 and for 17 to 64 columns shared by many
+ * CTAs, has X in a ring of its own and never waits for it before it decodes).
  *   decode_before_x  launches with at most this many tiles per CTA decode a block as soon as it is
  *                    in shared memory instead of waiting for its X tile as well (X may come from the
  *                    kernel before, which the launch overlaps; the weights never do).  Measured on
@@ -319,6 +324,9 @@ int tl3_set_tuning(const tl3_tuning* t);
 
 /* Kernel launch geometry of the last tl3_spmm on this handle (for reporting): CTAs, stages. */
 int tl3_last_launch(const tl3_matrix* m, int* ctas, int* stages, int* smem_bytes);
+/* Its passes over W (for reporting): the columns of one, as planned for a workspace of this N; the CTAs that
+ * work on one as a cluster, 1 or 2; the accumulators that take turns. */
+int tl3_last_pass(const tl3_matrix* m, int* columns, int* cluster, int* accumulators);
 
 const char* tl3_strerror(int code);
 int tl3_last_cuda_error(void);      /* cudaError_t of the last failed runtime call, this thread */

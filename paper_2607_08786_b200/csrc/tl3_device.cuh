@@ -362,7 +362,7 @@ WorkspaceLayout workspace_layout(int N, int sm_count);
 constexpr int kWideColumns = 256;                               // most columns of one pass over W
 constexpr int kRoomUnit = 16;                                   // unit of the workspace's record of its size, in columns per CTA
 int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t ldy, int N, const tl3_epilogue* ep, bool xt,
-              void* workspace, void* stream);                   // kWideNoPlan: blocks too large for it
+              void* workspace, void* stream);                   // kWideNoPlan: blocks too large for it, or 2^32 / (CTAs + 1) tiles and more
 
 constexpr int kWideNoPlan = 1;
 

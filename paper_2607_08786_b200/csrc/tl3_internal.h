@@ -101,6 +101,7 @@ struct tl3_matrix {
 
   // last launch geometry (reporting only)
   mutable std::atomic<int> last_ctas{0}, last_stages{0}, last_smem{0};
+  mutable std::atomic<int> last_pass{0};    // columns | CTAs of a cluster << 16 | accumulators << 24
 };
 
 namespace tl3 {

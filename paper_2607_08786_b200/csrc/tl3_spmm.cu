@@ -911,9 +911,11 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   // (us here / there: 1024 x 1024, N = 64 15.3 / 9.4; 4096 x 4096, N = 64 17.4 / 14.3; 1024 x 4096, N = 32 16.9 /
   // 13.4; staged: 5120 x 5120, N = 64 14.9 / 17.0; 2000 x 8000, N = 32 11.2 / 14.5.  8 KB slots: 700 x 24000, N = 16,
   // 27 CTAs per row-tile, 18.2 / 19.4.)
-  // Blocks so large that fewer stages than decode groups fit go there from six CTAs per row-tile on, at N > 32
-  // (1024 x 1024 at 40 %, N = 64 15.4 / 9.4); below that the gain is smaller (4096 x 2048 at 40 %, N = 64, five
-  // CTAs, 14.9 / 12.3; 2048 x 2048 dense, N = 32 14.1 / 12.7) and this kernel keeps its case of a short ring.
+  // Blocks so large that fewer stages than decode groups fit go there only from six CTAs per row-tile on and at
+  // N > 32 (1024 x 1024 at 40 %, N = 64 15.4 / 9.4).  That is not where the two are level: below it the other
+  // kernel is the faster one as well (4096 x 2048 at 40 %, N = 64, five CTAs, 14.9 / 12.3; 2048 x 2048 dense,
+  // N = 32 14.1 / 12.7).  Those launches stay because they are what runs a ring of two or three stages round
+  // many times, here and in the tests; moving the line is worth 10 to 17 % to them.
   if (n_pad > 16) {
     const unsigned long long sharing = (static_cast<unsigned long long>(m->tiles_k) * grid + total - 1) / total;   // CTAs per row-tile
     const unsigned long long staging = static_cast<unsigned long long>(stages) * stage_stride;
@@ -956,6 +958,7 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   args.timing = nullptr;
 #endif
   m->last_ctas = grid; m->last_stages = stages; m->last_smem = static_cast<int>(smem_bytes);
+  m->last_pass.store(n_pad | 1 << 16 | 2 << 24, std::memory_order_relaxed);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (xt) {
     switch (n_pad) {
@@ -988,8 +991,10 @@ int tl3_spmm_ex(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_
     const int rc = tl3::spmm_wide(m, X, ldx, Y, ldy, N, ep, false, workspace, stream);
     if (rc != tl3::kWideNoPlan) return rc;
   }
-  // One launch of up to 64 columns; a wider product gets here only with blocks so large that the wide
-  // kernel's buffers do not fit beside them.
+  // One launch of up to 64 columns.  A wider product gets here only where tiles times column groups are more
+  // than the wide kernel's 32-bit split takes (28.8 million on 148 SMs; 64 columns of it may then still be
+  // fewer), or with blocks that no encoder makes (more Residual entries than a tile has windows), which are
+  // refused below, too.
   for (int n0 = 0; n0 < N; n0 += 64) {
     const int nb = N - n0 < 64 ? N - n0 : 64;
     const int rc = spmm_block(m, static_cast<const uint16_t*>(X) + n0, ldx, static_cast<uint16_t*>(Y) + n0, ldy, nb, ep, false, workspace, stream);
@@ -1117,6 +1122,15 @@ int tl3_last_launch(const tl3_matrix* m, int* ctas, int* stages, int* smem_bytes
   if (ctas) *ctas = m->last_ctas;
   if (stages) *stages = m->last_stages;
   if (smem_bytes) *smem_bytes = m->last_smem;
+  return TL3_OK;
+}
+
+int tl3_last_pass(const tl3_matrix* m, int* columns, int* cluster, int* accumulators) {
+  if (!m) return TL3_ERR_INVALID_ARG;
+  const int p = m->last_pass.load(std::memory_order_relaxed);
+  if (columns) *columns = p & 0xFFFF;
+  if (cluster) *cluster = (p >> 16) & 0xFF;
+  if (accumulators) *accumulators = p >> 24;
   return TL3_OK;
 }
 

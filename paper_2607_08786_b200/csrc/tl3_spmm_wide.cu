@@ -744,7 +744,7 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
     }
     a.n_w = blocks();
     if (a.n_w > kMaxRing) a.n_w = kMaxRing;
-    if (a.n_w < a.n_wr) return kWideNoPlan;
+    if (a.n_w < a.n_wr) return kWideNoPlan;                       // (blocks of more Residual entries than a tile has windows: none that an encoder makes)
   }
   const uint32_t smem_bytes = a.n_w * a.block_area + a.n_x * a.x_bytes + a.n_wr * kWrBytes + kSlack;
 
@@ -784,6 +784,7 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   a.status = reinterpret_cast<unsigned int*>(ws + wl.status_off);
   a.room = ws + wl.room_off;
   m->last_ctas = grid; m->last_stages = a.n_w; m->last_smem = static_cast<int>(smem_bytes);
+  m->last_pass.store(n_pad | S << 16 | a.n_acc << 24, std::memory_order_relaxed);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (S == 2) return xt ? launch_wide<true, 2>(map, a, grid, smem_bytes, st) : launch_wide<false, 2>(map, a, grid, smem_bytes, st);
   return xt ? launch_wide<true, 1>(map, a, grid, smem_bytes, st) : launch_wide<false, 1>(map, a, grid, smem_bytes, st);

@@ -31,7 +31,7 @@ _CANONICAL_DTYPES = (np.uint16, np.uint8, np.uint16, np.uint16, np.uint8, np.uin
 # every symbol include/tl3.h declares
 SYMBOLS = ("tl3_encode", "tl3_encode_device", "tl3_encode_device_only", "tl3_decode", "tl3_canonical", "tl3_stats", "tl3_serialize", "tl3_serialize_compact", "tl3_deserialize", "tl3_trim",
            "tl3_free", "tl3_device_bytes", "tl3_pack", "tl3_upload", "tl3_bind", "tl3_plan_device", "tl3_upload_device", "tl3_workspace_bytes", "tl3_workspace_init",
-           "tl3_spmm", "tl3_spmm_ex", "tl3_spmm_nt", "tl3_spmm_host", "tl3_spmm_host_async", "tl3_spmm_static_scratch", "tl3_static_scratch_status", "tl3_status", "tl3_status_word", "tl3_selftest_bounded_wait", "tl3_last_launch", "tl3_strerror",
+           "tl3_spmm", "tl3_spmm_ex", "tl3_spmm_nt", "tl3_spmm_host", "tl3_spmm_host_async", "tl3_spmm_static_scratch", "tl3_static_scratch_status", "tl3_status", "tl3_status_word", "tl3_selftest_bounded_wait", "tl3_last_launch", "tl3_last_pass", "tl3_strerror",
            "tl3_last_cuda_error", "tl3_get_tuning", "tl3_set_tuning")
 
 
@@ -113,6 +113,8 @@ def lib() -> ctypes.CDLL:
         L.tl3_status_word.argtypes = [vp, vp, ctypes.POINTER(ctypes.c_uint32)]
         L.tl3_selftest_bounded_wait.argtypes = [vp, vp]
         L.tl3_last_launch.argtypes = [vp, ctypes.POINTER(ci), ctypes.POINTER(ci), ctypes.POINTER(ci)]
+        L.tl3_last_pass.argtypes = [vp, ctypes.POINTER(ci), ctypes.POINTER(ci), ctypes.POINTER(ci)]
+        L.tl3_trim.argtypes = []
         L.tl3_strerror.argtypes = [ci]
         L.tl3_strerror.restype = ctypes.c_char_p
         L.tl3_last_cuda_error.argtypes = []
@@ -419,6 +421,11 @@ class Matrix:
         c, s, b = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
         _check(lib().tl3_last_launch(self._h, ctypes.byref(c), ctypes.byref(s), ctypes.byref(b)), "tl3_last_launch")
         return {"ctas": c.value, "stages": s.value, "smem_bytes": b.value}
+
+    def last_pass(self) -> dict:
+        c, s, a = ctypes.c_int(), ctypes.c_int(), ctypes.c_int()
+        _check(lib().tl3_last_pass(self._h, ctypes.byref(c), ctypes.byref(s), ctypes.byref(a)), "tl3_last_pass")
+        return {"columns": c.value, "cluster": s.value, "accumulators": a.value}
 
 
 def encode(W, **kw) -> Matrix:
