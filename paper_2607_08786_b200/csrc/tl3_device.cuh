@@ -193,8 +193,9 @@ static __device__ __noinline__ float4 activate4(float4 v, float bias, int act) {
   return make_float4(x[0], x[1], x[2], x[3]);
 }
 
-// Epilogue of tl3_spmm_ex for the first `cols` of n sums of a row (what lies beyond may change or not):
-// bias and ReLU in place, the functions by call.
+// Epilogue of tl3_spmm_ex for the first `cols` of n sums of a row (what lies beyond may change or not; 0 for a
+// row that is not stored: its zeros would take the slow way through SiLU's division): bias and ReLU in
+// place, the functions by call.
 template <int n>
 __device__ __forceinline__ void apply_epilogue(uint32_t* v, float bias, int act, int cols) {
   if (act <= TL3_ACT_RELU) {

@@ -439,7 +439,7 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
       auto store_y = [&](uint32_t* v, int c0) {                 // (bias, activation,) fp32 -> fp16 (round to nearest even) -> Y
         // (bias and ReLU in place: as calls, one per column, they took 1-3 us of a launch's tail -- 5120 x
         // 5120, N = 32 with a bias 14.8 -> 12.8, 4096 x 4096, N = 1 11.1 -> 10.1)
-        if (!plain) apply_epilogue<CH>(v, bias_v, a.act, a.N - c0);   // one test per call, not one per element
+        if (!plain) apply_epilogue<CH>(v, bias_v, a.act, row < a.M ? a.N - c0 : 0);   // one test per call, not one per element
         if constexpr (XT) {
           if (row >= a.M) return;
           __half* yc = y + static_cast<long long>(c0) * a.ldy;          // column c0 of this row: Yt[c0][row]

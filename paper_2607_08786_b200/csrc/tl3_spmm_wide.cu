@@ -227,7 +227,7 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
         }
       }
     }
-    if (!plain) apply_epilogue<CH>(v, bias, a.act, cols - c0);
+    if (!plain) apply_epilogue<CH>(v, bias, a.act, row < a.M ? cols - c0 : 0);
     uint32_t o[CH / 2];
 #pragma unroll
     for (int c = 0; c < CH / 2; ++c) {
