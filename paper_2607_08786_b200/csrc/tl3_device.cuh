@@ -259,7 +259,7 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t* v) {
 // refuses matrices with (G + 1) * T >= 2^32 (hundreds of gigabytes), and a 64-bit division costs a
 // CTA 0.15 us each at its cold start, where there are three of them.
 __device__ __forceinline__ uint32_t range_begin(uint32_t c, uint32_t T, uint32_t G) { return c * T / G; }
-__device__ __forceinline__ int owner_of(uint32_t t, uint32_t T, uint32_t G) { return static_cast<int>(((t + 1u) * G - 1u) / T); }
+__host__ __device__ __forceinline__ int owner_of(uint32_t t, uint32_t T, uint32_t G) { return static_cast<int>(((t + 1u) * G - 1u) / T); }
 
 __device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
   uint32_t v;

@@ -918,8 +918,17 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   // many times, here and in the tests; moving the line is worth 10 to 17 % to them.
   if (n_pad > 16) {
     const unsigned long long sharing = (static_cast<unsigned long long>(m->tiles_k) * grid + total - 1) / total;   // CTAs per row-tile
-    const unsigned long long staging = static_cast<unsigned long long>(stages) * stage_stride;
-    const bool unstaged = sharing * (n_pad * 512ull) > (n_pad == 32 ? staging + staging / 4 : staging);
+    const unsigned long long staging = static_cast<unsigned long long>(stages) * stage_stride, slot = n_pad * 512ull;
+    bool unstaged = sharing * slot > (n_pad == 32 ? staging + staging / 4 : staging);
+    if (unstaged && (sharing - 1) * slot <= staging) {
+      // Just above: the reducer is one of the CTAs that share a row-tile, so it is unstaged only if a row-tile
+      // has `sharing` others (4608 x 1024, N = 64, four others where four fit, 8.8 / 9.8; 4096 x 4096, five,
+      // 17.4 / 14.3).
+      unstaged = false;
+      const uint32_t T = static_cast<uint32_t>(total), TK = static_cast<uint32_t>(m->tiles_k), G = static_cast<uint32_t>(grid);
+      for (uint32_t t = 0; t < T && !unstaged; t += TK)
+        unstaged = static_cast<unsigned long long>(owner_of(t + TK - 1, T, G) - owner_of(t, T, G)) >= sharing;
+    }
     if (unstaged && (stages >= kGroups || (n_pad == 64 && sharing > 5))) {
       const int rc = spmm_wide(m, X, ldx, Y, ldy, N, ep, xt, workspace, stream);
       if (rc != kWideNoPlan) return rc;

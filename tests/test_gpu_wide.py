@@ -210,3 +210,30 @@ def test_a_workspace_for_fewer_columns_still_serves_wide_products(tl3):
     for got in (Y, Yt.T):                                   # other split of K: fp32 sums in another order, one rounding
         assert (got - want).abs().max() <= 2.0**-9 * want.abs().max()
     assert m.status(ws) == tl3.OK
+
+
+@pytest.mark.parametrize("M,K,others", [(4608, 1024, 4), (4600, 1000, 4), (4096, 768, 4), (4096, 1024, 4), (4608, 4096, 4), (4096, 4096, 5), (3584, 2048, 5), (3328, 2048, 6),
+                                        (1024, 1024, 7), (5120, 5120, 4)])
+@pytest.mark.parametrize("N", [33, 64])
+def test_where_the_kernels_meet(tl3, M, K, others, N):
+    """With four stages at 64 columns and 50 % sparsity, four partial sums besides the reducer's own fit
+    them: then the product stays with the other kernel (four stages), from five on it comes here."""
+    import torch
+    tiles_m, tiles_k = -(-M // 128), -(-K // 128)
+    T = tiles_m * tiles_k
+    G = min(T, torch.cuda.get_device_properties(0).multi_processor_count)
+    owner = [((t + 1) * G - 1) // T for t in range(T)]
+    assert max(owner[(r + 1) * tiles_k - 1] - owner[r * tiles_k] for r in range(tiles_m)) == others
+    case = wl.Case(0, "meet", M, K, N, 5, 0.5, "magnitude")
+    W, X = case.make_W(), case.make_X()
+    m = tl3.Matrix.encode_on_device(torch.from_numpy(W).cuda(), device_only=True)
+    m.upload_packed_on_device()
+    Xt = torch.zeros((N, (K + 7) // 8 * 8), dtype=torch.float16, device="cuda")
+    Xt[:, :K] = torch.from_numpy(np.ascontiguousarray(X.T))
+    Xd = torch.zeros((K, 64), dtype=torch.float16, device="cuda")
+    Xd[:, :N] = Xt[:, :K].T
+    Y = m.spmm(Xd[:, :N])
+    assert (m.last_launch()["stages"] == 4) == (others <= 4), m.last_launch()
+    Yt = m.spmm_nt(Xt[:, :K])
+    _check_linear(W, Xt[:, :K], None, None, Yt, 9)
+    _check_linear(W, Xt[:, :K], None, None, Y.T, 9)
