@@ -290,6 +290,14 @@ bool consistent(const tl3_matrix& m) {
 
 }  // namespace
 
+namespace tl3 {
+tl3_matrix* new_device_matrix(int64_t M, int64_t K) {
+  tl3_matrix* m = new (std::nothrow) tl3_matrix();
+  if (m) set_shape(*m, M, K, tl3_params{kTileM, kTileK, 15});
+  return m;
+}
+}  // namespace tl3
+
 extern "C" {
 
 int tl3_encode(const uint16_t* W, int64_t M, int64_t K, const tl3_params* params, tl3_matrix** out) {

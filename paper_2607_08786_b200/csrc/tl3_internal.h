@@ -106,8 +106,11 @@ struct tl3_matrix {
 
 namespace tl3 {
 
-// The canonical arrays on the device (between an encode or a copy there and tl3_upload_device).
+// What tl3_upload_device packs: the canonical arrays on the device, or (tl3_encode_device_only) the blocks
+// themselves in the order in which they were finished.
 struct DeviceCanon {
+  const uint8_t* image;                      // null: the arrays
+  const unsigned long long* where;           // per tile: its block in `image`
   const uint16_t* tc_vals; const uint8_t* tc_meta; const uint16_t* chain_tau0; const uint16_t* chain_rho0;
   const uint8_t* chain_len; const uint8_t* pdd_bytes; const uint32_t* tile_dir; const uint16_t* res_rho; const uint16_t* res_val;
   void* pack_scratch;                        // pack_scratch_bytes(): sizes of the packed blocks, then their offsets
@@ -150,6 +153,7 @@ struct DirEntry {
 
 size_t plan_device_layout(const tl3_matrix* m);           // fills device_bytes, offsets, max block (once, thread-safe)
 void pack_device_blob(const tl3_matrix* m, uint8_t* out); // out: device_bytes bytes, host
+tl3_matrix* new_device_matrix(int64_t M, int64_t K);      // 128 x 128 tiles, nothing in it; null: no memory
 void set_device_layout(const tl3_matrix* m, const uint32_t* sizes);   // layout from per-tile sizes computed on the GPU
 // (block_off: one entry per tile, and the end of the last block)
 void blob_header_and_offsets(const tl3_matrix* m, uint8_t* header256, std::vector<unsigned long long>* block_off);
