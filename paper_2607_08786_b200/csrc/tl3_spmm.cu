@@ -741,6 +741,48 @@ static const void* pinned_address(const void* p, size_t bytes) {
   return reinterpret_cast<const void*>(dev);
 }
 
+// Bytes between device memory and pinned host memory, 16 per thread and the last ones singly.
+__global__ void __launch_bounds__(256)
+tl3_copy_kernel(const uint8_t* src, uint8_t* dst, size_t bytes) {   // (not __restrict__: no load may move in front of the wait)
+  pdl_launch_dependents();                                         // (a product behind it waits before it reads X)
+  pdl_wait();                                                      // (Y may be the kernel's before this one)
+  const size_t at = (static_cast<size_t>(blockIdx.x) * blockDim.x + threadIdx.x) * 16;
+  if (at + 16 <= bytes) {
+    *reinterpret_cast<uint4*>(dst + at) = *reinterpret_cast<const uint4*>(src + at);
+  } else {
+    for (size_t i = at; i < bytes; ++i) dst[i] = src[i];
+  }
+}
+
+// X to the device or Y to the host.  The copy engine takes 3 to 5 us to begin and to report; a kernel begins while the
+// product still runs, its threads wait for it.  Both by a kernel, whole calls with pinned buffers: 1024 x 1024, N = 8
+// 34.0 -> 26.3 us; 4096 x 4096, N = 16 45.5 -> 34.7, N = 64 62.8 -> 57.0; 8192 x 4096, N = 61 (Y 1.0 MB) 71.2 -> 68.0.
+// Beyond a megabyte the copy is what takes the time and the engine is as good (Y of 1.3 MB 59.2 and 59.8, of
+// 2.6 MB 88.1 and 91.1), so the SMs are left to the products of other streams.
+constexpr size_t kCopyByKernel = size_t{1} << 20;
+static int copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, cudaStream_t stream) {
+  const bool up = kind == cudaMemcpyHostToDevice;
+  const void* device = up ? dst : src;
+  if (bytes <= kCopyByKernel && (reinterpret_cast<uintptr_t>(device) & 15) == 0) {
+    if (const void* host = pinned_address(up ? src : dst, bytes)) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(static_cast<unsigned>((bytes + 4095) / 4096));
+      cfg.blockDim = dim3(256);
+      cfg.stream = stream;
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      attr[0].val.programmaticStreamSerializationAllowed = 1;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_copy_kernel, static_cast<const uint8_t*>(up ? host : src),
+                                  static_cast<uint8_t*>(up ? dst : const_cast<void*>(host)), bytes));
+      return TL3_OK;
+    }
+  }
+  TL3_CUDA(cudaMemcpyAsync(dst, src, bytes, kind, stream));
+  return TL3_OK;
+}
+
 // Process-wide launch tuning (tl3_set_tuning); the default is what measured best on B200.
 static std::atomic<int> g_decode_before_x{TL3_DEFAULT_DECODE_BEFORE_X};
 
@@ -1042,7 +1084,7 @@ int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int
   const int64_t ldx = (N + 7) / 8 * 8;
   const size_t x_bytes = static_cast<size_t>(m->K) * N * 2;
   if (ldx == N) {
-    TL3_CUDA(cudaMemcpyAsync(dX, X, x_bytes, cudaMemcpyHostToDevice, st));
+    if (int rc = tl3::copy_host(dX, X, x_bytes, cudaMemcpyHostToDevice, st)) return rc;
   } else if (const void* src = tl3::pinned_address(X, x_bytes)) {
     const long long total = m->K * N;
     tl3::tl3_spread_rows_kernel<<<static_cast<unsigned>((total + 2047) / 2048), 256, 0, st>>>(static_cast<const uint16_t*>(src), static_cast<uint16_t*>(dX),
@@ -1053,8 +1095,7 @@ int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int
                                static_cast<size_t>(m->K), cudaMemcpyHostToDevice, st));
   }
   if (int rc = tl3_spmm(m, dX, ldx, dY, N, N, workspace, stream)) return rc;
-  TL3_CUDA(cudaMemcpyAsync(Y, dY, static_cast<size_t>(m->M) * N * 2, cudaMemcpyDeviceToHost, st));
-  return TL3_OK;
+  return tl3::copy_host(Y, dY, static_cast<size_t>(m->M) * N * 2, cudaMemcpyDeviceToHost, st);
 }
 
 int tl3_spmm_host(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY, void* workspace, void* stream) {

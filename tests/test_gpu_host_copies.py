@@ -1,0 +1,46 @@
+"""Host buffers in both directions, pinned and not, on 16 bytes or not, of sizes around a thread's 16 bytes,
+a block's 4096 and the largest that a kernel copies (needs a B200): bit for bit the device entry point."""
+import numpy as np
+import pytest
+
+from paper_2607_08786_b200 import build, tl3, workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (129, 16, 8), (256, 256, 8), (257, 264, 8), (255, 130, 16), (8192, 128, 64), (8193, 128, 64), (130, 8200, 64), (1000, 60, 5)])
+@pytest.mark.parametrize("x_shift,y_shift", [(0, 0), (8, 8), (1, 0), (0, 1), (None, 0), (0, None)])      # None: pageable
+def test_host_copies(M, K, N, x_shift, y_shift):
+    import torch
+    build.build_library()
+    case = wl.Case(0, "copies", M, K, N, 60 + N, 0.5, "magnitude")
+    X = case.make_X()
+    m = tl3.encode(case.make_W())
+    m.upload()
+    ld = (N + 7) // 8 * 8
+    Xd = torch.zeros((K, ld), dtype=torch.float16, device="cuda")
+    Xd[:, :N] = torch.from_numpy(X)
+    want = m.spmm(Xd[:, :N]).cpu().numpy()
+    ws = m.new_workspace(N)
+    dX = torch.zeros(K * ld, dtype=torch.float16, device="cuda")
+    dY = torch.empty(M * N, dtype=torch.float16, device="cuda")
+
+    def buffer(rows, cols, shift):
+        room = torch.full((rows * cols + 16,), 7.0, dtype=torch.float16, pin_memory=shift is not None)
+        return room, room.numpy()[(shift or 0):(shift or 0) + rows * cols].reshape(rows, cols)
+
+    (x_room, x), (y_room, y) = buffer(K, N, x_shift), buffer(M, N, y_shift)
+    x[:] = X
+    for _ in range(3):                                      # one after another on the same buffers
+        y[:] = 0
+        m.spmm_host(x, y, dX, dY, ws)
+        assert np.array_equal(y.view(np.uint16), want.view(np.uint16))
+    before = y_shift or 0
+    assert bool((y_room[:before] == 7).all()) and bool((y_room[before + M * N:] == 7).all())
+    # two products behind each other on one stream, with the same device buffers
+    y2_room, y2 = buffer(M, N, y_shift)
+    y[:] = 0
+    m.spmm_host_async(x, y, dX, dY, ws)
+    m.spmm_host_async(x, y2, dX, dY, ws)
+    torch.cuda.synchronize()
+    assert np.array_equal(y.view(np.uint16), want.view(np.uint16)) and np.array_equal(y2.view(np.uint16), want.view(np.uint16))
