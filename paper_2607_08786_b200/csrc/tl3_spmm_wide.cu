@@ -11,7 +11,7 @@
 //   * one launch covers all columns: a row-tile is worked on once per group of n_pad columns, the
 //     groups of a row-tile directly after one another (its blocks then come from L2);
 //   * two accumulators while they fit tensor memory beside the metadata, else one;
-//   * above 128 columns two CTAs of a cluster work on two row-tiles as one tcgen05.mma of 256 rows: each
+//   * above 128 columns, and above 64 in long launches, two CTAs of a cluster work on two row-tiles as one tcgen05.mma of 256 rows: each
 //     decodes its own blocks and loads half of the columns of X.
 // What bounds it at 256 columns (20480 x 5120, N = 512: 107 us, 1.0 PFLOP/s of what the two sparse
 // operands issue, counting empty slots): buffers.  A tile takes 1800 cycles; its MMAs are 1024 of them,
@@ -688,6 +688,19 @@ int launch_wide(const CUtensorMap& map, const WideArgs& args, int grid, uint32_t
 // 125 in 2, 142 in 3, 160 in 4, all with one CTA per tile.)
 constexpr int kAloneColumns = 128;
 
+// Long launches of 65 to 128 columns go in pairs as well: from 32 tiles per CTA on what a tile saves by half of X
+// outweighs the cluster's start and the columns that a multiple of 32 adds.  (us alone / in pairs, X [batch, hidden]: 20480 x
+// 5120, 43 tiles, N = 65 41.0 / 40.1, N = 128 45.5 / 43.4, at 40 % sparsity 53.3 / 49.4; 36864 x 9216, N = 128 127 / 118; 9000 x
+// 9000, 34 tiles, N = 96 37.0 / 35.9; with 19 to 20 tiles 0.94 to 1.05 of alone, N = 112 on 7000 x 7000 27.9 / 28.6; 4096 x 4096,
+// 7 tiles, 17.1 / 19.1.  X [hidden, batch]: 20480 x 5120, N = 65 50.0 / 46.2.)  Up to 64 columns a CTA alone is never
+// slower (1000 x 20000, N = 128 in passes of 64 23.4 / 24.4).
+constexpr int kPairTiles = 32;
+static int ctas_together(const tl3_matrix* m, int N, int n_pad, int sm_count) {
+  if (n_pad > kAloneColumns) return 2;
+  const int64_t tiles = m->n_tiles * ((N + n_pad - 1) / n_pad);
+  return n_pad > kAloneColumns / 2 && tiles >= static_cast<int64_t>(kPairTiles) * sm_count ? 2 : 1;
+}
+
 static int wide_columns(const tl3_matrix* m, int N, int sm_count) {
   double best = 0;
   int best_n = 0;
@@ -714,11 +727,12 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   if (di.cc_major != 10) return TL3_ERR_UNSUPPORTED;
 
   WideArgs a{};
-  const int n_pad = wide_columns(m, N, di.sm_count);
+  int n_pad = wide_columns(m, N, di.sm_count);
+  const int S = ctas_together(m, N, n_pad, di.sm_count);
+  if (S == 2) n_pad = (n_pad + 31) / 32 * 32;                       // (an MMA of 256 rows takes multiples of 32)
   a.block_area = (m->max_block_bytes + 1023u) / 1024u * 1024u;
-  const int S = n_pad > kAloneColumns ? 2 : 1;
   a.n_pad[0] = n_pad;
-  a.n_pad[1] = S == 1 ? n_pad : (n_pad / 2 + 31) / 32 * 32;         // (an MMA of 256 rows takes multiples of 32)
+  a.n_pad[1] = S == 1 ? n_pad : (n_pad / 2 + 31) / 32 * 32;
   for (int i = 0; i < 2; ++i) a.chunks[i] = static_cast<uint32_t>((N + a.n_pad[i] - 1) / a.n_pad[i]);
   a.x_bytes = xt ? static_cast<uint32_t>(n_pad / S) * 128u : static_cast<uint32_t>((n_pad / S + 63) / 64) * 8192u;   // per CTA
   a.n_acc = 2 * n_pad <= static_cast<int>(kColMetaT) ? 2 : 1;
