@@ -184,8 +184,8 @@ int tl3_upload(tl3_matrix* m, void* dptr, void* stream);
  * Errors: INVALID_ARG, UNSUPPORTED (tile shape other than 128 x 128), CUDA, NO_MEMORY. */
 int tl3_plan_device(tl3_matrix* m, void* stream);
 int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream);
-/* Gives back the 6 MB of pinned host memory that the library keeps, from the first container of more
- * than 8 MB that these two calls copy to a device on, for the next one.  Any thread, any time. */
+/* Gives back the 12 MB of pinned host memory that the library keeps, from the first container of more
+ * than 8 MB that is copied to or from a device on, for the next one.  Any thread, any time. */
 int tl3_trim(void);
 
 /* Bind a device buffer that already holds the packed blob -- the bytes of tl3_pack() copied to the

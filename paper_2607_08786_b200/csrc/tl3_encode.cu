@@ -287,25 +287,19 @@ extern "C" int tl3_encode_device(const void* dW, int64_t M, int64_t K, int64_t l
     a.emit = 1;
     tl3_encode_kernel<<<static_cast<unsigned>(m->n_tiles), kTileThreads, sizeof(EncodeSmem), st>>>(a);
     TL3_ENC_CUDA(cudaGetLastError());
+    std::vector<HostPiece> arrays;
     try {
       m->tc_vals.resize(n_vals); m->tc_meta.resize(n_meta);
       m->chain_tau0.resize(n_chain); m->chain_rho0.resize(n_chain); m->chain_len.resize(n_chain);
       m->tile_dir.resize(n_dir);
       m->pdd_bytes.resize(totals[0]); m->res_rho.resize(totals[1]); m->res_val.resize(totals[1]);
+      arrays = {
+        {m->tc_vals.data(), a.tc_vals, n_vals * 2}, {m->tc_meta.data(), a.tc_meta, n_meta},
+        {m->chain_tau0.data(), a.chain_tau0, n_chain * 2}, {m->chain_rho0.data(), a.chain_rho0, n_chain * 2},
+        {m->chain_len.data(), a.chain_len, n_chain}, {m->tile_dir.data(), a.tile_dir, n_dir * 4},
+        {m->pdd_bytes.data(), a.pdd_bytes, totals[0]}, {m->res_rho.data(), a.res_rho, totals[1] * 2}, {m->res_val.data(), a.res_val, totals[1] * 2}};
     } catch (const std::bad_alloc&) { rc = TL3_ERR_NO_MEMORY; goto done; }
-    prefault(m->tc_vals.data(), n_vals * 2);                       // while the kernel runs
-    prefault(m->tc_meta.data(), n_meta);
-    TL3_ENC_CUDA(cudaMemcpyAsync(m->tc_vals.data(), a.tc_vals, n_vals * 2, cudaMemcpyDeviceToHost, st));
-    TL3_ENC_CUDA(cudaMemcpyAsync(m->tc_meta.data(), a.tc_meta, n_meta, cudaMemcpyDeviceToHost, st));
-    TL3_ENC_CUDA(cudaMemcpyAsync(m->chain_tau0.data(), a.chain_tau0, n_chain * 2, cudaMemcpyDeviceToHost, st));
-    TL3_ENC_CUDA(cudaMemcpyAsync(m->chain_rho0.data(), a.chain_rho0, n_chain * 2, cudaMemcpyDeviceToHost, st));
-    TL3_ENC_CUDA(cudaMemcpyAsync(m->chain_len.data(), a.chain_len, n_chain, cudaMemcpyDeviceToHost, st));
-    TL3_ENC_CUDA(cudaMemcpyAsync(m->tile_dir.data(), a.tile_dir, n_dir * 4, cudaMemcpyDeviceToHost, st));
-    if (totals[0]) TL3_ENC_CUDA(cudaMemcpyAsync(m->pdd_bytes.data(), a.pdd_bytes, totals[0], cudaMemcpyDeviceToHost, st));
-    if (totals[1]) {
-      TL3_ENC_CUDA(cudaMemcpyAsync(m->res_rho.data(), a.res_rho, totals[1] * 2, cudaMemcpyDeviceToHost, st));
-      TL3_ENC_CUDA(cudaMemcpyAsync(m->res_val.data(), a.res_val, totals[1] * 2, cudaMemcpyDeviceToHost, st));
-    }
+    TL3_ENC_CUDA(copy_pieces(arrays, cudaMemcpyDeviceToHost, st));
     TL3_ENC_CUDA(cudaMemcpyAsync(stats, a.stats, sizeof(stats), cudaMemcpyDeviceToHost, st));
     TL3_ENC_CUDA(cudaStreamSynchronize(st));
     m->nnz = static_cast<int64_t>(stats[0]); m->n_tc = static_cast<int64_t>(stats[1]); m->n_sf = static_cast<int64_t>(stats[2]);

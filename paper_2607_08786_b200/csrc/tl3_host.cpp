@@ -34,14 +34,17 @@ static void run_parallel(int64_t n, unsigned most, const F& f) {
 
 constexpr size_t kCopyChunk = size_t{1} << 20;
 
-void parallel_copy(void* dst, const void* src, size_t bytes) {
+// What takes the time is the first touch of `dst`, page by page, so more threads help beyond what memory moves (132 MB
+// into huge pages 7.2 ms with eight threads, 5.1 with sixteen; 55 MB into small ones 5.1 and 4.0), and two that
+// meet in one huge page wait for each other (6.0 ms in chunks of 1 MB there).
+void parallel_copy(void* dst, const void* src, size_t bytes, size_t chunk) {
   if (bytes < 4 * kCopyChunk) {
     if (bytes) std::memcpy(dst, src, bytes);
     return;
   }
-  run_parallel(static_cast<int64_t>((bytes + kCopyChunk - 1) / kCopyChunk), 8, [&](int64_t i) {
-    const size_t at = static_cast<size_t>(i) * kCopyChunk;
-    std::memcpy(static_cast<uint8_t*>(dst) + at, static_cast<const uint8_t*>(src) + at, std::min(kCopyChunk, bytes - at));
+  run_parallel(static_cast<int64_t>((bytes + chunk - 1) / chunk), 16, [&](int64_t i) {
+    const size_t at = static_cast<size_t>(i) * chunk;
+    std::memcpy(static_cast<uint8_t*>(dst) + at, static_cast<const uint8_t*>(src) + at, std::min(chunk, bytes - at));
   });
 }
 
@@ -712,7 +715,7 @@ int tl3_deserialize(const void* buf, size_t bytes, tl3_matrix** out) {
     p += 8;
     if (n > static_cast<uint64_t>(end - p) || n % sizeof(T) != 0) return false;
     vec.resize(n / sizeof(T));
-    parallel_copy(vec.data(), p, n);
+    parallel_copy(vec.data(), p, n, tl3::RawAllocator<T>::kHuge);
     p += n;
     return true;
   };

@@ -44,8 +44,8 @@ template <class T> struct RawAllocator {
 };
 template <class T> using raw_vector = std::vector<T, RawAllocator<T>>;
 
-// Large copies and first touches of fresh memory, shared out over up to eight threads (tl3_host.cpp).
-void parallel_copy(void* dst, const void* src, size_t bytes);
+// Large copies and first touches of fresh memory, shared out over up to sixteen and eight threads (tl3_host.cpp).
+void parallel_copy(void* dst, const void* src, size_t bytes, size_t chunk = size_t{1} << 20);
 void prefault(void* p, size_t bytes);                        // fresh memory that a copy engine is about to fill
 
 }  // namespace tl3
@@ -159,5 +159,15 @@ void set_device_layout(const tl3_matrix* m, const uint32_t* sizes);   // layout 
 void blob_header_and_offsets(const tl3_matrix* m, uint8_t* header256, std::vector<unsigned long long>* block_off);
 
 void set_cuda_error(int e);
+
+#ifdef __CUDACC__
+// tl3_pack_device.cu: large arrays in pageable memory to or from the device
+struct HostPiece {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+cudaError_t copy_pieces(const std::vector<HostPiece>& arrays, cudaMemcpyKind kind, cudaStream_t st);
+#endif
 
 }  // namespace tl3

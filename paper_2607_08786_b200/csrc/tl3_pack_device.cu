@@ -192,17 +192,12 @@ void release_canon(void* p) {
     }                                                         \
   } while (0)
 
-struct HostPiece {
-  void* dst;
-  const void* src;
-  size_t bytes;
-};
-
-// The pinned memory of copy_from_host(): 6 MB that stay between calls (pinning them costs more than a copy
+// The pinned memory of copy_pieces(): 12 MB that stay between calls (pinning them costs more than a copy
 // of 100 MB) until tl3_trim(), for one caller at a time.  Somebody's cudaDeviceReset() takes such memory
 // away, and its address may then be another allocation's: what is kept is used only while the driver
 // still knows it by the number that it gave it.
-constexpr int kRingSlots = 6;
+constexpr int kRingThreads = 6;
+constexpr int kRingSlots = 2 * kRingThreads;
 constexpr size_t kRingSlotBytes = size_t{1} << 20;
 
 template <class Fn> Fn driver_entry(const char* name) {
@@ -245,10 +240,15 @@ PinnedRing& ring_of_process() {
   return *r;
 }
 
-// Pageable host memory to the device, complete on return.  The runtime's own copy moves 11 GB/s, one
-// thread of its filling one staging buffer; here six threads fill a pinned megabyte each (one caller at a
-// time; another one that comes meanwhile takes the runtime's way).  132 MB: 12.2 -> 5 ms.
-cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st) {
+}  // namespace
+
+// Pageable host memory to or from the device, behind what is on `st`, complete on return.  The runtime's own copy moves
+// 11 GB/s, one thread of its filling or emptying one staging buffer; here six threads do that with two
+// pinned megabytes each, one of them under way while the other is worked on (one caller at a
+// time; another one that comes meanwhile takes the runtime's way).  132 MB up: 12.2 ms the runtime's way, 5.9 with one megabyte per thread, 4.7
+// with two (5.9 with two halves, 4.5 with two of two); 55 MB down 5.0 and 2.0.
+cudaError_t copy_pieces(const std::vector<HostPiece>& arrays, cudaMemcpyKind kind, cudaStream_t st) {
+  const bool up = kind == cudaMemcpyHostToDevice;
   size_t total = 0;
   for (const HostPiece& p : arrays) total += p.bytes;
   PinnedRing& pinned = ring_of_process();
@@ -266,7 +266,8 @@ cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st
   if (!staged) {
     for (const HostPiece& p : arrays) {
       if (!p.bytes) continue;
-      if (cudaError_t e = cudaMemcpyAsync(p.dst, p.src, p.bytes, cudaMemcpyHostToDevice, st)) return e;
+      if (!up) prefault(p.dst, p.bytes);
+      if (cudaError_t e = cudaMemcpyAsync(p.dst, p.src, p.bytes, kind, st)) return e;
     }
     return cudaStreamSynchronize(st);
   }
@@ -274,32 +275,45 @@ cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st
   std::vector<std::thread> pool;
   std::atomic<size_t> next{0};
   std::atomic<int> failed{cudaSuccess};
-  auto worker = [&](int slot) {
-    uint8_t* buf = ring + static_cast<size_t>(slot) * kRingSlotBytes;
-    cudaEvent_t done = nullptr;
+  auto worker = [&](int thread) {
+    uint8_t* buf[2];
+    cudaEvent_t done[2] = {nullptr, nullptr};
+    const HostPiece* under_way[2] = {nullptr, nullptr};
     cudaError_t e = set_context(context) == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
-    bool busy = false;
-    while (e == cudaSuccess && failed.load(std::memory_order_relaxed) == cudaSuccess) {
-      const size_t i = next.fetch_add(1);
-      if (i >= pieces.size()) break;
-      if (busy) e = cudaEventSynchronize(done);
-      if (e != cudaSuccess) break;
-      std::memcpy(buf, pieces[i].src, pieces[i].bytes);
-      e = cudaMemcpyAsync(pieces[i].dst, buf, pieces[i].bytes, cudaMemcpyHostToDevice, own);
-      if (e == cudaSuccess) e = cudaEventRecord(done, own);
-      busy = true;
+    for (int k = 0; k < 2; ++k) {
+      buf[k] = ring + static_cast<size_t>(2 * thread + k) * kRingSlotBytes;
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[k], cudaEventDisableTiming);
     }
-    if (done) cudaEventDestroy(done);
+    auto finish = [&](int k) {                                     // the slot's copy is through; what came down goes to its place
+      if (e != cudaSuccess || !under_way[k]) return;
+      e = cudaEventSynchronize(done[k]);
+      if (e == cudaSuccess && !up) std::memcpy(under_way[k]->dst, buf[k], under_way[k]->bytes);
+      under_way[k] = nullptr;
+    };
+    for (int k = 0; e == cudaSuccess && failed.load(std::memory_order_relaxed) == cudaSuccess; k ^= 1) {
+      const size_t i = next.fetch_add(1);
+      finish(k);
+      if (i >= pieces.size() || e != cudaSuccess) break;
+      const HostPiece& p = pieces[i];
+      if (up) std::memcpy(buf[k], p.src, p.bytes);
+      e = up ? cudaMemcpyAsync(p.dst, buf[k], p.bytes, kind, own) : cudaMemcpyAsync(buf[k], p.src, p.bytes, kind, own);
+      if (e == cudaSuccess) e = cudaEventRecord(done[k], own);
+      under_way[k] = &p;
+    }
+    finish(0);
+    finish(1);
+    for (int k = 0; k < 2; ++k)
+      if (done[k]) cudaEventDestroy(done[k]);
     if (e != cudaSuccess) failed.store(e, std::memory_order_relaxed);
   };
+  if (!up) failed.store(cudaStreamSynchronize(st));                // (what comes down has been written)
   bool listed = false;
   try {
     for (const HostPiece& p : arrays)
       for (size_t at = 0; at < p.bytes; at += kRingSlotBytes)
         pieces.push_back({static_cast<uint8_t*>(p.dst) + at, static_cast<const uint8_t*>(p.src) + at, std::min(kRingSlotBytes, p.bytes - at)});
     listed = true;
-    for (int t = 1; t < kRingSlots; ++t) pool.emplace_back(worker, t);
+    for (int t = 1; t < kRingThreads; ++t) pool.emplace_back(worker, t);
   } catch (const std::exception&) {                              // fewer threads, or no list at all
   }
   if (!listed) failed.store(cudaErrorMemoryAllocation);
@@ -309,6 +323,8 @@ cudaError_t copy_from_host(const std::vector<HostPiece>& arrays, cudaStream_t st
   cudaStreamDestroy(own);
   return failed.load() != cudaSuccess ? static_cast<cudaError_t>(failed.load()) : e;
 }
+
+namespace {
 
 // Copies the canonical arrays of the handle to the device (one allocation, kept in the handle) and
 // fills the kernel arguments that point into it.
@@ -338,7 +354,7 @@ int canon_to_device(tl3_matrix* m, cudaStream_t st, PackArgs* out) {
     cudaError_t e = cudaErrorMemoryAllocation;
     try {
       for (int i = 0; i < 9; ++i) arrays.push_back({b + off[i], src[i], sz[i]});
-      e = copy_from_host(arrays, st);
+      e = copy_pieces(arrays, cudaMemcpyHostToDevice, st);
     } catch (const std::bad_alloc&) {
     }
     if (e != cudaSuccess) {                                        // nothing half-copied stays with the handle
