@@ -339,6 +339,31 @@ __device__ __forceinline__ void decode_chain(uint32_t stage, uint32_t wr, uint32
   }
 }
 
+// Residual layer of a tile for thread r of a decode group: (position, value) entries go to W_r.  Tiles with many (kLong)
+// take four at a time, loads before stores: one after another, 13 per thread at 40 % sparsity, their round
+// trips stood in the decode's way (11008 x 4096 at 40 %, N = 24 23.2 -> 22.2 us, N = 16 18.9 -> 18.2; 20480 x 5120 at 40 %, N = 128
+// 49.4 -> 46.8).  A kernel of its own, because tiles with one or two per thread only lose by the longer code
+// (9216 x 9216, N = 64 30.5 -> 30.8).
+template <bool kLong>
+__device__ __forceinline__ void scatter_residual(uint32_t res, uint32_t wr, uint32_t r, uint32_t res_cnt, uint32_t* bad) {
+  uint32_t k = r;
+  if constexpr (kLong) {
+    for (uint32_t left = res_cnt; left >= 512u; left -= 512u, k += 512u) {
+      uint32_t rv[4], any = 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { rv[q] = lds_u32(res + 4 * (k + 128u * q)); any |= rv[q]; }
+      if (any & 0xE000u) { *bad = 4u; return; }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) sts_u16(wr + swizzled_offset(rv[q] & 0xFFFFu), rv[q] >> 16);
+    }
+  }
+  for (; k < res_cnt; k += 128) {
+    const uint32_t rv = lds_u32(res + 4 * k);
+    if ((rv & 0xFFFFu) < 8192u) sts_u16(wr + swizzled_offset(rv & 0xFFFFu), rv >> 16);
+    else *bad = 4u;
+  }
+}
+
 // ---------------------------------------------------------------------------------------------
 // Host side, in tl3_spmm.cu
 // ---------------------------------------------------------------------------------------------
@@ -353,6 +378,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 EncodeTiledFn encode_tiled_fn();
+
+// whether a matrix's tiles have so many Residual entries that scatter_residual<true> pays: one batch of four per thread
+// on average, which leaves out 50 % sparsity and more (1.6 % of the weights, 130 entries a tile) and takes in 40 % (1640)
+inline bool long_residual(const tl3_matrix* m) { return m->dev_n_res >= 512 * m->n_tiles; }
 
 struct WorkspaceLayout {
   size_t status_off = 0, flags_off = 256, room_off = 0, partials_off = 0, total = 0;

@@ -109,7 +109,8 @@ __device__ __forceinline__ long long clock_now() { long long c; asm volatile("mo
 // XT: the activations are given as X^T (N x K row-major, the [batch, hidden] layout of an inference
 // stack, Sec. 2.1) and the result is written as Y^T (N x M row-major).  The X tile then arrives as
 // two boxes of 64 k-values (128 bytes per row, 128-byte swizzle) and is a K-major B operand.
-template <int NPAD, bool XT>
+// kLongRes: see scatter_residual().
+template <int NPAD, bool XT, bool kLongRes>
 __global__ void __launch_bounds__(kThreads, 1)
 tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
   extern __shared__ uint8_t smem_raw[];
@@ -384,12 +385,7 @@ tl3_spmm_kernel(const __grid_constant__ CUtensorMap x_map, const KernelArgs a) {
       __syncwarp();
       // Residual layer: (position, value) entries go to W_r too
       if (lens_ok) {
-        const uint32_t res = stage + kPddOff + ((pdd_len + 3u) & ~3u);
-        for (uint32_t k = r; k < res_cnt; k += 128) {
-          const uint32_t rv = lds_u32(res + 4 * k);
-          if ((rv & 0xFFFFu) < 8192u) sts_u16(wr + swizzled_offset(rv & 0xFFFFu), rv >> 16);
-          else bad = 4u;
-        }
+        scatter_residual<kLongRes>(stage + kPddOff + ((pdd_len + 3u) & ~3u), wr, r, res_cnt, &bad);
       }
       if (bad) atomicCAS(a.status, 0u, kStBadBlock | (bad << 8) | (static_cast<uint32_t>(i) << 12));
       fence_proxy_async_smem();                                   // generic-proxy writes -> MMA reads
@@ -786,8 +782,8 @@ static int copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind ki
 // Process-wide launch tuning (tl3_set_tuning); the default is what measured best on B200.
 static std::atomic<int> g_decode_before_x{TL3_DEFAULT_DECODE_BEFORE_X};
 
-template <int NPAD, bool XT>
-static int launch(const CUtensorMap& map, const KernelArgs& args, int grid, uint32_t smem_bytes, cudaStream_t stream) {
+template <int NPAD, bool XT, bool kLongRes>
+static int launch_kernel(const CUtensorMap& map, const KernelArgs& args, int grid, uint32_t smem_bytes, cudaStream_t stream) {
   // The opt-in to more than 48 KB of dynamic shared memory is a property of the function on ONE
   // device: it is set once per device and template instance.
   {
@@ -798,7 +794,7 @@ static int launch(const CUtensorMap& map, const KernelArgs& args, int grid, uint
     std::lock_guard<std::mutex> lock(mu);
     if (static_cast<size_t>(dev) >= configured.size()) configured.resize(dev + 1, 0);
     if (!configured[dev]) {
-      TL3_CUDA(cudaFuncSetAttribute(tl3_spmm_kernel<NPAD, XT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemLimit)));
+      TL3_CUDA(cudaFuncSetAttribute(tl3_spmm_kernel<NPAD, XT, kLongRes>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemLimit)));
       configured[dev] = 1;
     }
   }
@@ -812,9 +808,13 @@ static int launch(const CUtensorMap& map, const KernelArgs& args, int grid, uint
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_spmm_kernel<NPAD, XT>, map, args));
+  TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_spmm_kernel<NPAD, XT, kLongRes>, map, args));
   TL3_CUDA(cudaGetLastError());
   return TL3_OK;
+}
+template <int NPAD, bool XT>
+static int launch(const CUtensorMap& map, const KernelArgs& args, bool long_res, int grid, uint32_t smem_bytes, cudaStream_t stream) {
+  return long_res ? launch_kernel<NPAD, XT, true>(map, args, grid, smem_bytes, stream) : launch_kernel<NPAD, XT, false>(map, args, grid, smem_bytes, stream);
 }
 
 }  // namespace tl3
@@ -1011,17 +1011,18 @@ static int spmm_block(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, 
   m->last_ctas = grid; m->last_stages = stages; m->last_smem = static_cast<int>(smem_bytes);
   m->last_pass.store(n_pad | 1 << 16 | 2 << 24, std::memory_order_relaxed);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const bool long_res = long_residual(m);
   if (xt) {
     switch (n_pad) {
-      case 16: return launch<16, true>(map, args, grid, smem_bytes, st);
-      case 32: return launch<32, true>(map, args, grid, smem_bytes, st);
-      default: return launch<64, true>(map, args, grid, smem_bytes, st);
+      case 16: return launch<16, true>(map, args, long_res, grid, smem_bytes, st);
+      case 32: return launch<32, true>(map, args, long_res, grid, smem_bytes, st);
+      default: return launch<64, true>(map, args, long_res, grid, smem_bytes, st);
     }
   }
   switch (n_pad) {
-    case 16: return launch<16, false>(map, args, grid, smem_bytes, st);
-    case 32: return launch<32, false>(map, args, grid, smem_bytes, st);
-    default: return launch<64, false>(map, args, grid, smem_bytes, st);
+    case 16: return launch<16, false>(map, args, long_res, grid, smem_bytes, st);
+    case 32: return launch<32, false>(map, args, long_res, grid, smem_bytes, st);
+    default: return launch<64, false>(map, args, long_res, grid, smem_bytes, st);
   }
 }
 

@@ -291,7 +291,8 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
 
 // XT as in tl3_spmm.cu: activations and result transposed ([batch, hidden]).
 // S: CTAs that work together, 1 or 2 (a cluster).
-template <bool XT, int S>
+// kLongRes: see scatter_residual().
+template <bool XT, int S, bool kLongRes>
 __global__ void __launch_bounds__(kThreadsOf<S>, 1)
 tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_constant__ WideArgs a) {
   constexpr int kGroups = kGroupsOf<S>, kEpilogueWarp0 = kDecodeWarp0 + 4 * kGroups;
@@ -515,12 +516,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
       else bad = 3u;
       __syncwarp();
       if (lens_ok) {                                              // Residual layer: (position, value) entries go to W_r too
-        const uint32_t res = stage + kPddOff + ((pdd_len + 3u) & ~3u);
-        for (uint32_t k = r; k < res_cnt; k += 128) {
-          const uint32_t rv = lds_u32(res + 4 * k);
-          if ((rv & 0xFFFFu) < 8192u) sts_u16(wr + swizzled_offset(rv & 0xFFFFu), rv >> 16);
-          else bad = 4u;
-        }
+        scatter_residual<kLongRes>(stage + kPddOff + ((pdd_len + 3u) & ~3u), wr, r, res_cnt, &bad);
       }
       if (bad) atomicCAS(a.status, 0u, kStBadBlock | (bad << 8) | (static_cast<uint32_t>(i) << 12));
       fence_proxy_async_smem();                                   // generic-proxy writes -> MMA reads
@@ -643,8 +639,8 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
   }
 }
 
-template <bool XT, int S>
-int launch_wide(const CUtensorMap& map, const WideArgs& args, int grid, uint32_t smem_bytes, cudaStream_t stream) {
+template <bool XT, int S, bool kLongRes>
+int launch_wide_kernel(const CUtensorMap& map, const WideArgs& args, int grid, uint32_t smem_bytes, cudaStream_t stream) {
   {
     int dev = 0;
     TL3_CUDA(cudaGetDevice(&dev));
@@ -653,7 +649,7 @@ int launch_wide(const CUtensorMap& map, const WideArgs& args, int grid, uint32_t
     std::lock_guard<std::mutex> lock(mu);
     if (static_cast<size_t>(dev) >= configured.size()) configured.resize(dev + 1, 0);
     if (!configured[dev]) {
-      TL3_CUDA(cudaFuncSetAttribute(tl3_spmm_wide_kernel<XT, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemLimit)));
+      TL3_CUDA(cudaFuncSetAttribute(tl3_spmm_wide_kernel<XT, S, kLongRes>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmemLimit)));
       configured[dev] = 1;
     }
   }
@@ -670,9 +666,14 @@ int launch_wide(const CUtensorMap& map, const WideArgs& args, int grid, uint32_t
   attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = S == 1 ? 1 : 2;
-  TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_spmm_wide_kernel<XT, S>, map, args));
+  TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_spmm_wide_kernel<XT, S, kLongRes>, map, args));
   TL3_CUDA(cudaGetLastError());
   return TL3_OK;
+}
+
+template <bool XT, int S>
+int launch_wide(const CUtensorMap& map, const WideArgs& args, bool long_res, int grid, uint32_t smem_bytes, cudaStream_t stream) {
+  return long_res ? launch_wide_kernel<XT, S, true>(map, args, grid, smem_bytes, stream) : launch_wide_kernel<XT, S, false>(map, args, grid, smem_bytes, stream);
 }
 
 }  // namespace
@@ -800,8 +801,8 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   m->last_ctas = grid; m->last_stages = a.n_w; m->last_smem = static_cast<int>(smem_bytes);
   m->last_pass.store(n_pad | S << 16 | a.n_acc << 24, std::memory_order_relaxed);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (S == 2) return xt ? launch_wide<true, 2>(map, a, grid, smem_bytes, st) : launch_wide<false, 2>(map, a, grid, smem_bytes, st);
-  return xt ? launch_wide<true, 1>(map, a, grid, smem_bytes, st) : launch_wide<false, 1>(map, a, grid, smem_bytes, st);
+  if (S == 2) return xt ? launch_wide<true, 2>(map, a, long_residual(m), grid, smem_bytes, st) : launch_wide<false, 2>(map, a, long_residual(m), grid, smem_bytes, st);
+  return xt ? launch_wide<true, 1>(map, a, long_residual(m), grid, smem_bytes, st) : launch_wide<false, 1>(map, a, long_residual(m), grid, smem_bytes, st);
 }
 
 }  // namespace tl3
