@@ -198,14 +198,17 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
   const int lane = et & 31;
   // XT: four lanes hand each other their values, so that a thread stores four rows of one column
   const bool quads = XT && row - lane + 32 <= a.M && (a.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(a.Y) & 7) == 0;
-  // A row-tile of its own is read one step ahead; one that others contribute to keeps the registers for
+  // A CTA alone reads a row-tile of its own one step ahead (4096 x 4096, N = 100 19.6 us, without 19.9).  In pairs the
+  // registers for it cost more than the wait (20000 x 256, N = 500 29.1 and 27.7, 20480 x 5120, N = 512 111.1 and 109.7,
+  // 5120 x 5120, N = 256 29.4 and 28.9), and a row-tile that others contribute to keeps them for
   // their partial sums, two slots' loads in flight.
+  constexpr bool kAhead = !kShared && S == 1;
   uint32_t next[CH];
-  if (!kShared) TmemLd<CH>::ld(acc_tmem + c_begin, next);
+  if constexpr (kAhead) TmemLd<CH>::ld(acc_tmem + c_begin, next);
 #pragma unroll 1
   for (int c0 = c_begin; c0 < cols; c0 += c_step) {
     uint32_t v[CH];
-    if (!kShared) {
+    if constexpr (kAhead) {
       tmem_wait_ld<CH>(next);
 #pragma unroll
       for (int c = 0; c < CH; ++c) v[c] = next[c];
@@ -213,6 +216,8 @@ __device__ __noinline__ void write_columns(const WideArgs& a, int less, uint32_t
     } else {
       TmemLd<CH>::ld(acc_tmem + c0, v);
       tmem_wait_ld<CH>(v);
+    }
+    if constexpr (kShared) {
       const float* p = a.partials + slot * (blockIdx.x + S) + c0 * 128 + et;   // the next CTA, or the same one of the next pair
       for (int k = 0; k < n_others; k += 2, p += 2 * S * slot) {
         float p0[CH], p1[CH];
