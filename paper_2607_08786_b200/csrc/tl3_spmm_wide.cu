@@ -13,10 +13,9 @@
 //   * two accumulators while they fit tensor memory beside the metadata, else one;
 //   * above 128 columns, and above 64 in long launches, two CTAs of a cluster work on two row-tiles as one tcgen05.mma of 256 rows: each
 //     decodes its own blocks and loads half of the columns of X.
-// What bounds it at 256 columns (20480 x 5120, N = 512: 107 us, 1.0 PFLOP/s of what the two sparse
-// operands issue, counting empty slots): buffers.  A tile takes 1800 cycles; its MMAs are 1024 of them,
-// its decode 2000 in each of four groups, and the issuing warp waits 1000 for blocks, X and the
-// accumulator that one epilogue per 40 tiles empties.
+// What bounds it at 256 columns (20480 x 5120, N = 512: 110 us at 1965 MHz, 135 at the clock that the power cap leaves): without
+// decode 97, without MMAs 87, without either 80, which is 61 for the bytes from L2 (53 KB a tile and CTA at 77
+// GB/s) and the ends of the launch; 11 pass while the one accumulator is written out.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
