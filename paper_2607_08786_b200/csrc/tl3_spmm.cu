@@ -38,7 +38,12 @@
 namespace tl3 {
 
 static thread_local int g_last_cuda_error = 0;
-void set_cuda_error(int e) { g_last_cuda_error = e; }
+// (The runtime keeps a failed call's error for this thread until it is asked for; left there, the check behind the
+// next launch would take it for its own and report a good call as failed.)
+void set_cuda_error(int e) {
+  g_last_cuda_error = e;
+  cudaGetLastError();
+}
 
 // ---------------------------------------------------------------------------------------------
 // Kernel configuration

@@ -80,3 +80,39 @@ def test_conversion_on_a_nearly_full_device(tl3):
     del filler
     torch.cuda.empty_cache()
     assert torch.equal(blob, want)
+
+
+@pytest.mark.parametrize("call", ["encode_device_only", "encode_device", "plan_device"])
+def test_calls_after_one_that_found_no_memory(tl3, call):
+    """A conversion or an upload that the device has no room for reports that, and the calls after it on the same
+    thread report themselves: not the failed allocation once more."""
+    import torch
+    W = torch.from_numpy(_random(8192, 4096, 0.5)).cuda()
+    MB = 1 << 20
+    ref = tl3.Matrix.encode_on_device(W)
+    want = torch.from_numpy(ref.pack()).cuda()
+    W2 = torch.from_numpy(_random(300, 260, 0.5)).cuda()
+    X = torch.zeros((260, 16), dtype=torch.float16, device="cuda").normal_()
+    small = tl3.Matrix.encode_on_device(W2, device_only=True)
+    small.upload_packed_on_device()
+    ws, Y, again = small.new_workspace(16), small.spmm(X), torch.zeros((300, 16), dtype=torch.float16, device="cuda")
+    plan = tl3.Matrix.deserialize(ref.serialize())
+    calls = {"encode_device_only": lambda: tl3.Matrix.encode_on_device(W, device_only=True),
+             "encode_device": lambda: tl3.Matrix.encode_on_device(W),
+             "plan_device": lambda: tl3._check(tl3.lib().tl3_plan_device(plan._h, torch.cuda.current_stream().cuda_stream), "plan")}
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - 24 * MB, dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(tl3.Tl3Error) as e:
+            calls[call]()
+        assert e.value.code == tl3.ERR_CUDA and tl3.lib().tl3_last_cuda_error() == 2  # cudaErrorMemoryAllocation
+        small.spmm(X, again, workspace=ws)                                             # (allocates nothing)
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert torch.equal(again, Y)
+    m = tl3.Matrix.encode_on_device(W, device_only=True)
+    assert torch.equal(m.upload_packed_on_device(), want)
+    assert torch.equal(plan.upload_packed_on_device(), want)
+    assert torch.equal(small.spmm(X, again, workspace=ws), Y)
