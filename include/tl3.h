@@ -254,7 +254,9 @@ int tl3_spmm_nt(const tl3_matrix* m, const void* Xt, int64_t ldxt, void* Yt, int
 
 /* Same product with HOST buffers: copies X to dX, runs tl3_spmm, copies dY to Y and waits for the
  * stream.  X, Y: host (pinned memory makes the copies asynchronous), dense leading dimensions
- * ldx = ldy = N.  dX (>= K*N*2 bytes) and dY (>= M*N*2 bytes): device scratch owned by the caller. */
+ * ldx = ldy = N.  dX (>= K*N8*2 bytes, N8 = N rounded up to a multiple of eight, the pitch of the rows
+ * there; 16-byte aligned) and dY (>= M*N*2 bytes): device scratch owned by the caller.  Errors: as for tl3_spmm; CUDA
+ * also for a dX that lies in an allocation too small for X. */
 int tl3_spmm_host(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY,
                   void* workspace, void* stream);
 

@@ -717,9 +717,8 @@ tl3_spread_rows_kernel(const uint16_t* __restrict__ src, uint16_t* __restrict__ 
   }
 }
 
-// The address under which kernels read [p, p + bytes), if all of it lies in one pinned allocation (or
-// registration) and on 16 bytes; else null.
-static const void* pinned_address(const void* p, size_t bytes) {
+// Whether [p, p + bytes) lies in one allocation (or registration) of that type.  (40 ns.)
+static bool lies_in(CUmemorytype type, const void* p, size_t bytes) {
   typedef CUresult (*AttributesFn)(unsigned int, CUpointer_attribute*, void**, CUdeviceptr);
   static AttributesFn fn = []() -> AttributesFn {
     void* f = nullptr;
@@ -728,18 +727,25 @@ static const void* pinned_address(const void* p, size_t bytes) {
       return nullptr;
     return reinterpret_cast<AttributesFn>(f);
   }();
-  if (!fn) return nullptr;
-  unsigned int type = 0, managed = 0;
+  if (!fn) return false;
+  unsigned int got = 0, managed = 0;
   CUdeviceptr dev = 0, start = 0;
   size_t size = 0;
   CUpointer_attribute which[5] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
                                   CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
-  void* out[5] = {&type, &managed, &dev, &start, &size};
-  if (fn(5, which, out, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return nullptr;
-  if (type != CU_MEMORYTYPE_HOST || managed || !dev || (dev & 15) != 0) return nullptr;
-  if (dev != reinterpret_cast<CUdeviceptr>(p)) return nullptr;     // (a mapping at another address: the range is not in its terms)
-  if (dev < start || bytes > size || dev - start > size - bytes) return nullptr;
-  return reinterpret_cast<const void*>(dev);
+  void* out[5] = {&got, &managed, &dev, &start, &size};
+  if (fn(5, which, out, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+  if (got != static_cast<unsigned int>(type) || managed) return false;
+  if (dev != reinterpret_cast<CUdeviceptr>(p)) return false;       // (a mapping at another address: the range is not in its terms)
+  return dev && dev >= start && bytes <= size && dev - start <= size - bytes;
+}
+
+// Whether a kernel may do the copy of `bytes` between these: pinned host memory on 16 bytes and, for what it
+// writes to the device, an allocation that holds it.  The runtime's copies refuse one that does not; a kernel
+// would write beyond it.  (dY is the product's before it is a copy's.)
+static bool host_by_kernel(const void* host, size_t bytes) { return (reinterpret_cast<uintptr_t>(host) & 15) == 0 && lies_in(CU_MEMORYTYPE_HOST, host, bytes); }
+static bool up_by_kernel(const void* host, size_t bytes, const void* device, size_t device_bytes) {
+  return host_by_kernel(host, bytes) && lies_in(CU_MEMORYTYPE_DEVICE, device, device_bytes);
 }
 
 // Bytes between device memory and pinned host memory, 16 per thread and the last ones singly.
@@ -764,21 +770,18 @@ constexpr size_t kCopyByKernel = size_t{1} << 20;
 static int copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, cudaStream_t stream) {
   const bool up = kind == cudaMemcpyHostToDevice;
   const void* device = up ? dst : src;
-  if (bytes <= kCopyByKernel && (reinterpret_cast<uintptr_t>(device) & 15) == 0) {
-    if (const void* host = pinned_address(up ? src : dst, bytes)) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = dim3(static_cast<unsigned>((bytes + 4095) / 4096));
-      cfg.blockDim = dim3(256);
-      cfg.stream = stream;
-      cudaLaunchAttribute attr[1];
-      attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      attr[0].val.programmaticStreamSerializationAllowed = 1;
-      cfg.attrs = attr;
-      cfg.numAttrs = 1;
-      TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_copy_kernel, static_cast<const uint8_t*>(up ? host : src),
-                                  static_cast<uint8_t*>(up ? dst : const_cast<void*>(host)), bytes));
-      return TL3_OK;
-    }
+  if (bytes <= kCopyByKernel && (reinterpret_cast<uintptr_t>(device) & 15) == 0 && (up ? up_by_kernel(src, bytes, dst, bytes) : host_by_kernel(dst, bytes))) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((bytes + 4095) / 4096));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    TL3_CUDA(cudaLaunchKernelEx(&cfg, tl3_copy_kernel, static_cast<const uint8_t*>(src), static_cast<uint8_t*>(dst), bytes));
+    return TL3_OK;
   }
   TL3_CUDA(cudaMemcpyAsync(dst, src, bytes, kind, stream));
   return TL3_OK;
@@ -1091,10 +1094,9 @@ int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int
   const size_t x_bytes = static_cast<size_t>(m->K) * N * 2;
   if (ldx == N) {
     if (int rc = tl3::copy_host(dX, X, x_bytes, cudaMemcpyHostToDevice, st)) return rc;
-  } else if (const void* src = tl3::pinned_address(X, x_bytes)) {
+  } else if (tl3::up_by_kernel(X, x_bytes, dX, (static_cast<size_t>(m->K - 1) * ldx + N) * 2)) {
     const long long total = m->K * N;
-    tl3::tl3_spread_rows_kernel<<<static_cast<unsigned>((total + 2047) / 2048), 256, 0, st>>>(static_cast<const uint16_t*>(src), static_cast<uint16_t*>(dX),
-                                                                                            total, static_cast<unsigned>(N), ldx);
+    tl3::tl3_spread_rows_kernel<<<static_cast<unsigned>((total + 2047) / 2048), 256, 0, st>>>(X, static_cast<uint16_t*>(dX), total, static_cast<unsigned>(N), ldx);
     TL3_CUDA(cudaGetLastError());
   } else {
     TL3_CUDA(cudaMemcpy2DAsync(dX, static_cast<size_t>(ldx) * 2, X, static_cast<size_t>(N) * 2, static_cast<size_t>(N) * 2,

@@ -44,3 +44,32 @@ def test_host_copies(M, K, N, x_shift, y_shift):
     m.spmm_host_async(x, y2, dX, dY, ws)
     torch.cuda.synchronize()
     assert np.array_equal(y.view(np.uint16), want.view(np.uint16)) and np.array_equal(y2.view(np.uint16), want.view(np.uint16))
+
+
+@pytest.mark.parametrize("N", [8, 5])
+def test_device_scratch_that_is_too_small_is_refused(N):
+    """Pinned X goes to dX by a kernel: only where dX holds it.  Otherwise the runtime's copy gets the call, and refuses."""
+    import ctypes
+    import torch
+    build.build_library()
+    case = wl.Case(0, "small", 256, 4096, N, 5, 0.5, "magnitude")
+    m = tl3.encode(case.make_W())
+    m.upload()
+    X = torch.from_numpy(case.make_X()).pin_memory()
+    Y = torch.full((256, N), 7.0, dtype=torch.float16, pin_memory=True)
+    dY, ws = torch.empty(256 * N, dtype=torch.float16, device="cuda"), m.new_workspace(N)
+    cu, d = ctypes.CDLL("libcuda.so.1"), ctypes.c_uint64()
+    assert cu.cuMemAlloc_v2(ctypes.byref(d), ctypes.c_size_t(4096)) == 0              # of 65536 bytes
+    try:
+        stream = torch.cuda.current_stream().cuda_stream
+        rc = tl3.lib().tl3_spmm_host(m._h, X.data_ptr(), Y.data_ptr(), N, d.value, dY.data_ptr(), ws.data_ptr(), stream)
+        assert rc == tl3.ERR_CUDA and tl3.lib().tl3_last_cuda_error() == 1             # cudaErrorInvalidValue
+        torch.cuda.synchronize()
+        assert bool((Y == 7).all())
+    finally:
+        assert cu.cuMemFree_v2(d) == 0
+    dX = torch.zeros(4096 * 8, dtype=torch.float16, device="cuda")
+    m.spmm_host(X.numpy(), Y.numpy(), dX, dY, ws)
+    Xd = torch.zeros((4096, 8), dtype=torch.float16, device="cuda")
+    Xd[:, :N] = X.cuda()
+    assert torch.equal(Y, m.spmm(Xd[:, :N]).cpu())
