@@ -52,7 +52,7 @@ struct WideArgs {
   const DirEntry* dir;
   uint32_t tiles_m, tiles_k;              // tiles of W
   int M, N;
-  int n_pad[2];                           // columns of a pass; for pairs also: in a workspace made for 128 columns or fewer
+  int n_pad[2];                           // columns of a pass; above 128 also: in a workspace with room for no more than that
   uint32_t chunks[2];                     // groups of so many columns
   const unsigned char* room;              // columns of partial sums per CTA that the workspace holds, / kRoomUnit
   long long ldy;
@@ -320,7 +320,7 @@ tl3_spmm_wide_kernel(const __grid_constant__ CUtensorMap x_map, const __grid_con
   // group minor), k-tile v % tiles_k.  An odd last row-tile is done by both CTAs of a pair (the second
   // one's rows lie beyond M and are not stored).
   const uint32_t rank = blockIdx.x % S, unit = blockIdx.x / S;
-  // The partial sums of a pair are up to 256 columns per CTA.  A workspace made for fewer, which
+  // The partial sums of a pair are up to 256 columns per CTA.  Above 128, a workspace made for fewer, which
   // tl3_workspace_init() recorded in it, gets passes of half the columns: the slices of X are then loaded
   // as wide as ever and used in part.  (The record is older than anything a kernel before this one does:
   // no wait for it.)
@@ -737,7 +737,9 @@ int spmm_wide(const tl3_matrix* m, const void* X, int64_t ldx, void* Y, int64_t 
   if (S == 2) n_pad = (n_pad + 31) / 32 * 32;                       // (an MMA of 256 rows takes multiples of 32)
   a.block_area = (m->max_block_bytes + 1023u) / 1024u * 1024u;
   a.n_pad[0] = n_pad;
-  a.n_pad[1] = S == 1 ? n_pad : (n_pad / 2 + 31) / 32 * 32;
+  // (The smallest workspace that serves any N has room for 128 columns: only wider passes are ever halved.  20480 x 5120, N = 128
+  // with memory that was only zeroed: in one pass 42.5 us, in two 69.7.)
+  a.n_pad[1] = n_pad <= kAloneColumns ? n_pad : (n_pad / 2 + 31) / 32 * 32;
   for (int i = 0; i < 2; ++i) a.chunks[i] = static_cast<uint32_t>((N + a.n_pad[i] - 1) / a.n_pad[i]);
   a.x_bytes = xt ? static_cast<uint32_t>(n_pad / S) * 128u : static_cast<uint32_t>((n_pad / S + 63) / 64) * 8192u;   // per CTA
   a.n_acc = 2 * n_pad <= static_cast<int>(kColMetaT) ? 2 : 1;

@@ -40,3 +40,28 @@ def test_pairs_of_few_columns(M, K, N, columns, cluster):
     small = torch.zeros(m.workspace_bytes(N), dtype=torch.uint8, device="cuda")     # only zeroed: counts as the smallest
     assert bool(((m.spmm_nt(Xt[:, :K], workspace=small).double() - sums).abs() <= tol).all()) and m.status(small) == tl3.OK
     assert torch.equal(results[0].view(torch.int16), results[1].view(torch.int16))
+
+
+@pytest.mark.parametrize("N", [65, 96, 128])
+def test_pairs_of_few_columns_in_a_workspace_that_was_only_zeroed(N):
+    """The smallest workspace holds all columns of such a pass: the same passes as with an initialised one, and so
+    the same partial sums and the same bits."""
+    import torch
+    build.build_library()
+    M, K = 128 * 42, 128 * 114
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the shape is 32.4 tiles per CTA of 148")
+    g = torch.Generator(device="cuda").manual_seed(N)
+    W = torch.randn((M, K), generator=g, device="cuda").mul_(0.02).half()
+    W[torch.rand((M, K), generator=g, device="cuda") < 0.5] = 0
+    m = tl3.Matrix.encode_on_device(W, device_only=True)
+    m.upload_packed_on_device()
+    Xt = torch.randn((N, K), generator=g, device="cuda").half()
+    Xd = torch.zeros((K, (N + 7) // 8 * 8), dtype=torch.float16, device="cuda")
+    Xd[:, :N] = Xt.T
+    made, zeroed = m.new_workspace(N), torch.zeros(m.workspace_bytes(N), dtype=torch.uint8, device="cuda")
+    for product, X in ((m.spmm, Xd[:, :N]), (m.spmm_nt, Xt)):
+        want, got = product(X, workspace=made), product(X, workspace=zeroed)
+        assert m.last_pass()["cluster"] == 2
+        assert torch.equal(got.view(torch.int16), want.view(torch.int16))
+    assert m.status(zeroed) == tl3.OK
