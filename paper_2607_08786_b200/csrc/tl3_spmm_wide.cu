@@ -694,16 +694,21 @@ int launch_wide(const CUtensorMap& map, const WideArgs& args, bool long_res, int
 constexpr int kAloneColumns = 128;
 
 // Long launches of 65 to 128 columns go in pairs as well: from 32 tiles per CTA on what a tile saves by half of X
-// outweighs the cluster's start and the columns that a multiple of 32 adds.  (us alone / in pairs, X [batch, hidden]: 20480 x
-// 5120, 43 tiles, N = 65 41.0 / 40.1, N = 128 45.5 / 43.4, at 40 % sparsity 53.3 / 49.4; 36864 x 9216, N = 128 127 / 118; 9000 x
-// 9000, 34 tiles, N = 96 37.0 / 35.9; with 19 to 20 tiles 0.94 to 1.05 of alone, N = 112 on 7000 x 7000 27.9 / 28.6; 4096 x 4096,
-// 7 tiles, 17.1 / 19.1.  X [hidden, batch]: 20480 x 5120, N = 65 50.0 / 46.2.)  Up to 64 columns a CTA alone is never
+// outweighs the cluster's start and the columns that a multiple of 32 adds.  (us alone / in pairs, N = 128, X [batch, hidden] and
+// [hidden, batch]: 20480 x 5120, 43 tiles, 45.0 / 42.2 and 46.2 / 43.8; 33 tiles, 8704 x 9216, 37.7 / 36.4 and 39.0 / 38.7, 20480 x
+// 3840 35.7 / 33.8 and 36.2 / 35.2; 36864 x 9216 127 / 118.  With 19 to 20 tiles 0.94 to 1.05 of alone, N = 112 on 7000 x 7000
+// 27.9 / 28.6; 4096 x 4096, 7 tiles, 17.1 / 19.1.)  Up to 64 columns a CTA alone is never
 // slower (1000 x 20000, N = 128 in passes of 64 23.4 / 24.4).
-constexpr int kPairTiles = 32;
+// Few row-tiles are shared by many CTAs, and pairs take longer to hand over the partial sums (and do an odd last row-tile
+// twice): above 80 columns they lose there.  (N = 128, the same two layouts: 9 row-tiles 47.1 / 47.9 and 49.9 / 56.4, 15
+// 43.1 / 44.7 and 45.5 / 49.8, 29 40.3 / 39.7 and 42.0 / 43.0, 37 38.3 / 38.4 and 40.1 / 41.3, 45 39.3 / 38.3 and 40.7 / 40.9, 61
+// 40.2 / 38.7 and 41.8 / 41.7; N = 96 and 112 as N = 128.)  Up to 80 they win from two on (N = 80, 5 row-tiles 49.6 / 47.3, 15 39.2 / 38.8,
+// 29 37.0 / 36.0; 1 row-tile 73.7 / 74.7).  One rule for both layouts, so that they give the same bits.
+constexpr int kPairTiles = 32, kPairRowTiles = 36;
 static int ctas_together(const tl3_matrix* m, int N, int n_pad, int sm_count) {
   if (n_pad > kAloneColumns) return 2;
   const int64_t tiles = m->n_tiles * ((N + n_pad - 1) / n_pad);
-  return n_pad > kAloneColumns / 2 && tiles >= static_cast<int64_t>(kPairTiles) * sm_count ? 2 : 1;
+  return n_pad > kAloneColumns / 2 && tiles >= static_cast<int64_t>(kPairTiles) * sm_count && m->tiles_m >= (n_pad > 80 ? kPairRowTiles : 2) ? 2 : 1;
 }
 
 static int wide_columns(const tl3_matrix* m, int N, int sm_count) {

@@ -65,3 +65,26 @@ def test_pairs_of_few_columns_in_a_workspace_that_was_only_zeroed(N):
         assert m.last_pass()["cluster"] == 2
         assert torch.equal(got.view(torch.int16), want.view(torch.int16))
     assert m.status(zeroed) == tl3.OK
+
+
+@pytest.mark.parametrize("row_tiles,N,cluster", [(9, 128, 1), (9, 100, 1), (35, 96, 1), (36, 96, 2), (9, 80, 2), (2, 66, 2), (1, 80, 1)])
+def test_few_row_tiles_go_in_pairs_up_to_80_columns_only(row_tiles, N, cluster):
+    import torch
+    build.build_library()
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the shapes are a little more than 32 tiles per CTA of 148")
+    M, K = 128 * row_tiles, 128 * -(-(72 if row_tiles == 2 else 33) * 148 // row_tiles)
+    g = torch.Generator(device="cuda").manual_seed(M + N)
+    W = torch.randn((M, K), generator=g, device="cuda").mul_(0.02).half()
+    W[torch.rand((M, K), generator=g, device="cuda") < 0.5] = 0
+    m = tl3.Matrix.encode_on_device(W, device_only=True)
+    m.upload_packed_on_device()
+    Xt = torch.randn((N, K), generator=g, device="cuda").half()
+    Xd = torch.zeros((K, (N + 7) // 8 * 8), dtype=torch.float16, device="cuda")
+    Xd[:, :N] = Xt.T
+    Y, Yt = m.spmm(Xd[:, :N]), m.spmm_nt(Xt)
+    assert m.last_pass()["cluster"] == cluster
+    sums, bound = Xt.double() @ W.double().T, Xt.double().abs() @ W.double().abs().T
+    # as above: chains of MMA steps and partial sums in fp32, one rounding to fp16
+    assert bool(((Yt.double() - sums).abs() <= (K / 16 + 9) * 2.0**-23 * bound + (2.0**-11 + 2.0**-18) * sums.abs() + 2.0**-25).all())
+    assert torch.equal(Y.T.contiguous().view(torch.int16), Yt.view(torch.int16))
