@@ -121,9 +121,9 @@ int tl3_encode_device(const void* dW, int64_t M, int64_t K, int64_t ldw, void* s
  * releases them; tl3_spmm*, tl3_bind, tl3_stats (layer counts; the sizes of the compact forms
  * read -1), tl3_workspace_bytes and tl3_free work as on any handle.  The calls that need the
  * container on the host -- tl3_decode, tl3_canonical, tl3_serialize*, tl3_pack, tl3_upload --
- * return UNSUPPORTED.  Until it is packed the handle holds about 28 KB of device memory per tile whatever
- * the sparsity (0.9 of W; what the blocks need, 21 KB at 50 %, where that is more or where the device has
- * no more).  dW, ldw, stream, errors: as for tl3_encode_device. */
+ * return UNSUPPORTED.  Until it is packed the handle holds about 29 KB of device memory per tile whatever
+ * the sparsity (0.9 of W; what the blocks need, 21 KB at 50 %, where that is more, below 35.5 %, or where the device
+ * has no more).  dW, ldw, stream, errors: as for tl3_encode_device. */
 int tl3_encode_device_only(const void* dW, int64_t M, int64_t K, int64_t ldw, void* stream, tl3_matrix** out);
 
 /* Decode back to dense: Algorithm 1 run on the host, then the 2:4 expansion and the Residual

@@ -26,14 +26,15 @@ namespace {
 struct ConvertArgs {
   DenseView dense;
   int tiles_k;
+  int again;                            // second pass: only the tiles whose blocks have not been made yet
   uint8_t* image;
   unsigned long long capacity;          // bytes of `image`
   uint32_t* sizes;                      // per tile: {pdd_len, res_cnt, real delta bytes} of its block
-  unsigned long long* where;            // per tile: its block in `image`
+  uint8_t** where;                      // per tile: its block; null: no room for it
   unsigned long long* counters;
 };
-// the six layer statistics, delta bytes of the container, bytes of image
-enum { kCountStats = 0, kCountRes = 3, kCountPdd = 6, kCountImage = 7, kCounters = 8 };
+// the six layer statistics, delta bytes of the container; bytes of all blocks, and of those that found no room
+enum { kCountStats = 0, kCountRes = 3, kCountPdd = 6, kCountImage = 7, kCountBeyond = 8, kCounters = 9 };
 
 struct ConvertSmem {
   uint16_t vals[kSlots];                // image of W_t
@@ -84,6 +85,7 @@ tl3_convert_kernel(const ConvertArgs a) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const long long tile = blockIdx.x;
   const long long tm = tile / a.tiles_k, tk = tile % a.tiles_k;
+  if (a.again && a.where[tile]) return;
   if (tid == 16) { sm.nnz = 0; sm.n_chains = 0; }
   classify_tile(a.dense, tm, tk, sm, true);
   __syncthreads();
@@ -151,7 +153,9 @@ tl3_convert_kernel(const ConvertArgs a) {
         a.sizes[tile * 3 + 0] = pdd_len;
         a.sizes[tile * 3 + 1] = res_cnt;
         a.sizes[tile * 3 + 2] = real_bytes;
-        a.where[tile] = sm.place = atomicAdd(a.counters + kCountImage, bytes);
+        const unsigned long long at = sm.place = atomicAdd(a.counters + kCountImage, bytes);
+        if (at + bytes <= a.capacity) a.where[tile] = a.image + at;
+        else atomicAdd(a.counters + kCountBeyond, bytes);
       }
       __syncthreads();
       return sm.place + bytes <= a.capacity ? a.image + sm.place : nullptr;
@@ -160,11 +164,11 @@ tl3_convert_kernel(const ConvertArgs a) {
     [&](uint32_t j) { return make_uint2(residual[j], high[residual[j]]); });
 }
 
-// The blocks of the image to their places in the blob, and the tile directory.
+// The blocks to their places in the blob, and the tile directory.
 __global__ void __launch_bounds__(256)
-tl3_place_kernel(const uint8_t* image, const unsigned long long* where, const unsigned long long* block_off, uint8_t* blob, unsigned long long dir_offset) {
+tl3_place_kernel(const uint8_t* const* where, const unsigned long long* block_off, uint8_t* blob, unsigned long long dir_offset) {
   const long long t = blockIdx.x;
-  const uint8_t* src = image + where[t];
+  const uint8_t* src = where[t];
   const unsigned long long off = block_off[t];
   const uint2 info = *reinterpret_cast<const uint2*>(src + kInfoOff);             // pdd_len, res_cnt
   const uint32_t bytes = align_up_d(kPddOff + info.x + 4u * info.y, 16);
@@ -186,7 +190,7 @@ void release_image(void* p) {
 }  // namespace
 
 cudaError_t place_image(const DeviceCanon& c, const unsigned long long* d_block_off, uint8_t* blob, size_t dir_offset, int64_t n_tiles, cudaStream_t st) {
-  tl3_place_kernel<<<static_cast<unsigned>(n_tiles), 256, 0, st>>>(c.image, c.where, d_block_off, blob, dir_offset);
+  tl3_place_kernel<<<static_cast<unsigned>(n_tiles), 256, 0, st>>>(c.where, d_block_off, blob, dir_offset);
   return cudaGetLastError();
 }
 
@@ -203,10 +207,10 @@ extern "C" int tl3_encode_device_only(const void* dW, int64_t M, int64_t K, int6
   auto up = [](size_t x) { return (x + 255) / 256 * 256; };
   const size_t o_where = up(pack_scratch_bytes(m->n_tiles)), o_counters = o_where + up(tiles * 8), o_image = o_counters + 256;
   // One allocation (cudaMalloc takes 0.33 ms and cudaFree 0.29, from a megabyte on whatever the size: more than the
-  // kernels of a 5120 x 5120 matrix) with a guess at the image that holds down to 40 % sparsity (27.4 KB per tile
-  // there).  Where that is too little, or more than the device has, a pass that writes no blocks gives
-  // the size and the image is allocated as large as it is.
-  size_t guess = tiles * 28672 + 32768;
+  // kernels of a 5120 x 5120 matrix) with 29.25 KB a tile for the blocks, which holds down to 35.5 % sparsity.  Blocks that find no room
+  // there get a second allocation and a second pass over their tiles.  (5120 x 5120, whole conversions: at
+  // 36 % 800 us, at 30 % 1390; 2110 and 2140 with 28 KB a tile, given up for one allocation of the blocks' size where that was too little.)  Where the device has no memory for that, the
+  // first pass writes no blocks and the second one all, into exactly what they need.
   uint8_t *scratch = nullptr, *image = nullptr;
   unsigned long long got[kCounters] = {};
   std::vector<uint32_t> sizes;
@@ -215,19 +219,20 @@ extern "C" int tl3_encode_device_only(const void* dW, int64_t M, int64_t K, int6
   a.tiles_k = static_cast<int>(m->tiles_k);
   int rc = TL3_OK;
   cudaError_t e = cudaSuccess;
-  auto pass = [&](uint8_t* to, size_t capacity) {
+  auto pass = [&](bool again, uint8_t* to, size_t capacity) {
+    a.again = again;
     a.sizes = reinterpret_cast<uint32_t*>(scratch);
-    a.where = reinterpret_cast<unsigned long long*>(scratch + o_where);
-    a.counters = reinterpret_cast<unsigned long long*>(scratch + o_counters);
+    a.where = reinterpret_cast<uint8_t**>(scratch + o_where);
+    a.counters = reinterpret_cast<unsigned long long*>(scratch + o_counters) + (again ? 16 : 0);   // (a tile made again counts once)
     a.image = to;
     a.capacity = capacity;
-    e = cudaMemsetAsync(a.counters, 0, sizeof(got), st);
+    e = again ? cudaSuccess : cudaMemsetAsync(scratch + o_where, 0, o_image - o_where, st);
     if (e == cudaSuccess) {
       tl3_convert_kernel<<<static_cast<unsigned>(tiles), kTileThreads, sizeof(ConvertSmem), st>>>(a);
       e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(got, a.counters, sizeof(got), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(sizes.data(), a.sizes, tiles * 12, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && !again) e = cudaMemcpyAsync(got, a.counters, sizeof(got), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && !again) e = cudaMemcpyAsync(sizes.data(), a.sizes, tiles * 12, cudaMemcpyDeviceToHost, st);
     const cudaError_t done = cudaStreamSynchronize(st);             // (also when something failed: nothing of it may still run)
     if (e == cudaSuccess) e = done;
     return e == cudaSuccess;
@@ -238,23 +243,17 @@ extern "C" int tl3_encode_device_only(const void* dW, int64_t M, int64_t K, int6
   if (rc == TL3_OK) {
     // (on every call, like the packer's: an opt-in that is remembered does not outlive a cudaDeviceReset())
     e = cudaFuncSetAttribute(tl3_convert_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(ConvertSmem)));
-    if (e == cudaSuccess) {
-      e = cudaMalloc(reinterpret_cast<void**>(&scratch), o_image + guess);
-      if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        scratch = nullptr;
-        guess = 0;
-        e = cudaMalloc(reinterpret_cast<void**>(&scratch), o_image);
+    for (const size_t room : {tiles * 29952 + 32768, size_t{0}}) {
+      if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&scratch), o_image + room);
+      if (e == cudaSuccess && pass(false, scratch + o_image, room) && got[kCountBeyond]) {
+        e = cudaMalloc(reinterpret_cast<void**>(&image), got[kCountBeyond]);
+        if (e == cudaSuccess) pass(true, image, got[kCountBeyond]);
       }
-    }
-    if (e == cudaSuccess && pass(guess ? scratch + o_image : nullptr, guess) && got[kCountImage] > guess) {
-      if (guess) {
-        cudaFree(scratch);
-        scratch = nullptr;
-        e = cudaMalloc(reinterpret_cast<void**>(&scratch), o_image);
-      }
-      if (e == cudaSuccess) e = cudaMalloc(reinterpret_cast<void**>(&image), got[kCountImage]);
-      if (e == cudaSuccess) pass(image, got[kCountImage]);
+      if (e != cudaErrorMemoryAllocation || room == 0) break;
+      cudaGetLastError();
+      if (scratch) cudaFree(scratch);
+      scratch = image = nullptr;
+      e = cudaSuccess;
     }
     if (e != cudaSuccess) { set_cuda_error(static_cast<int>(e)); rc = TL3_ERR_CUDA; }
     else if (got[kCountPdd] > 0xFFFFFFFFull || got[kCountRes] > 0xFFFFFFFFull) rc = TL3_ERR_UNSUPPORTED;   // 32-bit offsets of the container's directory
@@ -273,7 +272,6 @@ extern "C" int tl3_encode_device_only(const void* dW, int64_t M, int64_t K, int6
   }
   const size_t n_vals = static_cast<size_t>(m->M_pad) * m->K_pad / 2;
   m->canon_bytes = static_cast<int64_t>(n_vals * 2 + n_vals / 4 + tiles * kTileM * 5 + tiles * 16 + got[kCountPdd] + got[kCountRes] * 4);
-  c->image = a.image;
   c->where = a.where;
   c->pack_scratch = scratch;
   c->alloc[0] = scratch;

@@ -107,10 +107,9 @@ struct tl3_matrix {
 namespace tl3 {
 
 // What tl3_upload_device packs: the canonical arrays on the device, or (tl3_encode_device_only) the blocks
-// themselves in the order in which they were finished.
+// themselves, wherever they were put when they were finished.
 struct DeviceCanon {
-  const uint8_t* image;                      // null: the arrays
-  const unsigned long long* where;           // per tile: its block in `image`
+  const uint8_t* const* where;               // per tile: its block; null: the arrays
   const uint16_t* tc_vals; const uint8_t* tc_meta; const uint16_t* chain_tau0; const uint16_t* chain_rho0;
   const uint8_t* chain_len; const uint8_t* pdd_bytes; const uint32_t* tile_dir; const uint16_t* res_rho; const uint16_t* res_val;
   void* pack_scratch;                        // pack_scratch_bytes(): sizes of the packed blocks, then their offsets

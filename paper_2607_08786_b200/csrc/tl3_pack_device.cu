@@ -345,7 +345,7 @@ int canon_to_device(tl3_matrix* m, cudaStream_t st, PackArgs* out) {
     DeviceCanon* c = new (std::nothrow) DeviceCanon();
     if (!c) { cudaFree(p); return TL3_ERR_NO_MEMORY; }
     uint8_t* b = static_cast<uint8_t*>(p);
-    *c = DeviceCanon{nullptr, nullptr, reinterpret_cast<const uint16_t*>(b + off[0]), b + off[1], reinterpret_cast<const uint16_t*>(b + off[2]),
+    *c = DeviceCanon{nullptr, reinterpret_cast<const uint16_t*>(b + off[0]), b + off[1], reinterpret_cast<const uint16_t*>(b + off[2]),
                      reinterpret_cast<const uint16_t*>(b + off[3]), b + off[4], b + off[5], reinterpret_cast<const uint32_t*>(b + off[6]),
                      reinterpret_cast<const uint16_t*>(b + off[7]), reinterpret_cast<const uint16_t*>(b + off[8]), b + o_pack, {p, nullptr}};
     m->device_canon = c;
@@ -439,7 +439,7 @@ extern "C" int tl3_upload_device(tl3_matrix* m, void* dptr, void* stream) {
     a.dir_offset = m->dir_offset;
     a.emit = 1;
     const DeviceCanon& c = *static_cast<const DeviceCanon*>(m->device_canon);
-    if (c.image) {
+    if (c.where) {
       e = place_image(c, d_off, a.blob, a.dir_offset, m->n_tiles, st);
     } else {
       tl3_pack_kernel<<<static_cast<unsigned>(m->n_tiles), kTileThreads, sizeof(PackSmem), st>>>(a);

@@ -30,9 +30,10 @@ def _random(M, K, p):
 
 
 @pytest.mark.parametrize("W", [_cut([0]), _cut([0, 60]), _cut([5, 6, 127]), np.vstack([_cut([0]), _cut([3, 90])]), clustered_surplus_tile(),
-                               _random(128, 128, 1.0),                  # dense: more than the first guess at the image
-                               _random(640, 900, 1.0), _random(640, 900, 0.75), np.zeros((300, 140), dtype=np.float16), _random(1, 1, 1.0)],
-                         ids=["cut", "cut_and_beyond", "cut_3", "two_tiles_cut", "clustered", "dense_tile", "dense", "a_quarter", "zeros", "one_weight"])
+                               _random(128, 128, 1.0),                  # 51840 bytes, which the first allocation has room for; not
+                               _random(128, 256, 1.0), _random(640, 900, 1.0),      # for two such tiles, nor for forty: a second pass makes the others
+                               _random(640, 900, 0.75), np.zeros((300, 140), dtype=np.float16), _random(1, 1, 1.0)],
+                         ids=["cut", "cut_and_beyond", "cut_3", "two_tiles_cut", "clustered", "dense_tile", "two_dense_tiles", "dense", "a_quarter", "zeros", "one_weight"])
 def test_device_only(W):
     import torch
     from paper_2607_08786_b200 import build, tl3
