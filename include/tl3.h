@@ -263,7 +263,8 @@ int tl3_spmm_host(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, vo
 /* The same without the wait: the three steps are only enqueued on `stream`.  X must stay valid and
  * Y is defined once the stream has passed this point (cudaStreamSynchronize, an event).  Calls on
  * different streams may be in flight together as long as each has its own dX, dY and workspace:
- * the copies of one then overlap the kernel of another. */
+ * the copies of one then overlap the kernel of another.  (Copies of pinned memory are done by kernels up to
+ * 192 KB, up to 1 MB in a blocking call with no other one beside it, and for X with N no multiple of eight.) */
 int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY,
                         void* workspace, void* stream);
 

@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -35,6 +36,11 @@ def build_library(force: bool = False, verbose: bool = False) -> str:
         print(res.stderr)
     if res.returncode != 0:
         raise RuntimeError("nvcc failed building libtl3.so")
+    # what tl3_copy_kernel counts on (tl3_spmm.cu) and launch bounds cannot ask for
+    used = re.search(r"Compiling entry function '\w*tl3_copy_kernel\w*'.*?Used (\d+) registers", res.stdout + res.stderr, re.S)
+    if used is None or int(used.group(1)) > 16:
+        os.remove(LIB)
+        raise RuntimeError(f"tl3_copy_kernel takes {used.group(1) if used else 'an unknown number of'} registers, not 16: it no longer fits beside a product")
     return LIB
 
 

@@ -749,6 +749,10 @@ static bool up_by_kernel(const void* host, size_t bytes, const void* device, siz
 }
 
 // Bytes between device memory and pinned host memory, 16 per thread and the last ones singly.
+// It is to stay at 16 registers (build.py checks): a block of 256 threads then fits beside a product's (61440 of an SM's 65536
+// registers) and a copy need not wait for an SM to be free.  With 28 or 40 a call beside the products of another stream takes 12 us
+// longer.  (__maxnreg__ goes down to 24 only.  Blocks of 128 threads and 32 registers fit as well, but three and four streams with 130 to
+// 190 KB each lose up to 1 us a call by the larger number of blocks.)
 __global__ void __launch_bounds__(256)
 tl3_copy_kernel(const uint8_t* src, uint8_t* dst, size_t bytes) {   // (not __restrict__: no load may move in front of the wait)
   pdl_launch_dependents();                                         // (a product behind it waits before it reads X)
@@ -761,16 +765,24 @@ tl3_copy_kernel(const uint8_t* src, uint8_t* dst, size_t bytes) {   // (not __re
   }
 }
 
-// X to the device or Y to the host.  The copy engine takes 3 to 5 us to begin and to report; a kernel begins while the
-// product still runs, its threads wait for it.  Both by a kernel, whole calls with pinned buffers: 1024 x 1024, N = 8
-// 34.0 -> 26.3 us; 4096 x 4096, N = 16 45.5 -> 34.7, N = 64 62.8 -> 57.0; 8192 x 4096, N = 61 (Y 1.0 MB) 71.2 -> 68.0.
-// Beyond a megabyte the copy is what takes the time and the engine is as good (Y of 1.3 MB 59.2 and 59.8, of
-// 2.6 MB 88.1 and 91.1), so the SMs are left to the products of other streams.
-constexpr size_t kCopyByKernel = size_t{1} << 20;
-static int copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, cudaStream_t stream) {
+// X to the device or Y to the host.  The copy engine takes 3 to 5 us to begin and to report, or 20 more when it has been idle; a
+// kernel begins while the product still runs, its threads wait for it.  But it takes room on SMs that products of other
+// streams could have.  Engine / kernel, us per call:
+//                                      one call at a time | calls from 4 threads | enqueued on 1, 3 and 4 streams
+//   1024 x 1024, N = 8    (16 KB)             53 / 39             13 / 14            23 / 15, 12 / 13, 12 / 13
+//   4096 x 4096, N = 16   (131 KB)            57 / 46             15 / 14            35 / 24, 14 / 13, 11 / 13
+//   6000 x 5000, N = 16   (192 KB)            61 / 52             17 / 17            38 / 29, 17 / 16, 14 / 15
+//   8192 x 8192, N = 16   (262 KB)            74 / 65             22 / 27            50 / 41, 22 / 25, 20 / 23
+//   4096 x 4096, N = 64   (524 KB)            73 / 65             23 / 31            50 / 42, 25 / 27, 22 / 26
+//   8000 x 8000, N = 64   (1 MB)             108 / 96             34 / 48            83 / 72, 39 / 48, 39 / 48
+// (The last column at 16 and 131 KB is the host's time: a launch takes 1 us more than a copy.)  So calls that may be in flight
+// together take kernels up to 192 KB, a blocking call that no other one is under way beside up to a megabyte (beside long
+// products of another stream that costs it 8 to 18 us from 700 KB on).
+constexpr size_t kCopyByKernel = size_t{192} << 10, kCopyByKernelAlone = size_t{1} << 20;
+static int copy_host(void* dst, const void* src, size_t bytes, cudaMemcpyKind kind, size_t by_kernel, cudaStream_t stream) {
   const bool up = kind == cudaMemcpyHostToDevice;
   const void* device = up ? dst : src;
-  if (bytes <= kCopyByKernel && (reinterpret_cast<uintptr_t>(device) & 15) == 0 && (up ? up_by_kernel(src, bytes, dst, bytes) : host_by_kernel(dst, bytes))) {
+  if (bytes <= by_kernel && (reinterpret_cast<uintptr_t>(device) & 15) == 0 && (up ? up_by_kernel(src, bytes, dst, bytes) : host_by_kernel(dst, bytes))) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>((bytes + 4095) / 4096));
     cfg.blockDim = dim3(256);
@@ -1085,7 +1097,8 @@ int tl3_spmm_nt(const tl3_matrix* m, const void* Xt, int64_t ldxt, void* Yt, int
   return TL3_OK;
 }
 
-int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY, void* workspace, void* stream) {
+static int enqueue_host(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY, void* workspace, void* stream,
+                        size_t by_kernel) {
   if (!m || !X || !Y || !dX || !dY) return TL3_ERR_INVALID_ARG;
   if (N < 1 || N > TL3_MAX_N) return TL3_ERR_UNSUPPORTED;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -1093,7 +1106,7 @@ int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int
   const int64_t ldx = (N + 7) / 8 * 8;
   const size_t x_bytes = static_cast<size_t>(m->K) * N * 2;
   if (ldx == N) {
-    if (int rc = tl3::copy_host(dX, X, x_bytes, cudaMemcpyHostToDevice, st)) return rc;
+    if (int rc = tl3::copy_host(dX, X, x_bytes, cudaMemcpyHostToDevice, by_kernel, st)) return rc;
   } else if (tl3::up_by_kernel(X, x_bytes, dX, (static_cast<size_t>(m->K - 1) * ldx + N) * 2)) {
     const long long total = m->K * N;
     tl3::tl3_spread_rows_kernel<<<static_cast<unsigned>((total + 2047) / 2048), 256, 0, st>>>(X, static_cast<uint16_t*>(dX), total, static_cast<unsigned>(N), ldx);
@@ -1103,11 +1116,20 @@ int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int
                                static_cast<size_t>(m->K), cudaMemcpyHostToDevice, st));
   }
   if (int rc = tl3_spmm(m, dX, ldx, dY, N, N, workspace, stream)) return rc;
-  return tl3::copy_host(Y, dY, static_cast<size_t>(m->M) * N * 2, cudaMemcpyDeviceToHost, st);
+  return tl3::copy_host(Y, dY, static_cast<size_t>(m->M) * N * 2, cudaMemcpyDeviceToHost, by_kernel, st);
+}
+
+int tl3_spmm_host_async(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY, void* workspace, void* stream) {
+  return enqueue_host(m, X, Y, N, dX, dY, workspace, stream, tl3::kCopyByKernel);
 }
 
 int tl3_spmm_host(const tl3_matrix* m, const uint16_t* X, uint16_t* Y, int N, void* dX, void* dY, void* workspace, void* stream) {
-  if (int rc = tl3_spmm_host_async(m, X, Y, N, dX, dY, workspace, stream)) return rc;
+  static std::atomic<int> under_way{0};                           // blocking calls, of any thread
+  struct Call {
+    const bool alone = under_way.fetch_add(1, std::memory_order_relaxed) == 0;
+    ~Call() { under_way.fetch_sub(1, std::memory_order_relaxed); }
+  } call;
+  if (int rc = enqueue_host(m, X, Y, N, dX, dY, workspace, stream, call.alone ? tl3::kCopyByKernelAlone : tl3::kCopyByKernel)) return rc;
   TL3_CUDA(cudaStreamSynchronize(static_cast<cudaStream_t>(stream)));
   return TL3_OK;
 }

@@ -8,7 +8,7 @@ from paper_2607_08786_b200 import build, tl3, workloads as wl
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (129, 16, 8), (256, 256, 8), (257, 264, 8), (255, 130, 16), (8192, 128, 64), (8193, 128, 64), (130, 8200, 64), (1000, 60, 5)])
+@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (129, 16, 8), (256, 256, 8), (257, 264, 8), (255, 130, 16), (8192, 128, 64), (8193, 128, 64), (130, 8200, 64), (1000, 60, 5), (1536, 1536, 64), (1537, 1544, 64)])
 @pytest.mark.parametrize("x_shift,y_shift", [(0, 0), (8, 8), (1, 0), (0, 1), (None, 0), (0, None)])      # None: pageable
 def test_host_copies(M, K, N, x_shift, y_shift):
     import torch
