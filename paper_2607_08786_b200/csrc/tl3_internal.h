@@ -44,7 +44,8 @@ template <class T> struct RawAllocator {
 };
 template <class T> using raw_vector = std::vector<T, RawAllocator<T>>;
 
-// Large copies and first touches of fresh memory, shared out over up to sixteen and eight threads (tl3_host.cpp).
+// Large copies and first touches of fresh memory, shared out over up to sixteen and eight threads (tl3_host.cpp); `chunk`: the
+// pieces of a copy that takes more than eight.
 void parallel_copy(void* dst, const void* src, size_t bytes, size_t chunk = size_t{1} << 20);
 void prefault(void* p, size_t bytes);                        // fresh memory that a copy engine is about to fill
 

@@ -26,6 +26,18 @@ def test_round_trip(matrix, kind, compact):
         assert np.array_equal(m.canonical(name), matrix.canonical(name)), name
 
 
+@pytest.mark.parametrize("M,K", [(4096, 4991), (4096, 5119), (6000, 4200)])
+def test_arrays_around_the_size_that_more_threads_copy(M, K):
+    """Value arrays a column of tiles short of 20 MB, of 20 MB and of 25."""
+    rng = np.random.default_rng(K)
+    W = np.zeros((M, K), dtype=np.float16)
+    W[rng.random(W.shape) < 0.5] = 0.25
+    m = tl3.encode(W)
+    data = m.serialize()
+    again = tl3.Matrix.deserialize(data)
+    assert again.serialize() == data and np.array_equal(again.decode(), W.view(np.uint16))
+
+
 def test_a_bad_position_in_any_tile_is_found(matrix):
     data = bytearray(matrix.serialize())
     n_tiles = matrix.stats()["n_tiles"]
