@@ -8,7 +8,9 @@ from paper_2607_08786_b200 import build, tl3, workloads as wl
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (129, 16, 8), (256, 256, 8), (257, 264, 8), (255, 130, 16), (8192, 128, 64), (8193, 128, 64), (130, 8200, 64), (1000, 60, 5), (1536, 1536, 64), (1537, 1544, 64)])
+@pytest.mark.parametrize("M,K,N", [(1, 8, 8), (129, 16, 8), (256, 256, 8), (257, 264, 8), (255, 130, 16), (8192, 128, 64), (8193, 128, 64), (130, 8200, 64), (1000, 60, 5), (1536, 1536, 64), (1537, 1544, 64),
+                                   # Y ends within a thread's 16 bytes: 2, 14, 18, 50010 bytes, two short of 192 KB and of a megabyte, two more than 192 KB
+                                   (1, 8, 1), (7, 8, 1), (9, 16, 1), (5001, 300, 5), (98303, 8, 1), (524287, 8, 1), (98305, 8, 1)])
 @pytest.mark.parametrize("x_shift,y_shift", [(0, 0), (8, 8), (1, 0), (0, 1), (None, 0), (0, None)])      # None: pageable
 def test_host_copies(M, K, N, x_shift, y_shift):
     import torch
@@ -73,3 +75,38 @@ def test_device_scratch_that_is_too_small_is_refused(N):
     Xd = torch.zeros((4096, 8), dtype=torch.float16, device="cuda")
     Xd[:, :N] = X.cuda()
     assert torch.equal(Y, m.spmm(Xd[:, :N]).cpu())
+
+
+def test_blocking_calls_from_several_threads():
+    """Beside another blocking call large copies go another way than alone: the same bits."""
+    import threading
+    import torch
+    build.build_library()
+    case = wl.Case(0, "threads", 2048, 2048, 64, 9, 0.5, "magnitude")
+    X = case.make_X()
+    m = tl3.encode(case.make_W())
+    m.upload()
+    want = m.spmm(torch.from_numpy(X).cuda()).cpu()
+    calls = []
+    for _ in range(4):
+        calls.append((torch.from_numpy(X).pin_memory(), torch.zeros((2048, 64), dtype=torch.float16, pin_memory=True),
+                      torch.empty(2048 * 64, dtype=torch.float16, device="cuda"), torch.empty(2048 * 64, dtype=torch.float16, device="cuda"),
+                      m.new_workspace(64), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    wrong, errors = [], []
+
+    def work(x, y, dX, dY, ws, stream):
+        try:
+            for _ in range(20):
+                y.zero_()
+                m.spmm_host(x.numpy(), y.numpy(), dX, dY, ws, stream)
+                wrong.append(not torch.equal(y, want))
+        except Exception as e:                                  # reported below, in the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=c) for c in calls]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors and len(wrong) == 80 and not any(wrong)

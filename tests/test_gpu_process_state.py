@@ -33,8 +33,19 @@ def upload(data, want):
     ck(cu.cuMemcpyDtoH_v2(got.ctypes.data_as(vp), d, ctypes.c_size_t(got.size)), "copy")
     ck(cu.cuMemFree_v2(d), "free")
     assert np.array_equal(got, want)
-m = tl3.encode(wl.Case(0, "state", 4096, 2048, 8, 5, 0.5, "bernoulli").make_W())
+def download(data, want):
+    d, h = u64(), vp()
+    ck(cu.cuMemAlloc_v2(ctypes.byref(d), ctypes.c_size_t(W.nbytes)), "alloc")
+    ck(cu.cuMemcpyHtoD_v2(d, W.ctypes.data_as(vp), ctypes.c_size_t(W.nbytes)), "copy")
+    rc = tl3.lib().tl3_encode_device(vp(d.value), 4096, 2048, 2048, None, ctypes.byref(h))
+    assert rc == 0, (rc, tl3.lib().tl3_last_cuda_error())
+    ck(cu.cuMemFree_v2(d), "free")
+    assert tl3.Matrix(h.value).serialize() == data
+W = wl.Case(0, "state", 4096, 2048, 8, 5, 0.5, "bernoulli").make_W()
+m = tl3.encode(W)
 data, want = m.serialize(), m.pack()
+if sys.argv[2] == "down":
+    upload = download
 assert len(data) > 9 << 20                                   # beyond the size from which the pinned memory is used
 primary()
 upload(data, want)
@@ -73,5 +84,12 @@ print("done")
 
 @pytest.mark.parametrize("what", ["trim", "context", "reset"])
 def test_uploads_around(what):
-    res = subprocess.run([sys.executable, "-c", PROGRAM, what], capture_output=True, text=True, timeout=300)
+    res = subprocess.run([sys.executable, "-c", PROGRAM, what, "up"], capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and res.stdout.endswith("done\n"), res.stdout + res.stderr[-2000:]
+
+
+@pytest.mark.parametrize("what", ["trim", "context", "reset"])
+def test_downloads_around(what):
+    """The same for containers that come from the device."""
+    res = subprocess.run([sys.executable, "-c", PROGRAM, what, "down"], capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and res.stdout.endswith("done\n"), res.stdout + res.stderr[-2000:]

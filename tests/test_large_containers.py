@@ -85,3 +85,27 @@ def test_loading_from_several_threads(matrix):
     assert not errors
     for blob in got:
         assert np.array_equal(blob, want)
+
+
+@pytest.mark.gpu
+def test_encoding_on_several_threads(matrix):
+    """The way down: one thread's container comes through the pinned pieces, the others' meanwhile without."""
+    import torch
+    W, want = torch.from_numpy(matrix.decode().view(np.float16)).cuda(), matrix.serialize()
+    got, errors = [None] * 4, []
+    torch.cuda.synchronize()
+
+    def encode(i):
+        try:
+            for _ in range(3):
+                got[i] = tl3.Matrix.encode_on_device(W, stream=torch.cuda.Stream()).serialize()
+        except Exception as e:                                  # reported below, in the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=encode, args=(i,)) for i in range(len(got))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors
+    assert all(data == want for data in got)
