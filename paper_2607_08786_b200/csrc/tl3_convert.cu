@@ -9,8 +9,8 @@
 // image is put in order when the caller says where the blob is to lie.
 // What bounds it is instructions (62 % of the issue slots) and barriers in front of the threads that walk a tile's lists and
 // chains, four tiles per SM (56 KB each) at once; DRAM is at 9 %.
-// 5120 x 5120 at 50 % sparsity: 74 us, and 9 to put the image in order; the encoder's two passes, its scan and
-// the packer's two, with the container written and read in between, took 31 + 46 + 4 + 47 + 65 us.
+// 5120 x 5120 at 50 % sparsity: 73 us, and 9 to put the image in order; the encoder's two passes, its scan between them and
+// the packer's two, with the container written and read in between, take 30 + 5 + 51 + 55 + 75 us.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -59,7 +59,7 @@ static_assert(sizeof(PackWork) == 4 * (512 + 49) + 8 * kTileM, "sets over the ma
 static_assert(4 * (sizeof(ConvertSmem) + 1024) <= 233472, "four tiles per SM");
 static_assert(sizeof(ConvertSmem::nib) >= kMaxHead, "the head of a block fits");
 
-// bit c of lane r -> bit r of lane c
+// bit c of lane r -> bit r of lane c: the transposition by halves of halves in Warren, "Hacker's Delight", 7-3, a lane per row
 __device__ __forceinline__ uint32_t transpose_bits(uint32_t x, int lane) {
   uint32_t m = 0x0000FFFFu;
 #pragma unroll

@@ -380,7 +380,10 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
 EncodeTiledFn encode_tiled_fn();
 
 // whether a matrix's tiles have so many Residual entries that scatter_residual<true> pays: one batch of four per thread
-// on average, which leaves out 50 % sparsity and more (1.6 % of the weights, 130 entries a tile) and takes in 40 % (1640)
+// on average, which leaves out 48 % sparsity and more and takes in 46 %.  (us short / long: 656 entries a tile, 46 %, 11008 x 4096, N =
+// 16, 24, 64, 128 17.3 / 17.1, 18.5 / 18.2, 21.2 / 20.9, 26.6 / 26.0, 9216 x 9216 26.7 / 26.3, 28.4 / 28.1, 32.7 / 32.3, 39.0 / 39.0; 491, 47 %,
+// 17.1 / 16.9, 18.1 / 17.8, 20.9 / 20.7, 26.4 / 26.0, but 26.3 / 26.7, 28.1 / 28.4, 32.1 / 32.5, 38.6 / 39.1; 328, 48 %, level; 164, 49 %,
+// 16.1 / 16.2, 17.4 / 17.4, 19.9 / 20.0, 25.8 / 25.9.)
 inline bool long_residual(const tl3_matrix* m) { return m->dev_n_res >= 512 * m->n_tiles; }
 
 struct WorkspaceLayout {

@@ -19,7 +19,7 @@
 // a one-block scan turns the counts into the offsets of the tile directory, then it runs again
 // and writes the bytes where they belong.
 // What bounds it is the number of instructions it issues (its memory traffic, W once per pass and the
-// container once, is a few microseconds).  Two passes on 5120 x 5120 at 50 % sparsity: 31 + 52 us.
+// container once, is a few microseconds).  Two passes on 5120 x 5120 at 50 % sparsity: 30 + 51 us.
 // A thread per row, two-byte accesses a row pitch apart and 512 atomics per tile on four
 // addresses took 351 + 898 us; coalesced rows that every lane classified for itself, with chains
 // walked by a thread per row, 57 + 89 us.

@@ -35,8 +35,8 @@ static void run_parallel(int64_t n, unsigned most, const F& f) {
 constexpr size_t kCopyChunk = size_t{1} << 20;
 
 // Large copies wait for the first touch of `dst`, page by page, so more threads help beyond what memory moves (132 MB
-// into huge pages 7.2 ms with eight threads, 5.1 with sixteen; 55 MB into small ones 5.1 and 4.0), and two that
-// meet in one huge page wait for each other (6.0 ms in chunks of 1 MB there).  Below 20 MB, where malloc hands out memory that
+// into huge pages 6.3 ms with eight threads, 5.1 with sixteen; 55 MB into small ones 3.9 and 2.3), and two that
+// meet in one huge page wait for each other (132 MB with sixteen threads in pieces of 2 MB 3.5 ms).  Below 20 MB, where malloc hands out memory that
 // has been touched and two megabytes a piece leave threads without one, that is slower: reading a container of 10.6 MB (8.4 of
 // them values) takes 0.58 ms with eight threads and 0.75 with sixteen in pieces of 2 MB, of 21 MB (16.8) 1.15 and 1.22, of 31 MB (24.6) 1.55
 // and 1.41, of 42 MB (33.5) 2.7 and 2.0.

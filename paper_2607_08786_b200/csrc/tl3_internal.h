@@ -16,8 +16,8 @@
 namespace tl3 {
 
 // Memory of the container's arrays: not cleared (every byte is written after a resize), and large
-// arrays on huge pages.  A first copy into 132 MB of fresh memory takes one thread 62 ms on 4 KB pages
-// and 28 ms on huge ones; eight threads 8.5 and 4.4 ms.
+// arrays on huge pages.  A first copy into 132 MB of fresh memory takes one thread 60 ms on 4 KB pages
+// and 27 on huge ones; sixteen threads 5.5 and 3.5.
 template <class T> struct RawAllocator {
   using value_type = T;
   static constexpr size_t kHuge = size_t{2} << 20;
@@ -168,6 +168,8 @@ struct HostPiece {
   size_t bytes;
 };
 cudaError_t copy_pieces(const std::vector<HostPiece>& arrays, cudaMemcpyKind kind, cudaStream_t st);
+// tl3_convert.cu: the blocks to their places in the blob, and the directory
+cudaError_t place_image(const DeviceCanon& c, const unsigned long long* d_block_off, uint8_t* blob, size_t dir_offset, int64_t n_tiles, cudaStream_t st);
 #endif
 
 }  // namespace tl3

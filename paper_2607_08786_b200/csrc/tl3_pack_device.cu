@@ -14,7 +14,7 @@
 // plan_device_layout() does, and an emit pass that writes the blocks.
 // What bounds it is the latency of a tile's serial steps (the chains), hidden by three tiles per SM.
 // With two-byte copies, a thread per 64 coordinates tested one by one and one thread sharing out the
-// banks, the two passes took 181 + 247 us on 5120 x 5120 at 50 % sparsity; now 57 + 77 us.
+// banks, the two passes took 181 + 247 us on 5120 x 5120 at 50 % sparsity; now 55 + 75 us.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -31,9 +31,6 @@
 #include "tl3_internal.h"
 
 namespace tl3 {
-
-// tl3_convert.cu: the blocks of an image to their places in the blob, and the directory
-cudaError_t place_image(const DeviceCanon& c, const unsigned long long* d_block_off, uint8_t* blob, size_t dir_offset, int64_t n_tiles, cudaStream_t st);
 
 namespace {
 
@@ -242,7 +239,9 @@ PinnedRing& ring_of_process() {
 
 }  // namespace
 
-// Pageable host memory to or from the device, behind what is on `st`, complete on return.  The runtime's own copy moves
+// Pageable host memory to or from the device, complete on return.  What comes down is read behind what is on `st`.  What goes up is
+// not ordered behind it (a stream of its own carries it): its destination has to be memory that nothing on `st` uses
+// any more, such as a fresh allocation.  The runtime's own copy moves
 // 11 GB/s, one thread of its filling or emptying one staging buffer; here six threads do that with two
 // pinned megabytes each, one of them under way while the other is worked on (one caller at a
 // time; another one that comes meanwhile takes the runtime's way).  132 MB up: 12.2 ms the runtime's way, 5.9 with one megabyte per thread, 4.7

@@ -686,9 +686,10 @@ int launch_wide(const CUtensorMap& map, const WideArgs& args, bool long_res, int
 // matrix more row-tiles to share out and less to add up at the end.  The estimate of a launch, in us, from
 // measured launches: a tile costs 0.45 (its decode) + 0.0036 per column for a CTA alone, 0.8 + 0.0014 for a
 // pair, which is the way above 128 columns: half of X per CTA leaves room for more blocks in flight and
-// halves what the tensor cores read of it (20480 x 5120, N = 512: 107 us, alone 123; 5120 x 20480, N = 200:
-// 56 and 66), while up to 128 columns a cluster's start costs more than that gains (1024 x 1024, N = 128:
-// 11.3 us, alone 9.5; 5120 x 5120, N = 160: 23.6, alone 23.7).  The CTAs that share a row-tile hand over n_pad columns each at
+// halves what the tensor cores read of it (20480 x 5120, N = 512: 110 us, alone 123; 5120 x 20480, N = 200:
+// 56 and 66), while up to 128 columns a cluster's start costs a short launch more than that gains (1024 x 1024, N = 128:
+// 11.3 us, alone 9.5; 5120 x 5120, N = 160: 23.6, alone 23.7).  Passes of up to 128 columns are priced as a CTA alone
+// also where ctas_together() then takes pairs for them: those differ by a few per cent, passes by tens.  The CTAs that share a row-tile hand over n_pad columns each at
 // 0.008 per column and CTA.  (1024 x 1024, N = 500: 23 us in 2 passes, 17 in 3, 13 in 4; 20480 x 5120, N = 512:
 // 125 in 2, 142 in 3, 160 in 4, all with one CTA per tile.)
 constexpr int kAloneColumns = 128;
